@@ -28,6 +28,7 @@ constexpr int kM0 = 64;           // rows per block at the top level
 constexpr int kMr = 32;           // rows per block at the reduced levels
 constexpr int kMaxLevels = 8;
 constexpr size_t kScratchBytes = size_t(2) << 20;  // 2 MiB per GPU
+constexpr size_t kHeadOnchip = 128;  // the on-chip launch's status word and two counters
 
 // The scratch array.  In host code `g_scratch` names a host-side shadow,
 // not device memory: its device address comes from cudaGetSymbolAddress.
@@ -144,13 +145,7 @@ cudaError_t run(unsigned char* ws, const Layout& L, int idx, int64_t n, const Ti
 }
 
 // Translate the status bits into a tps_status for the caller's output.
-__global__ void k_report(const int* st, int32_t* out) {
-  const int w = *st;
-  *out = (w & ST_BAD_PIVOT) ? TPS_ERR_ZERO_PIVOT
-         : (w & ST_TIMEOUT) ? TPS_ERR_TIMEOUT
-         : (w & ST_RANGE)   ? TPS_ERR_RANGE
-                            : TPS_OK;
-}
+__global__ void k_report(const int* st, int32_t* out) { *out = status_code(*st); }
 
 // A cooperative launch the device refuses for its size or resources (fewer
 // SMs than the cached occupancy assumed, e.g. under an SM partition):
@@ -185,26 +180,30 @@ extern "C" tps_status tps_solve_noalloc(int32_t dtype, int64_t n, const void* a,
   tps_status ts = scratch_address(&ws);
   if (ts != TPS_OK) return ts;
   cudaStream_t s = (cudaStream_t)stream;
-  int* st = reinterpret_cast<int*>(ws);
-  // the first 64 bytes (status word, on-chip barrier counter, the three
-  // range codes at 40) are the only scratch that must start from zero; the
-  // reduced systems and checkpoints are fully rewritten by every call
-  unsigned* dmax = dtype == TPS_F64_DF ? reinterpret_cast<unsigned*>(ws + 40) : nullptr;
-  cudaError_t e = cudaMemsetAsync(st, 0, 64, s);
-  // the whole system in one on-chip launch where it fits (its barrier
-  // counter and exchange rows sit where the levels would go); a test switch
-  // (TPS_TEST_NOALLOC_LEVELS=1) keeps the level-by-level route
+  // the whole system in one on-chip launch where it fits, which reports and
+  // clears its own status word (its words of the header, kHeadOnchip, are
+  // zero between launches; its exchange rows sit where the levels would go);
+  // a test switch (TPS_TEST_NOALLOC_LEVELS=1) keeps the level-by-level route
   bool onchip = false;
   const char* lvl = std::getenv("TPS_TEST_NOALLOC_LEVELS");
-  if (e == cudaSuccess && !(lvl && lvl[0] == '1')) {
-    e = onchip_solve(dtype, n, a, b, c, d, x, ws + align_up(64),
-                     reinterpret_cast<unsigned*>(ws + 32), st, s, onchip, dmax);
+  cudaError_t e = cudaSuccess;
+  if (!(lvl && lvl[0] == '1')) {
+    unsigned* head = reinterpret_cast<unsigned*>(ws + kHeadOnchip);
+    e = onchip_solve(dtype, n, a, b, c, d, x, ws + align_up(64), head + 1,
+                     reinterpret_cast<int*>(head), status_out, s, onchip);
+    if (e == cudaSuccess && onchip) return TPS_OK;
     if (e != cudaSuccess && launch_refused(e)) {
       cudaGetLastError();
       e = cudaSuccess;
       onchip = false;
     }
   }
+  // the first 64 bytes (status word, the three range codes at 40) are the
+  // only scratch of the levels that must start from zero; the reduced
+  // systems and checkpoints are fully rewritten by every call
+  int* st = reinterpret_cast<int*>(ws);
+  unsigned* dmax = dtype == TPS_F64_DF ? reinterpret_cast<unsigned*>(ws + 40) : nullptr;
+  if (e == cudaSuccess) e = cudaMemsetAsync(st, 0, 64, s);
   if (e == cudaSuccess && !onchip) {
     switch (dtype) {
       case TPS_F64:

@@ -46,6 +46,7 @@
 #include <type_traits>
 
 #include "arith.cuh"
+#include "tps.h"
 
 namespace tps {
 
@@ -116,6 +117,14 @@ struct Bounds {
 
 // Status bits written into the device status word.
 enum : int { ST_BAD_PIVOT = 1, ST_NO_CONVERGENCE = 2, ST_TIMEOUT = 4, ST_RANGE = 8 };
+
+// The tps_status of a status word (numeric values of tps.h).
+__device__ __forceinline__ int32_t status_code(int w) {
+  return (w & ST_BAD_PIVOT) ? TPS_ERR_ZERO_PIVOT
+         : (w & ST_TIMEOUT) ? TPS_ERR_TIMEOUT
+         : (w & ST_RANGE)   ? TPS_ERR_RANGE
+                            : TPS_OK;
+}
 
 // Range codes of packed systems: three words per system (RowChk's dcode,
 // ecode, fcode maxima).  Raise system `sys`'s codes to v (an atomic only

@@ -34,23 +34,33 @@ size_t truncate_rel_bytes(int64_t n_max, int R, int h, int dtype) {
 struct OcGeom {
   int mt;     // level-0 block rows (odd)
   int64_t p;  // level-0 blocks
+  int B;      // level-0 blocks per CTA
   int G;      // CTAs
 };
 
-// The smallest odd block length (>= 3) whose CTA count fits `ctas_max`;
-// a one-row tail is merged into the block before it.
+// Blocks of mt rows, B to a CTA; a one-row tail is merged into the block
+// before it.  False: more than `ctas_max` CTAs, or more rows than one holds.
 template <class Tin>
+static bool oc_fits(int64_t n, int mt, int B, int ctas_max, OcGeom& g) {
+  if (mt * B >= oc_rows_max<Tin>()) return false;
+  int64_t p = (n + mt - 1) / mt;
+  if (n - (p - 1) * mt == 1) --p;
+  const int64_t G = (p + B - 1) / B;
+  if (G > ctas_max) return false;
+  g = {mt, p, B, (int)G};
+  return true;
+}
+
+// One CTA where its longer blocks cost less than the grid barrier and the
+// exchange, else the shortest odd block length whose CTAs fit.
+template <class Ar, class Tin>
 static bool oc_geometry(int64_t n, int ctas_max, OcGeom& g) {
-  if (n <= kBaseMax) return false;
-  for (int mt = 3; mt <= oc_mt_max<Tin>(); mt += 2) {
-    int64_t p = (n + mt - 1) / mt;
-    if (n - (p - 1) * mt == 1) --p;
-    const int64_t G = (p + kOcThreads - 1) / kOcThreads;
-    if (G <= ctas_max) {
-      g = {mt, p, (int)G};
-      return true;
-    }
-  }
+  if (n <= kBaseMax || ctas_max < 1) return false;
+  for (int mt = 3; mt <= kOcSoloRows<Ar>; mt += 2)
+    if (oc_fits<Tin>(n, mt, kOcBlocks<Ar>, 1, g)) return true;
+  for (int B = kOcBlocks<Ar>; B <= kOcThreads; B *= 2)
+    for (int mt = 3; mt <= oc_block_rows_max<Tin>(B); mt += 2)
+      if (oc_fits<Tin>(n, mt, B, ctas_max, g)) return true;
   return false;
 }
 
@@ -83,24 +93,23 @@ static int oc_ctas_max() {
 }
 
 // Solve the system on chip if it fits (used = true), else leave it.  xch:
-// onchip_exchange_bytes() of device memory; bar: a counter (zeroed here).
+// onchip_exchange_bytes() of device memory; bar: the launch's two counters,
+// zero between launches; report: see OcShared (own_status where given).
 template <class Ar, class Tin>
 static cudaError_t launch_onchip_raw(int64_t n, const Tin* a, const Tin* b, const Tin* c,
-                                     const Tin* d, Tin* x, void* xch_bytes, unsigned* bar,
+                                     const Tin* d, Tin* x, void* xch, unsigned* bar,
                                      int* status, bool extra_arrival, cudaStream_t s,
-                                     bool& used, unsigned* dmax) {
+                                     bool& used, bool codes, bool own_status = false,
+                                     int32_t* report = nullptr) {
   used = false;
   OcGeom g;
-  if (!oc_geometry<Tin>(n, oc_ctas_max<Ar, Tin>(), g)) return cudaSuccess;
+  if (!oc_geometry<Ar, Tin>(n, oc_ctas_max<Ar, Tin>(), g)) return cudaSuccess;
   using T = typename Ar::T;
-  T* xch = reinterpret_cast<T*>(xch_bytes);
   const uintptr_t al = (uintptr_t)a | (uintptr_t)b | (uintptr_t)c | (uintptr_t)d | (uintptr_t)x;
   const int vec16 = (al % 16) == 0;
-  cudaError_t e = cudaMemsetAsync(bar, 0, sizeof(unsigned), s);
-  if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)g.G);
-  cfg.blockDim = dim3(kOcThreads);
+  cfg.blockDim = dim3((unsigned)g.B);
   cfg.dynamicSmemBytes = OcLayout<Ar, Tin>::kBytes;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
@@ -108,23 +117,25 @@ static cudaError_t launch_onchip_raw(int64_t n, const Tin* a, const Tin* b, cons
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  const unsigned arrivals = (unsigned)g.G + (extra_arrival ? 1u : 0u);
-  e = cudaLaunchKernelEx(&cfg, k_onchip<Ar, Tin>, n, g.mt, g.p, a, b, c, d, x, xch, bar,
-                         arrivals, status, vec16, dmax);
+  const OcShared sh{bar, (unsigned)g.G + (extra_arrival ? 1u : 0u), status, report,
+                    own_status ? 1 : 0};
+  const cudaError_t e =
+      cudaLaunchKernelEx(&cfg, k_onchip<Ar, Tin>, n, g.mt, g.p, a, b, c, d, x,
+                         reinterpret_cast<T*>(xch), sh, vec16, codes ? 1 : 0);
   if (e == cudaSuccess) used = true;
   return e;
 }
 
-// dmax: the |d / b| codes where this is level 0 (level0_dmax), else null.
+// codes: this is level 0 of fp64 inputs in narrower arithmetic (level0_dmax).
 template <class Ar, class Tin>
 static cudaError_t launch_onchip(tps_plan_s* P, int64_t n, const Tin* a, const Tin* b,
                                  const Tin* c, const Tin* d, Tin* x, cudaStream_t s,
-                                 bool& used, unsigned* dmax) {
+                                 bool& used, bool codes) {
   used = false;
   if (P->desc.flags & TPS_NO_ONCHIP) return cudaSuccess;
   return launch_onchip_raw<Ar, Tin>(n, a, b, c, d, x, P->ws + P->off_xch,
                                     reinterpret_cast<unsigned*>(P->ws + 32), P->d_status,
-                                    P->test_barrier_extra, s, used, dmax);
+                                    P->test_barrier_extra, s, used, codes);
 }
 
 unsigned* level0_dmax(tps_plan_s* P) {
@@ -295,7 +306,7 @@ static cudaError_t run_levels(tps_plan_s* P, const std::vector<LevelPlan>& level
     return cudaGetLastError();
   }
   bool used = false;
-  cudaError_t eo = launch_onchip<Ar, Tin>(P, n, a, b, c, d, x, s, used, nullptr);
+  cudaError_t eo = launch_onchip<Ar, Tin>(P, n, a, b, c, d, x, s, used, false);
   if (eo != cudaSuccess || used) {
     if (used) {
       P->last_onchip = 2;
@@ -591,7 +602,8 @@ static tps_status run_solve_direct(tps_plan_s* P, int64_t n, const void* a, cons
       using Tin = std::remove_pointer_t<decltype(tin)>;
       (void)tred;
       return launch_onchip<Ar, Tin>(P, n, (const Tin*)a, (const Tin*)b, (const Tin*)c,
-                                    (const Tin*)d, (Tin*)x, s, onchip, level0_dmax(P));
+                                    (const Tin*)d, (Tin*)x, s, onchip,
+                                    level0_dmax(P) != nullptr);
     });
     if (onchip) {
       P->last_onchip = 1;
@@ -698,14 +710,14 @@ tps_status run_truncated(tps_plan_s* P, int64_t n, const void* a, const void* b,
 
 cudaError_t onchip_solve(int dtype, int64_t n, const void* a, const void* b, const void* c,
                          const void* d, void* x, void* xch, unsigned* bar, int* status,
-                         cudaStream_t s, bool& used, unsigned* dmax) {
+                         int32_t* report, cudaStream_t s, bool& used) {
   return dispatch(dtype, [&](auto ar, auto* tin, auto* tred) -> cudaError_t {
     using Ar = decltype(ar);
     using Tin = std::remove_pointer_t<decltype(tin)>;
     (void)tred;
     return launch_onchip_raw<Ar, Tin>(n, (const Tin*)a, (const Tin*)b, (const Tin*)c,
                                       (const Tin*)d, (Tin*)x, xch, bar, status, false, s, used,
-                                      dmax);
+                                      dtype == TPS_F64_DF, true, report);
   });
 }
 

@@ -77,7 +77,7 @@ static void default_params(const tps_plan_desc& d, int32_t& m, int32_t& mr, int3
 
 static size_t workspace_for(tps_plan_s* P, size_t* off_levels_out, size_t* off_dev_out) {
   size_t off = 0;
-  off = align_up(off + 64);  // status word, refinement maxima, grid-barrier counter
+  off = align_up(off + 64);  // status word, refinement maxima, grid-barrier counters
   P->off_dmax = off;         // per-system range codes (zero between solves)
   off = align_up(off + 4 * kCodes * (size_t)std::max<int64_t>(1, P->desc.batch_max));
   P->off_xch = off;          // interface rows of the on-chip solve

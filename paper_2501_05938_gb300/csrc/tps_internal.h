@@ -161,12 +161,11 @@ cudaError_t refine_step(tps_plan_s* P, const std::vector<LevelPlan>& levels, con
 size_t onchip_exchange_bytes();
 // The single-launch on-chip solve of one system if it fits on this device
 // (used = true), else nothing.  xch: onchip_exchange_bytes() of device
-// memory; bar: a device counter (zeroed by the call); status: the device
-// status word; dmax: for double-float, one system's kCodes range codes,
-// zero before the launch and left zero after it (else null).
+// memory; bar: two device counters, status: a status word, all three zero
+// between launches; report: the solve's tps_status, or null.
 cudaError_t onchip_solve(int dtype, int64_t n, const void* a, const void* b, const void* c,
                          const void* d, void* x, void* xch, unsigned* bar, int* status,
-                         cudaStream_t s, bool& used, unsigned* dmax);
+                         int32_t* report, cudaStream_t s, bool& used);
 // TPS_TRUNCATE: the windowed solve of one device-resident system.
 tps_status run_truncated(tps_plan_s* P, int64_t n, const void* a, const void* b, const void* c,
                          const void* d, void* x, cudaStream_t s);

@@ -115,3 +115,45 @@ def test_barrier_timeout_is_reported_and_the_gpu_stays_usable(monkeypatch):
     assert info["status_name"] == "TPS_ERR_TIMEOUT"
     # the context survives: the next solve on a normal plan is correct
     check("f64", n, 3, 1)
+
+
+@pytest.mark.parametrize("dtype,n", [
+    ("f64_df", 2304), ("f64_df", 2305), ("f64_df", 2306),      # one CTA of 256 blocks, then four
+    ("f32", 5888), ("f32", 5889), ("f32", 5890),
+    ("f64", 320), ("f64", 448), ("f64", 449), ("f64", 450),    # one CTA of 64 blocks, then two
+    ("f64", 152 * 64 * 7), ("f64", 152 * 64 * 7 + 1), ("f64", 152 * 64 * 7 + 2),  # 64 or 128 blocks
+    ("f64", 152 * 128 * 45 + 1), ("f64", 152 * 128 * 45 + 2),  # 128 or 256 blocks
+    ("f64_df", 769 + 3), ("f64_df", 33 * 3 + 1), ("f32", 95), ("f64", 161),
+])
+def test_block_and_cta_edges(dtype, n):
+    """The rules that choose the block length, the blocks per CTA and one CTA."""
+    check(dtype, n, 7 + n, 1)
+
+
+@pytest.mark.parametrize("dtype,ulp", [("f64", 2.0 ** -53), ("f64_df", 2.0 ** -46),
+                                       ("f32", 2.0 ** -24)])
+@pytest.mark.parametrize("n", [5000, 20011, 120001])
+def test_couplings_that_do_not_decay(dtype, ulp, n):
+    """a = c = -1, b = 2 + 1e-4: the couplings of the interface rows fall by
+    e^-0.01 a row, so no few strides of the reduction settle them and every
+    CTA reduces all of them.  The matrix's condition number is 4e4; a direct
+    solve is off by a small multiple of that times the unit roundoff."""
+    delta = 1e-4
+    rng = np.random.default_rng(n)
+    one = np.ones(n)
+    a, c, b = -one, -one.copy(), (2.0 + delta) * one
+    a[0] = c[-1] = 0.0
+    if dtype == "f32":
+        b = b.astype(np.float32).astype(np.float64)
+    xt = rng.uniform(-1, 1, n)
+    d = b * xt
+    d[1:] += a[1:] * xt[:-1]
+    d[:-1] += c[:-1] * xt[1:]
+    s = {"a": a, "b": b, "c": c, "d": d}
+    tdt = torch.float64
+    if dtype == "f32":
+        s, tdt = synth.to_f32(s), torch.float32
+    x, info = solve(binding.Plan(n, dtype=dtype), s, tdt)
+    assert info["status"] == 0 and info["onchip"] == 1, info
+    ref = oracle.thomas(*(np.asarray(s[k], dtype=np.float64) for k in "abcd"))
+    assert oracle.rel_forward_error(x, ref) <= 16 * (4.0 / delta) * ulp
