@@ -71,7 +71,7 @@ bool make_layout(int64_t n, size_t top_elem, size_t red_elem, Layout& L) {
   while (N > kBaseMax) {
     if (L.levels == kMaxLevels) return false;
     LevelPlan& P = L.lv[L.levels++];
-    P = LevelPlan{};
+    P = LevelPlan{};  // rel = false: relations would not fit the scratch
     P.R = chunk_rows(elem);
     P.lv = make_level(N, m, P.R);
     const int64_t nr = 2 * P.lv.p;

@@ -231,6 +231,24 @@ struct RefineIO {
   unsigned long long* max2; // Stage 3: the two maxima (zeroed before the launch)
 };
 
+// The relations of a level's interior rows, x_j = g_j - al_j f - c_j x_{j+1},
+// written by Stage 1 and read by k_back in the order in which their lanes own
+// them: row j of the nb (32, or the launch's last few) blocks of the warp that
+// starts at block k0 is nb consecutive values from (k0 * cap + j * nb).
+// al has decayed below rounding a few chunks into a block of an ordinary
+// system: na[k0] says how many chunks of the warp have it.
+template <class T>
+struct alignas(2 * sizeof(T)) RelRow {
+  T c, g;
+};
+struct RelIO {
+  void* rel;  // RelRow<T>
+  void* al;   // T
+  int* na;    // one per block, used at each warp's first
+  int cap;    // rows per block: m + 1, rounded up to 4 (16-byte chunk starts)
+};
+__host__ __device__ constexpr int rel_cap(int m) { return (m + 4) / 4 * 4; }
+
 // Pieces of the current x a Stage-1 refinement chunk needs: its R rows and
 // the next piece (the row below the chunk), i.e. kPieces + 1 pieces filling
 // the block's padded slot; piece q = lane + 32 j (j <= kPieces) is piece
@@ -415,6 +433,10 @@ __device__ __forceinline__ int chunk_kind(int ch, int row0, int R, int lmin, int
 #ifndef TPS_STAGE1_STAGES
 #define TPS_STAGE1_STAGES 2
 #endif
+#ifndef TPS_REL_UNROLL
+#define TPS_REL_UNROLL 2
+#endif
+constexpr int kRelUnroll = TPS_REL_UNROLL;
 constexpr int kS1Stages = TPS_STAGE1_STAGES;
 static_assert(kS1Stages >= 2 && kS1Stages <= 4, "Stage-1 pipeline depth");
 // Shared memory of one Stage-1 warp (NA arrays per buffer).
@@ -425,21 +447,24 @@ constexpr size_t stage1_smem_per_warp() {
 
 // R rows per chunk; a checkpoint every K rows (K the chunk length of
 // Stage 3; one of R and K divides the other).  kRef: a refinement step
-// (RefineIO), the right-hand side being the residual of rf.x.
-template <class Ar, class Tin, class Tred, int R, int K, int W, bool kVec16, bool kRef = false>
+// (RefineIO), the right-hand side being the residual of rf.x.  kRel: every
+// interior row's relation goes out (RelIO) for k_back, and no checkpoints.
+template <class Ar, class Tin, class Tred, int R, int K, int W, bool kVec16, bool kRef = false,
+          bool kRel = false>
 __global__ void __launch_bounds__(W * 32)
     k_stage1(Level lv, const Tin* __restrict__ a, const Tin* __restrict__ b,
              const Tin* __restrict__ c, const Tin* __restrict__ d, Tred* __restrict__ ra,
              Tred* __restrict__ rb, Tred* __restrict__ rc, Tred* __restrict__ rd,
              Tred* __restrict__ ck_gam, Tred* __restrict__ ck_y, Tred* __restrict__ ck_v,
-             int* __restrict__ status, RefineIO rf = {}) {
+             int* __restrict__ status, RefineIO rf = {}, RelIO rl = {}) {
   using T = typename Ar::T;
   using TL = Tile<Tin, R, kRef ? 5 : 4>;
+  constexpr bool kSkip = Ar::kSkipChain || kRel;  // decayed chains are skipped
   constexpr int V = TL::kVec;
   static_assert(!kRef || std::is_same<Tin, double>::value, "refinement steps are fp64");
   static_assert(R % K == 0 || K % R == 0, "chunk rows and checkpoint spacing must nest");
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = W == 1 ? 0 : threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t k0 = lv.k_begin + ((int64_t)blockIdx.x * W + warp) * 32;
   if (k0 >= lv.k_end) return;
   const int nb = (int)(lv.k_end - k0 < 32 ? lv.k_end - k0 : 32);
@@ -498,19 +523,58 @@ __global__ void __launch_bounds__(W * 32)
   // rounding and the rows skip it (kChain false); they check |c| <= |beta|
   // instead, so S cannot grow back, and a block where that fails reports a
   // pivot failure (not dominant).
-  bool chain = true, nondom = false;
+  // With kRel every policy skips, and al with the chain, once S and every
+  // later al are below 2^-60 (Ar::decayed).  Both bounds rest on the rows
+  // being dominant, which the skipping rows check (Ar::dominant): if one is
+  // not, the warp starts over and skips nothing (`keep`).
+  bool chain = true, nondom = false, dom = true, keep = false, sdec = false;
+  int na = nch;
+  T alp = Ar::zero(), cp = Ar::zero();  // the last row's relation (al, c)
 
   // one interior row (1 <= row <= L-2).  The product chains alpha and S and
   // the accumulators P and Q are left unnormalised here and renormalised
   // once per chunk (renorm), which bounds their low parts to a few ulps.
-  auto interior = [&](const T av, const T bv, const T cv, const T dv, auto kChain) {
+  RelRow<T>* const rel = static_cast<RelRow<T>*>(rl.rel) + (kRel ? k0 * rl.cap : 0);
+  T* const rel_al = static_cast<T*>(rl.al) + (kRel ? k0 * rl.cap : 0);
+  auto interior = [&](const T av, const T bv, const T cv, const T dv, auto kChain, int row) {
     const T ratio = Ar::mul_nn(av, rbp);
     beta = Ar::sub_mul_dom(bv, ratio, cprev);
     g = Ar::sub_mul(dv, ratio, g);
-    al = Ar::mul_neg_nn(ratio, al);
+    if constexpr (!kRel || decltype(kChain)::value) al = Ar::mul_neg_nn(ratio, al);
     bad |= Ar::bad_pivot(beta);
     const T rbeta = Ar::rcp(beta);
-    if constexpr (decltype(kChain)::value) {
+    if constexpr (kRel) {
+      T gp;
+      if constexpr (sizeof(Tin) == 4) {  // bound by memory: round the quotients once
+        cp = Ar::quot(cv, beta, rbeta);
+        gp = Ar::quot(g, beta, rbeta);
+      } else {
+        cp = Ar::mul(cv, rbeta);
+        gp = Ar::mul(g, rbeta);
+      }
+      const RelRow<T> w{cp, gp};
+      if (active) rel[row * nb + lane] = w;
+      if constexpr (decltype(kChain)::value) {
+        alp = Ar::mul(Ar::norm(al), rbeta);
+        if (active) rel_al[row * nb + lane] = alp;
+        if constexpr (Ar::kSkipChain) {  // one fp64 product fewer
+          P = Ar::sub_mul_nn(P, S, w.g);
+          Q = Ar::sub_mul_nn(Q, S, alp);
+          S = Ar::mul_neg_nn(S, cp);
+        } else {  // shorter lives of w and alp: 260 against 296 us at n = 2^25
+          const T tt = Ar::mul_nn(S, rbeta);
+          P = Ar::sub_mul_nn(P, tt, g);
+          Q = Ar::sub_mul_nn(Q, tt, al);
+          S = Ar::mul_neg_nn(tt, cv);
+        }
+        if constexpr (Ar::kSkipChain) {
+          if (sdec) nondom |= !Ar::mag_le(cv, beta);
+        }
+      } else {
+        if constexpr (Ar::kSkipChain) nondom |= !Ar::mag_le(cv, beta);
+        dom &= Ar::dominant(av, bv, cv);
+      }
+    } else if constexpr (decltype(kChain)::value) {
       const T tt = Ar::mul_nn(S, rbeta);
       P = Ar::sub_mul_nn(P, tt, g);
       Q = Ar::sub_mul_nn(Q, tt, al);
@@ -530,7 +594,7 @@ __global__ void __launch_bounds__(W * 32)
   // checkpoint after row `row` (a multiple of K minus one), when the next K
   // rows start with an interior row (Stage 3 restarts its chunk there)
   auto checkpoint = [&](int row) {
-    if (active && row + 1 <= L - 2) {
+    if (!kRel && active && row + 1 <= L - 2) {
       const int64_t slot = (int64_t)((row + 1) / K - 1) * lv.p + k;
       Ar::to(ck_gam[slot], Ar::mul(cprev, rbp));
       Ar::to(ck_y[slot], Ar::mul(Ar::norm(g), rbp));
@@ -552,7 +616,7 @@ __global__ void __launch_bounds__(W * 32)
     // with and without the first unknown's chain
     auto fast_chunk = [&](auto kChain) {
       const bool first = kind == kFirst, last = kind == kLast;
-#pragma unroll
+#pragma unroll (kRel ? kRelUnroll : R / V)
       for (int r = 0; r < R; r += V) {
         const Vec16<Tin> xa = lds16(t + r), xb = lds16(t + TL::kArr + r),
                          xc = lds16(t + 2 * TL::kArr + r), xd = lds16(t + 3 * TL::kArr + r);
@@ -560,8 +624,8 @@ __global__ void __launch_bounds__(W * 32)
         for (int v = 0; v < V; ++v) {
           const int rr = r + v;
           // a of the system's first row and c of its last are never read
-          const bool cut_c = rr == R - 1 && last && k == lv.p - 1;
-          const Tin ain = (rr == 0 && first && k == 0) ? Tin{} : xa.v[v];
+          const bool cut_c = v == V - 1 && rr == R - 1 && last && k == lv.p - 1;
+          const Tin ain = (v == 0 && rr == 0 && first && k == 0) ? Tin{} : xa.v[v];
           const Tin cin = cut_c ? Tin{} : xc.v[v];
           Tin din = xd.v[v];
           if constexpr (kRef) {  // the residual of the current x
@@ -573,16 +637,16 @@ __global__ void __launch_bounds__(W * 32)
           }
           T av, bv, cv, dv;
           Ar::template row<true>(ain, xb.v[v], cin, din, av, bv, cv, dv, chk);
-          if (rr == 0 && first) {  // the block's first row: f's equation
+          if (v == 0 && rr == 0 && first) {  // the block's first row: f's equation
             a0 = av; b0 = bv; c0 = cv; d0 = dv;
-          } else if (rr == R - 1 && last) {  // the block's last row
+          } else if (v == V - 1 && rr == R - 1 && last) {  // the block's last row
             const T ratio = Ar::mul_nn(av, rbp);
             beta = Ar::sub_mul_dom(bv, ratio, cprev);
             g = Ar::sub_mul(dv, ratio, g);
             al = Ar::mul_neg_nn(ratio, al);
             clast = cv;
           } else {
-            interior(av, bv, cv, dv, kChain);
+            interior(av, bv, cv, dv, kChain, row0 + rr);
             if constexpr (R > K) {  // chunk spans several checkpoint intervals
               if ((rr + 1) % K == 0 && rr + 1 < R) checkpoint(row0 + rr);
             }
@@ -591,7 +655,7 @@ __global__ void __launch_bounds__(W * 32)
       }
     };
     if (kind != kSlow) {
-      if constexpr (Ar::kSkipChain) {
+      if constexpr (kSkip) {
         if (chain) fast_chunk(std::true_type{});
         else fast_chunk(std::false_type{});
       } else {
@@ -628,8 +692,8 @@ __global__ void __launch_bounds__(W * 32)
           if (row == 0) {
             a0 = av; b0 = bv; c0 = cv; d0 = dv;
           } else if (row < L - 1) {
-            if (!Ar::kSkipChain || chain) interior(av, bv, cv, dv, std::true_type{});
-            else interior(av, bv, cv, dv, std::false_type{});
+            if (!kSkip || chain) interior(av, bv, cv, dv, std::true_type{}, row);
+            else interior(av, bv, cv, dv, std::false_type{}, row);
             if constexpr (R > K) {
               if ((row + 1) % K == 0 && r + 1 < R) checkpoint(row);
             }
@@ -647,16 +711,44 @@ __global__ void __launch_bounds__(W * 32)
     // the checkpoint at the chunk's end (row0 + R is a multiple of K when
     // K divides R, and every K / R chunks otherwise)
     if (((row0 + R) % K) == 0) checkpoint(row0 + R - 1);
-    if constexpr (Ar::kSkipChain) {
+    if constexpr (kRel) {
+      if (chain) {
+        if (Ar::kSkipChain && __all_sync(0xffffffffu, !active || Ar::chain_small(S))) sdec = true;
+        if (!keep && __all_sync(0xffffffffu, !active || Ar::decayed(S, alp, cp))) {
+          chain = false;
+          na = ch + 1;
+          al = Ar::zero();
+        }
+      } else if (__any_sync(0xffffffffu, active && !dom)) {  // start over, skip nothing
+        cp_async_wait<0>();
+        __syncwarp();
+        chain = keep = dom = true;
+        sdec = bad = nondom = false;
+        na = nch;
+        rbp = Ar::one();
+        cprev = g = P = Q = Ar::zero();
+        al = S = Ar::neg(Ar::one());
+        if constexpr (kRef) xup = active && start > 0 ? rf.x[start - 1] : Tin{};
+        chk.reset_codes();  // what was raised stays; the rest is seen again
+        sys = lv.nbnd > 0 && active ? bd.first : 0;
+#pragma unroll
+        for (int c = 0; c < kS1Stages - 1; ++c) fetch(c);
+        ch = -1;
+        continue;
+      }
+    } else if constexpr (Ar::kSkipChain) {
       if (chain && __all_sync(0xffffffffu, !active || Ar::chain_small(S))) chain = false;
     }
-    if constexpr (kRef) {  // the chunk's residual (in the d slots) out
+    if constexpr (kRef && !kRel) {  // the chunk's residual (in the d slots) out
       __syncwarp();
       store_chunk<Tin, R, kVec16>(rf.r, tb + 3 * TL::kArr, pm, row0);
     }
     __syncwarp();  // the buffer is refilled by the next iteration's copies
   }
   bad |= nondom;
+  if constexpr (kRel) {
+    if (lane == 0) rl.na[k0] = na;
+  }
   if (active) {
     bad |= Ar::bad_pivot(beta);
     if (L == 1) {
@@ -894,6 +986,169 @@ __global__ void __launch_bounds__(W * 32)
   }
   if (active && bad) atomicOr(status, ST_BAD_PIVOT);
   if (active && oob) atomicOr(status, ST_RANGE);
+  if constexpr (kRef) {
+    for (int o = 16; o > 0; o >>= 1) {
+      mdel = max(mdel, __shfl_xor_sync(0xffffffffu, mdel, o));
+      mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    }
+    // most warps see maxima already raised past theirs: read before the atomic
+    if (lane == 0) {
+      if (mdel > *(volatile unsigned long long*)&rf.max2[0]) atomicMax(&rf.max2[0], mdel);
+      if (mx > *(volatile unsigned long long*)&rf.max2[1]) atomicMax(&rf.max2[1], mx);
+    }
+  }
+}
+
+// ------------------------------------------------------------------ Stage 3 from relations
+// Back-substitution of every block from its two interface values through the
+// relations Stage 1 wrote (kRel): one multiply-add a row where k_stage3
+// repeats the elimination, and 24 bytes a row (2 values of a relation in, x
+// out; fp32 12) where k_stage3 moves 40.  Bound by those bytes, so what
+// counts is how many are on their way: a chunk's relations are one contiguous
+// piece of memory, copied with cp.async kBackStages - 1 chunks ahead.
+// kRef: the result is added to x in place and the maxima go to rf.max2.
+#ifndef TPS_BACK_STAGES
+#define TPS_BACK_STAGES 3
+#endif
+constexpr int kBackStages = TPS_BACK_STAGES;
+template <class Ar, class Tin, int R, bool kRef>
+struct BackTile {
+  using T = typename Ar::T;
+  static constexpr size_t kRows = (size_t)32 * R * sizeof(RelRow<T>);
+  static constexpr size_t kAl = (size_t)32 * R * sizeof(T);
+  static constexpr size_t kX = Tile<Tin, R, 1>::kArr * sizeof(Tin);
+  static constexpr size_t kStage = kRows + kAl + (kRef ? kX : 0);
+  static constexpr size_t kBytes = kBackStages * kStage + (kRef ? 0 : kX);
+};
+template <class Ar, class Tin, class Tred, int R, bool kVec16, bool kRef = false>
+__global__ void __launch_bounds__(32)
+    k_back(Level lv, const Tred* __restrict__ xred, Tin* __restrict__ x, int* __restrict__ status,
+           RelIO rl, RefineIO rf) {
+  using T = typename Ar::T;
+  using TL = Tile<Tin, R, 1>;
+  using BT = BackTile<Ar, Tin, R, kRef>;
+  constexpr int V = TL::kVec;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int lane = threadIdx.x;
+  // the reverse of Stage 1's order: its last relations are still in L2
+  const int64_t k0 = lv.k_begin + (int64_t)(gridDim.x - 1 - blockIdx.x) * 32;
+  const int nb = (int)(lv.k_end - k0 < 32 ? lv.k_end - k0 : 32);
+  const int64_t k = k0 + lane;
+  const bool active = lane < nb;
+  const int L = active ? block_len(lv, k) : 0;
+  const int nch = warp_chunks(lv, k0, nb, R);
+  const int lmin = warp_lmin(lv, k0, nb);
+  const RelRow<T>* const rel = static_cast<const RelRow<T>*>(rl.rel) + k0 * rl.cap;
+  const T* const rel_al = static_cast<const T*>(rl.al) + k0 * rl.cap;
+  const int na = rl.na[k0];
+  PieceMap<Tin, R> pm;
+  pm.init(lv, k0, nb, lane);
+  const Tin* const xsrc[1] = {x};
+  auto rows_of = [&](int st) {
+    return reinterpret_cast<RelRow<T>*>(smem_raw + st * BT::kStage);
+  };
+  auto al_of = [&](int st) {
+    return reinterpret_cast<T*>(smem_raw + st * BT::kStage + BT::kRows);
+  };
+  auto x_of = [&](int st) {
+    return reinterpret_cast<Tin*>(smem_raw + (kRef ? st * BT::kStage + BT::kRows + BT::kAl
+                                                   : kBackStages * BT::kStage));
+  };
+  // `rows` rows (a multiple of 4) of nb elements each, in 16-byte pieces
+  auto copy = [&](auto* dst, const auto* src, int rows) {
+    constexpr int kSize = sizeof(*dst);
+    unsigned char* const o = reinterpret_cast<unsigned char*>(dst) + 16 * lane;
+    const unsigned char* const i = reinterpret_cast<const unsigned char*>(src) + 16 * lane;
+    if (rows == R && nb == 32) {
+#pragma unroll
+      for (int j = 0; j < R * kSize / 16; ++j) cp_async<16>(o + 512 * j, i + 512 * j);
+    } else {
+      for (int j = 0; j < rows * nb * kSize - 16 * lane; j += 512) cp_async<16>(o + j, i + j);
+    }
+  };
+  // chunk ch to stage st, one commit group (rows 0 and L - 1 have no relation:
+  // what their slots hold is copied and not used)
+  auto fetch = [&](int ch, int st) {
+    if (ch >= 0) {
+      const int row0 = ch * R, rows = min(R, rl.cap - row0);
+      copy(rows_of(st), rel + row0 * nb, rows);
+      if (ch < na) copy(al_of(st), rel_al + row0 * nb, rows);
+      if constexpr (kRef) load_chunk<Tin, R, kVec16>(x_of(st), xsrc, 1, pm, row0);
+    }
+    cp_async_commit();
+  };
+#pragma unroll
+  for (int i = 0; i < kBackStages - 1; ++i) fetch(nch - 1 - i, i);
+  T f = Ar::zero(), l = Ar::zero();
+  if (active) {
+    f = Ar::from(xred[2 * k]);
+    l = Ar::from(xred[2 * k + 1]);
+  }
+  T xn = l;
+  bool oob = false;
+  unsigned long long mdel = 0, mx = 0;  // refinement maxima (bit patterns)
+  int st = 0;
+  for (int ch = nch - 1; ch >= 0; --ch) {
+    const int row0 = ch * R;
+    fetch(ch - (kBackStages - 1), st == 0 ? kBackStages - 1 : st - 1);
+    cp_async_wait<kBackStages - 1>();
+    __syncwarp();  // other lanes' copies
+    const RelRow<T>* const w = rows_of(st) + lane;
+    const T* const wal = al_of(st) + lane;
+    Tin* const tile = x_of(st);
+    Tin* const t = tile + lane * TL::kStride;
+    // x of rows row0 + r; where every lane's rows are interior the tests go
+    auto chunk = [&](auto kMid, auto kAl) {
+      Tin xo[V];
+#pragma unroll
+      for (int r = R - 1; r >= 0; --r) {
+        const int row = row0 + r;
+        T xr = Ar::zero();
+        bool in = active;
+        if (decltype(kMid)::value || (row >= 1 && row < L - 1)) {
+          const RelRow<T> e = w[r * nb];
+          T g = e.g;
+          if constexpr (decltype(kAl)::value) g = Ar::sub_mul(g, wal[r * nb], f);
+          xn = Ar::sub_mul(g, e.c, xn);
+          xr = xn;
+        } else if (row == 0) {
+          xr = f;
+        } else if (row == L - 1) {
+          xr = l;
+        } else {
+          in = false;
+        }
+        Tin xv;
+        Ar::to(xv, xr);
+        oob |= in && Ar::out_bad(xv);
+        if constexpr (kRef) {  // x += delta
+          const Tin xs = t[r] + xv;
+          if (in) {
+            mdel = max(mdel, abs_bits(xv));
+            mx = max(mx, abs_bits(xs));
+          }
+          xv = xs;
+        }
+        xo[r % V] = xv;
+        if (r % V == 0) {
+          Vec16<Tin> o;
+#pragma unroll
+          for (int v = 0; v < V; ++v) o.v[v] = xo[v];
+          *reinterpret_cast<float4*>(t + r) = *reinterpret_cast<const float4*>(&o);
+        }
+      }
+    };
+    const bool mid = ch >= 1 && row0 + R <= lmin - 1;
+    if (mid && ch >= na) chunk(std::true_type{}, std::false_type{});
+    else if (mid) chunk(std::true_type{}, std::true_type{});
+    else if (ch >= na) chunk(std::false_type{}, std::false_type{});
+    else chunk(std::false_type{}, std::true_type{});
+    __syncwarp();
+    store_chunk<Tin, R, kVec16>(x, tile, pm, row0);
+    __syncwarp();  // the slots are refilled by a later chunk
+    st = st == kBackStages - 1 ? 0 : st + 1;
+  }
+  if (oob) atomicOr(status, ST_RANGE);
   if constexpr (kRef) {
     for (int o = 16; o > 0; o >>= 1) {
       mdel = max(mdel, __shfl_xor_sync(0xffffffffu, mdel, o));

@@ -133,6 +133,10 @@ static cudaError_t launch_onchip(tps_plan_s* P, int64_t n, const Tin* a, const T
                                  bool& used, bool codes) {
   used = false;
   if (P->desc.flags & TPS_NO_ONCHIP) return cudaSuccess;
+  if (P->desc.flags & TPS_EXTERNAL_WORKSPACE) {  // the caller may have used it in between
+    const cudaError_t e = cudaMemsetAsync(P->ws + 32, 0, 2 * sizeof(unsigned), s);
+    if (e != cudaSuccess) return e;
+  }
   return launch_onchip_raw<Ar, Tin>(n, a, b, c, d, x, P->ws + P->off_xch,
                                     reinterpret_cast<unsigned*>(P->ws + 32), P->d_status,
                                     P->test_barrier_extra, s, used, codes);
@@ -173,8 +177,8 @@ Level make_level(int64_t n, int m, int R) {
   return lv;
 }
 
-size_t build_levels(int64_t n, int m0, int mr, size_t top_elem, size_t red_elem, size_t base,
-                    std::vector<LevelPlan>& out) {
+size_t build_levels(int64_t n, int m0, int mr, size_t top_elem, size_t red_elem, bool rel,
+                    size_t base, std::vector<LevelPlan>& out) {
   out.clear();
   size_t off = base;
   int64_t N = n;
@@ -189,10 +193,21 @@ size_t build_levels(int64_t n, int m0, int mr, size_t top_elem, size_t red_elem,
       L.off_red[i] = off;
       off = align_up(off + (size_t)nr * red_elem);
     }
-    const size_t nck = (size_t)L.lv.ncap * (size_t)L.lv.p;
-    for (int i = 0; i < 3; ++i) {
-      L.off_ck[i] = off;
-      off = align_up(off + nck * red_elem);
+    L.rel = rel;
+    if (rel) {
+      const size_t rows = (size_t)L.lv.p * (size_t)rel_cap(m);
+      L.off_rel[0] = off;
+      off = align_up(off + 2 * rows * red_elem);
+      L.off_rel[1] = off;
+      off = align_up(off + rows * red_elem);
+      L.off_rel[2] = off;
+      off = align_up(off + (size_t)L.lv.p * sizeof(int));
+    } else {
+      const size_t nck = (size_t)L.lv.ncap * (size_t)L.lv.p;
+      for (int i = 0; i < 3; ++i) {
+        L.off_ck[i] = off;
+        off = align_up(off + nck * red_elem);
+      }
     }
     out.push_back(L);
     N = nr;
@@ -242,58 +257,85 @@ static cudaError_t set_smem(K kernel, size_t smem, std::atomic<uint64_t>& done) 
 #ifndef TPS_STAGE1_DIV
 #define TPS_STAGE1_DIV 1
 #endif
+// The workspace buffers of a level: reduced system (ra, rb, rc, rd, xr) and
+// what Stage 1 leaves for Stage 3, relations or checkpoints.
+template <class Tred>
+struct LevelBufs {
+  Tred* red[5];
+  Tred* ck[3];
+  RelIO rl;
+  LevelBufs(tps_plan_s* P, const LevelPlan& L) {
+    for (int i = 0; i < 5; ++i) red[i] = reinterpret_cast<Tred*>(P->ws + L.off_red[i]);
+    for (int i = 0; i < 3; ++i)
+      ck[i] = L.rel ? nullptr : reinterpret_cast<Tred*>(P->ws + L.off_ck[i]);
+    rl = L.rel ? RelIO{P->ws + L.off_rel[0], P->ws + L.off_rel[1],
+                       reinterpret_cast<int*>(P->ws + L.off_rel[2]), rel_cap(L.lv.m)}
+               : RelIO{nullptr, nullptr, nullptr, 0};
+  }
+};
+
 // kRef: a fused refinement step (RefineIO rf; fp64 arrays).
 template <class Ar, class Tin, class Tred, int K, bool kRef = false>
 static cudaError_t launch_stage1(const Level& lv, const Tin* a, const Tin* b, const Tin* c,
-                                 const Tin* d, Tred* ra, Tred* rb, Tred* rc, Tred* rd, Tred* cg,
-                                 Tred* cy, Tred* cv, int* status, cudaStream_t s,
-                                 RefineIO rf = {}) {
+                                 const Tin* d, const LevelBufs<Tred>& B, int* status,
+                                 cudaStream_t s, RefineIO rf = {}) {
   constexpr int W = kWarpsPerCta;
   constexpr int R = K * TPS_STAGE1_MUL / TPS_STAGE1_DIV;
   const size_t smem = stage1_smem_per_warp<Tin, R, kRef ? 5 : 4>() * W;
   const int64_t warps = (lv.k_end - lv.k_begin + 31) / 32;
   const unsigned grid = (unsigned)((warps + W - 1) / W);
   if (grid == 0) return cudaSuccess;
-  const void* ptrs[6] = {a, b, c, d, rf.x, rf.r};
-  cudaError_t e;
-  if (vec16_ok<Tin>(lv.m, ptrs, kRef ? 6 : 4)) {
+  const bool rel = B.rl.rel != nullptr;
+  const void* ptrs[6] = {a, b, c, d, rf.x, rel ? nullptr : rf.r};
+  auto go = [&](auto vec, auto rl) -> cudaError_t {
     static std::atomic<uint64_t> done{0};
-    auto k = k_stage1<Ar, Tin, Tred, R, K, W, true, kRef>;
-    if ((e = set_smem(k, smem, done)) != cudaSuccess) return e;
-    k<<<grid, 32 * W, smem, s>>>(lv, a, b, c, d, ra, rb, rc, rd, cg, cy, cv, status, rf);
-  } else {
-    static std::atomic<uint64_t> done{0};
-    auto k = k_stage1<Ar, Tin, Tred, R, K, W, false, kRef>;
-    if ((e = set_smem(k, smem, done)) != cudaSuccess) return e;
-    k<<<grid, 32 * W, smem, s>>>(lv, a, b, c, d, ra, rb, rc, rd, cg, cy, cv, status, rf);
-  }
-  return cudaGetLastError();
+    auto k = k_stage1<Ar, Tin, Tred, R, K, W, decltype(vec)::value, kRef, decltype(rl)::value>;
+    const cudaError_t e = set_smem(k, smem, done);
+    if (e != cudaSuccess) return e;
+    k<<<grid, 32 * W, smem, s>>>(lv, a, b, c, d, B.red[0], B.red[1], B.red[2], B.red[3], B.ck[0],
+                                 B.ck[1], B.ck[2], status, rf, B.rl);
+    return cudaGetLastError();
+  };
+  const bool vec = vec16_ok<Tin>(lv.m, ptrs, kRef ? 6 : 4);
+  if (rel) return vec ? go(std::true_type{}, std::true_type{})
+                      : go(std::false_type{}, std::true_type{});
+  return vec ? go(std::true_type{}, std::false_type{}) : go(std::false_type{}, std::false_type{});
 }
 
+// d: the right-hand side (a refinement step without relations: the residual).
 template <class Ar, class Tin, class Tred, int R, bool kRef = false>
 static cudaError_t launch_stage3(const Level& lv, const Tin* a, const Tin* b, const Tin* c,
-                                 const Tin* d, const Tred* xr, const Tred* cg, const Tred* cy,
-                                 const Tred* cv, Tin* x, int* status, cudaStream_t s,
-                                 RefineIO rf = {}) {
+                                 const Tin* d, const LevelBufs<Tred>& B, Tin* x, int* status,
+                                 cudaStream_t s, RefineIO rf = {}) {
+  const int64_t warps = (lv.k_end - lv.k_begin + 31) / 32;
+  if (warps == 0) return cudaSuccess;
+  if (B.rl.rel) {  // from the relations: a, b, c, d are not read again
+    const void* xp[1] = {x};
+    auto go = [&](auto vec) -> cudaError_t {
+      static std::atomic<uint64_t> done{0};
+      auto k = k_back<Ar, Tin, Tred, R, decltype(vec)::value, kRef>;
+      constexpr size_t bytes = BackTile<Ar, Tin, R, kRef>::kBytes;
+      const cudaError_t e = set_smem(k, bytes, done);
+      if (e != cudaSuccess) return e;
+      k<<<(unsigned)warps, 32, bytes, s>>>(lv, B.red[4], x, status, B.rl, rf);
+      return cudaGetLastError();
+    };
+    return vec16_ok<Tin>(lv.m, xp, 1) ? go(std::true_type{}) : go(std::false_type{});
+  }
   constexpr int W = kWarpsPerCta;
   const size_t smem = Tile3<Tin, Tred, R, kRef ? 5 : 4>::kBytesPerWarp * W;
-  const int64_t warps = (lv.k_end - lv.k_begin + 31) / 32;
   const unsigned grid = (unsigned)((warps + W - 1) / W);
-  if (grid == 0) return cudaSuccess;
   const void* ptrs[5] = {a, b, c, d, x};
-  cudaError_t e;
-  if (vec16_ok<Tin>(lv.m, ptrs, 5)) {
+  auto go = [&](auto vec) -> cudaError_t {
     static std::atomic<uint64_t> done{0};
-    auto k = k_stage3<Ar, Tin, Tred, R, W, true, kRef>;
-    if ((e = set_smem(k, smem, done)) != cudaSuccess) return e;
-    k<<<grid, 32 * W, smem, s>>>(lv, a, b, c, d, xr, cg, cy, cv, x, status, rf);
-  } else {
-    static std::atomic<uint64_t> done{0};
-    auto k = k_stage3<Ar, Tin, Tred, R, W, false, kRef>;
-    if ((e = set_smem(k, smem, done)) != cudaSuccess) return e;
-    k<<<grid, 32 * W, smem, s>>>(lv, a, b, c, d, xr, cg, cy, cv, x, status, rf);
-  }
-  return cudaGetLastError();
+    auto k = k_stage3<Ar, Tin, Tred, R, W, decltype(vec)::value, kRef>;
+    const cudaError_t e = set_smem(k, smem, done);
+    if (e != cudaSuccess) return e;
+    k<<<grid, 32 * W, smem, s>>>(lv, a, b, c, d, B.red[4], B.ck[0], B.ck[1], B.ck[2], x, status,
+                                 rf);
+    return cudaGetLastError();
+  };
+  return vec16_ok<Tin>(lv.m, ptrs, 5) ? go(std::true_type{}) : go(std::false_type{});
 }
 
 template <class Ar, class Tin, class Tred>
@@ -316,18 +358,13 @@ static cudaError_t run_levels(tps_plan_s* P, const std::vector<LevelPlan>& level
   }
   const LevelPlan& L = levels[idx];
   constexpr int R = kChunkRows<Tin>;
-  Tred* red[5];
-  for (int i = 0; i < 5; ++i) red[i] = reinterpret_cast<Tred*>(P->ws + L.off_red[i]);
-  Tred* ck[3];
-  for (int i = 0; i < 3; ++i) ck[i] = reinterpret_cast<Tred*>(P->ws + L.off_ck[i]);
-  cudaError_t e = launch_stage1<Ar, Tin, Tred, R>(L.lv, a, b, c, d, red[0], red[1], red[2], red[3],
-                                                  ck[0], ck[1], ck[2], P->d_status, s);
+  const LevelBufs<Tred> B(P, L);
+  cudaError_t e = launch_stage1<Ar, Tin, Tred, R>(L.lv, a, b, c, d, B, P->d_status, s);
   if (e != cudaSuccess) return e;
-  e = run_levels<Ar, Tred, Tred>(P, levels, idx + 1, 2 * L.lv.p, red[0], red[1], red[2], red[3],
-                                 red[4], s);
+  e = run_levels<Ar, Tred, Tred>(P, levels, idx + 1, 2 * L.lv.p, B.red[0], B.red[1], B.red[2],
+                                 B.red[3], B.red[4], s);
   if (e != cudaSuccess) return e;
-  return launch_stage3<Ar, Tin, Tred, R>(L.lv, a, b, c, d, red[4], ck[0], ck[1], ck[2], x,
-                                         P->d_status, s);
+  return launch_stage3<Ar, Tin, Tred, R>(L.lv, a, b, c, d, B, x, P->d_status, s);
 }
 
 // ------------------------------------------------------------------ kernel copies
@@ -396,13 +433,8 @@ cudaError_t stage1_range(tps_plan_s* P, const LevelPlan& L, int64_t kb, int64_t 
     lv.k_begin = kb;
     lv.k_end = ke;
     lv.dmax = level0_dmax(P);
-    Tred* red[4];
-    for (int i = 0; i < 4; ++i) red[i] = reinterpret_cast<Tred*>(P->ws + L.off_red[i]);
-    Tred* ck[3];
-    for (int i = 0; i < 3; ++i) ck[i] = reinterpret_cast<Tred*>(P->ws + L.off_ck[i]);
     return launch_stage1<Ar, Tin, Tred, R>(lv, (const Tin*)a, (const Tin*)b, (const Tin*)c,
-                                           (const Tin*)d, red[0], red[1], red[2], red[3], ck[0],
-                                           ck[1], ck[2], P->d_status, s);
+                                           (const Tin*)d, LevelBufs<Tred>(P, L), P->d_status, s);
   });
 }
 
@@ -417,11 +449,8 @@ cudaError_t stage3_range(tps_plan_s* P, const LevelPlan& L, int64_t kb, int64_t 
     Level lv = L.lv;
     lv.k_begin = kb;
     lv.k_end = ke;
-    const Tred* xr = reinterpret_cast<const Tred*>(P->ws + L.off_red[4]);
-    const Tred* ck[3];
-    for (int i = 0; i < 3; ++i) ck[i] = reinterpret_cast<const Tred*>(P->ws + L.off_ck[i]);
     return launch_stage3<Ar, Tin, Tred, R>(lv, (const Tin*)a, (const Tin*)b, (const Tin*)c,
-                                           (const Tin*)d, xr, ck[0], ck[1], ck[2], (Tin*)x,
+                                           (const Tin*)d, LevelBufs<Tred>(P, L), (Tin*)x,
                                            P->d_status, s);
   });
 }
@@ -438,22 +467,17 @@ cudaError_t refine_step(tps_plan_s* P, const std::vector<LevelPlan>& levels, con
   constexpr int R = kChunkRows<Tin>;
   const LevelPlan& L = levels[0];
   const RefineIO rf{x, r, max2};
-  Tred* red[5];
-  for (int i = 0; i < 5; ++i) red[i] = reinterpret_cast<Tred*>(P->ws + L.off_red[i]);
-  Tred* ck[3];
-  for (int i = 0; i < 3; ++i) ck[i] = reinterpret_cast<Tred*>(P->ws + L.off_ck[i]);
+  const LevelBufs<Tred> B(P, L);
   Level lv = L.lv;
   lv.k_begin = 0;
   lv.k_end = lv.p;
   lv.dmax = nullptr;  // a residual's range codes are not judged
   cudaError_t e = cudaMemsetAsync(max2, 0, 2 * sizeof(unsigned long long), s);
   if (e == cudaSuccess)
-    e = launch_stage1<Ar, Tin, Tred, R, true>(lv, a, b, c, d, red[0], red[1], red[2], red[3],
-                                              ck[0], ck[1], ck[2], P->d_status, s, rf);
+    e = launch_stage1<Ar, Tin, Tred, R, true>(lv, a, b, c, d, B, P->d_status, s, rf);
   if (e == cudaSuccess) e = reduced_solve(P, levels, s);
   if (e == cudaSuccess)
-    e = launch_stage3<Ar, Tin, Tred, R, true>(lv, a, b, c, r, red[4], ck[0], ck[1], ck[2], x,
-                                              P->d_status, s, rf);
+    e = launch_stage3<Ar, Tin, Tred, R, true>(lv, a, b, c, r, B, x, P->d_status, s, rf);
   return e;
 }
 
@@ -494,7 +518,7 @@ cudaError_t reduced_solve_graph(tps_plan_s* P, const std::vector<LevelPlan>& lev
                                 cudaStream_t s) {
   const Level& L0 = levels[0].lv;
   const int64_t key[12] = {2 * L0.p, (int64_t)levels.size(), P->m_reduced, (int64_t)P->ws,
-                           P->desc.dtype, (int64_t)levels[0].off_red[0], 0, 0, 0, 0, 0, 0};
+                           P->desc.dtype, (int64_t)levels[0].off_red[0], levels[0].rel, 0, 0, 0, 0, 0};
   bool same = P->graph != nullptr;
   for (int i = 0; i < 12 && same; ++i) same = P->gkey[i] == key[i];
   if (!same) {

@@ -53,6 +53,7 @@ static cudaError_t ensure_streams(HostPipe* H, int S) {
   return e;
 }
 constexpr int32_t kTuneMin = 16, kTuneMax = 1024;  // autotuner block-size grid
+constexpr int64_t kRelRowsMax = (int64_t)1 << 30;   // see tps_plan
 
 static cudaEvent_t* next_trace(tps_plan_s* P) {
   if (!P->trace_ev) return nullptr;
@@ -62,14 +63,27 @@ static cudaEvent_t* next_trace(tps_plan_s* P) {
 }
 
 // Defaults when the caller leaves a parameter at 0 and no predictor is asked
-// for.  Block size 128: at n = 2^27 within 1.4% of the best block size on
-// every GB300 measured (m = 64 is 1.4% faster on some boxes and 2.1% slower
-// on others; tps_autotune picks per box); a small system keeps at least ~4
-// blocks per SM so the per-lane serial sweeps run in parallel.
+// for.  Block size: the level-0 kernels run ten warps of 32 blocks on each of
+// 152 SMs at a time (20 KB of shared memory a warp).  A system that cannot
+// fill them twice takes 6.4 warps an SM (the sweeps are serial, so fewer and
+// longer blocks only wait, more and shorter ones cost reduced rows); a larger
+// one the longest blocks of at most 256 rows whose warps fill their last wave.
+// Measured, us a solve, against 128 rows at every size: double-float 2e6 rows
+// 58 (64), fp64 1e8 rows 2033 (2160), double-float 1e8 1208 (1206).
 static void default_params(const tps_plan_desc& d, int32_t& m, int32_t& mr, int32_t& S) {
   if (m == 0) {
-    m = 128;
-    while (m > 8 && d.n_max / m < 152 * 32 * 4) m /= 2;
+    const int64_t step = d.dtype == TPS_F32 ? 16 : 8;  // whole chunks
+    auto up = [&](int64_t v) { return std::max(step, (v + step - 1) / step * step); };
+    constexpr int64_t kWave = 32 * 152 * 10, kSmall = 32 * 152 * 64 / 10;
+    int64_t v = up((d.n_max + kSmall - 1) / kSmall);
+    for (int64_t k = 2; v > 128; ++k) {
+      const int64_t w = up((d.n_max + kWave * k - 1) / (kWave * k));
+      if (w <= 256) {
+        v = w;
+        break;
+      }
+    }
+    m = (int32_t)v;
   }
   if (mr == 0) mr = 32;
   if (S == 0) S = (d.residency == TPS_HOST_PINNED) ? 4 : 1;
@@ -94,7 +108,7 @@ static size_t workspace_for(tps_plan_s* P, size_t* off_levels_out, size_t* off_d
   const size_t eio = elem_bytes_io(P->desc.dtype);
   const size_t ered = elem_bytes_red(P->desc.dtype);
   int64_t nmax = P->desc.n_max;
-  size_t end = build_levels(nmax, P->m, P->m_reduced, eio, ered, off, lv);
+  size_t end = build_levels(nmax, P->m, P->m_reduced, eio, ered, P->rel, off, lv);
   if (P->desc.dtype == TPS_MIXED_F32_F64) {
     // residual r and correction delta (fp64)
     P->off_refine = end;
@@ -206,21 +220,27 @@ tps_status tps_plan(const tps_plan_desc* desc, tps_plan_t* out) {
   default_params(d, P->m, P->m_reduced, P->streams);
 
   size_t off_levels = 0, off_dev = 0;
-  if (d.flags & TPS_TUNE_EXHAUSTIVE) {
-    // the autotuner's smallest block size needs the largest workspace
-    const int32_t keep = P->m;
-    P->m = kTuneMin;
-    P->ws_needed = workspace_for(P, &off_levels, &off_dev);
-    P->m = keep;
-    size_t o2 = 0, d2 = 0;
-    const size_t own = workspace_for(P, &o2, &d2);
-    if (own > P->ws_needed) {
-      P->ws_needed = own;
-      off_dev = d2;
+  auto size_workspace = [&]() {
+    if (d.flags & TPS_TUNE_EXHAUSTIVE) {
+      // the autotuner's smallest block size needs the largest workspace
+      const int32_t keep = P->m;
+      P->m = kTuneMin;
+      P->ws_needed = workspace_for(P, &off_levels, &off_dev);
+      P->m = keep;
+      size_t o2 = 0, d2 = 0;
+      const size_t own = workspace_for(P, &o2, &d2);
+      if (own > P->ws_needed) {
+        P->ws_needed = own;
+        off_dev = d2;
+      }
+    } else {
+      P->ws_needed = workspace_for(P, &off_levels, &off_dev);
     }
-  } else {
-    P->ws_needed = workspace_for(P, &off_levels, &off_dev);
-  }
+  };
+  // relations: up to kRelRowsMax rows (25 GB of workspace); above, and where
+  // that much memory is not free, Stage 3 works from checkpoints
+  P->rel = d.n_max <= kRelRowsMax;
+  size_workspace();
   P->off_levels = off_levels;
 
   if (const char* t = std::getenv("TPS_TEST_ONCHIP_TIMEOUT"))
@@ -240,7 +260,6 @@ tps_status tps_plan(const tps_plan_desc* desc, tps_plan_t* out) {
     HostPipe* H = new (std::nothrow) HostPipe();
     if (!H) { delete P; return TPS_ERR_OOM; }
     P->pipe = H;
-    H->off_dev = off_dev;
     cudaError_t e = cudaEventCreateWithFlags(&H->ev_start, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&H->ev_red, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&H->ev_up, cudaEventDisableTiming);
@@ -264,6 +283,12 @@ tps_status tps_plan(const tps_plan_desc* desc, tps_plan_t* out) {
   if (!(d.flags & TPS_EXTERNAL_WORKSPACE)) {
     void* ws = nullptr;
     cudaError_t e = cudaMalloc(&ws, P->ws_needed);
+    if (e != cudaSuccess && P->rel) {
+      cudaGetLastError();
+      P->rel = false;
+      size_workspace();
+      e = cudaMalloc(&ws, P->ws_needed);
+    }
     if (e != cudaSuccess) {
       cudaGetLastError();
       tps_plan_destroy(P);
@@ -280,6 +305,7 @@ tps_status tps_plan(const tps_plan_desc* desc, tps_plan_t* out) {
       return TPS_ERR_CUDA;
     }
   }
+  if (P->pipe) P->pipe->off_dev = off_dev;
   if (d.flags & TPS_HOST_OVERLAP) {
     // the twin: the same plan with the parameters chosen above, fixed
     tps_plan_desc t = P->desc;
@@ -436,7 +462,7 @@ tps_status tps_solve(tps_plan_t P, int64_t n, const void* a, const void* b, cons
   if (P->desc.flags & TPS_TRUNCATE) return run_truncated(P, n, a, b, c, d, x, s);
   std::vector<LevelPlan> lv;
   build_levels(n, P->m, P->m_reduced, elem_bytes_io(P->desc.dtype),
-               elem_bytes_red(P->desc.dtype), P->off_levels, lv);
+               elem_bytes_red(P->desc.dtype), P->rel, P->off_levels, lv);
   P->last_levels = (int32_t)lv.size();
   if (P->desc.dtype == TPS_MIXED_F32_F64)
     return run_refine(P, n, (const double*)a, (const double*)b, (const double*)c,
@@ -472,7 +498,7 @@ tps_status tps_solve_batched(tps_plan_t P, int64_t count, const int64_t* offsets
   P->last_stream = s;
   std::vector<LevelPlan> lv;
   build_levels(n, P->m, P->m_reduced, elem_bytes_io(P->desc.dtype),
-               elem_bytes_red(P->desc.dtype), P->off_levels, lv);
+               elem_bytes_red(P->desc.dtype), P->rel, P->off_levels, lv);
   P->last_levels = (int32_t)lv.size();
   // system boundaries strictly inside [0, n): offsets[1 .. count-1]
   const int64_t* bnd = count > 1 ? offsets + 1 : nullptr;
@@ -511,7 +537,8 @@ tps_status tps_solve_host_async(tps_plan_t P, int64_t n, const void* a, const vo
                                   (const unsigned char*)c, (const unsigned char*)d,
                                   (const unsigned char*)x};
   std::vector<LevelPlan> lv;
-  build_levels(n, P->m, P->m_reduced, es, elem_bytes_red(P->desc.dtype), P->off_levels, lv);
+  build_levels(n, P->m, P->m_reduced, es, elem_bytes_red(P->desc.dtype), P->rel,
+               P->off_levels, lv);
   P->last_levels = (int32_t)lv.size();
   const int S = P->streams;  // the plan's S (the pipe may hold more streams)
   cudaError_t e = cudaEventRecord(H->ev_start, us);

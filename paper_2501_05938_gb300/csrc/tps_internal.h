@@ -37,6 +37,8 @@ struct LevelPlan {
   int R;
   size_t off_red[5];  // ra, rb, rc, rd, xr
   size_t off_ck[3];   // gamma, y, v
+  bool rel;           // Stage 1 writes relations (RelIO) instead of checkpoints
+  size_t off_rel[3];  // relation rows, al, na
 };
 
 // Block geometry for n rows and nominal block length m (m >= 2, n > m is
@@ -51,9 +53,10 @@ Level make_level(int64_t n, int m, int R);
 
 // Levels of the recursive solve of an n-row system (empty when n fits the
 // one-warp base solve), with workspace offsets starting at `base`; returns
-// the end offset.
-size_t build_levels(int64_t n, int m0, int mr, size_t top_elem, size_t red_elem, size_t base,
-                    std::vector<LevelPlan>& out);
+// the end offset.  rel: Stage 3 from relations (24 bytes of workspace per row
+// and 8-byte element) instead of from checkpoints.
+size_t build_levels(int64_t n, int m0, int mr, size_t top_elem, size_t red_elem, bool rel,
+                    size_t base, std::vector<LevelPlan>& out);
 
 struct HostPipe;  // streams and events of tps_solve_host_async
 
@@ -77,6 +80,7 @@ struct tps_plan_s {
   bool codes_off = false;
   double* d_scalars = nullptr; // refinement reductions (next bytes of ws)
   size_t off_levels = 0;       // first level buffer offset
+  bool rel = false;            // the levels keep relations (see build_levels)
   size_t off_refine = 0;       // refinement residual and correction vectors
   cudaStream_t last_stream = nullptr;
   int32_t last_levels = 0;

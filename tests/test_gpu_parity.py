@@ -597,3 +597,51 @@ def test_distinct_plans_from_two_host_threads():
         assert info["status"] == 0 and info["onchip"] == 0
         assert oracle.rel_forward_error(x, ref) <= F64_FWD
         assert oracle.rel_residual(s["a"], s["b"], s["c"], s["d"], x) <= F64_RES
+
+
+# Stage 3 from relations: Stage 1 drops the terms of the block's first unknown
+# once they have decayed, which rests on dominant rows.
+def _weak_rows(n, seed, m):
+    """Rows that decouple from the block's first unknown at once (|a|, |c| of
+    1e-3), then, 64 rows into every block, a stretch of barely dominant rows
+    (b = |a| + |c| + 1e-3), along which nothing decays."""
+    rng = np.random.default_rng(seed)
+    a, c = rng.uniform(-1, 1, n), rng.uniform(-1, 1, n)
+    r = np.arange(n) % m
+    calm = r < 64
+    a[calm] *= 1e-3
+    c[calm] *= 1e-3
+    a[0] = c[-1] = 0.0
+    b = np.abs(a) + np.abs(c) + np.where(calm, 1.0, 1e-3)
+    x = rng.uniform(-1, 1, n)
+    d = b * x
+    d[1:] += a[1:] * x[:-1]
+    d[:-1] += c[:-1] * x[1:]
+    return {"a": a, "b": b, "c": c, "d": d}
+
+
+@pytest.mark.parametrize("dtype", ["f64", "f64_df", "f32"])
+@pytest.mark.parametrize("kind", ["weak", "not_dominant"])
+def test_relations_with_rows_that_stop_decaying(dtype, kind):
+    """Also with rows that are not dominant (a = 1.5 b in one row of some
+    blocks, after everything has decayed): the warp starts over and keeps
+    every term.  The condition number stays below 1e4 in both, times the unit
+    roundoff (2^-53, 2^-46, 2^-24)."""
+    n, m = 128 * 700 + 57, 128
+    s = _weak_rows(n, 7, m)
+    if kind == "not_dominant":
+        k = np.arange(90, n, 128 * 45)
+        s["a"][k], s["b"][k], s["c"][k] = 1.5, 1.0, 0.0
+        s["d"][k] = 0.5
+    tdt = torch.float64
+    if dtype == "f32":
+        s, tdt = synth.to_f32(s), torch.float32
+    a, b, c, d = (torch.as_tensor(np.ascontiguousarray(s[k])).to("cuda", tdt) for k in "abcd")
+    x = torch.full_like(b, float("nan"))
+    plan = binding.Plan(n, dtype=dtype, m=m, flags=binding.NO_ONCHIP)
+    plan.solve(a, b, c, d, x)
+    torch.cuda.synchronize()
+    assert plan.query()["status"] == 0
+    ref = oracle.thomas(*(np.asarray(s[k], dtype=np.float64) for k in "abcd"))
+    ulp = {"f64": 2.0 ** -53, "f64_df": 2.0 ** -46, "f32": 2.0 ** -24}[dtype]
+    assert oracle.rel_forward_error(x.double().cpu().numpy(), ref) <= 1e4 * ulp
