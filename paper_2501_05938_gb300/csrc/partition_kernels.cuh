@@ -3,9 +3,12 @@
 // interface unknowns, a reduced interface solve, per-block recovery).
 //
 // System: a[i] x[i-1] + b[i] x[i] + c[i] x[i+1] = d[i]; a[0], c[n-1] unused.
-// Blocks: block k owns rows k*m .. k*m + L_k - 1, L_k = m except the last
-// block, whose length Llast lies in [2, m + 1] (a one-row tail is merged into
-// the block before it).  The first and last row of each block are its
+// Blocks: block k owns rows k*m .. k*m + m - 1.  The last block's rows past
+// the system's end are taken as decoupled identity rows (b that of the last
+// row, a = c = d = 0): the loads fill them in shared memory, the stores leave
+// them out, and every lane sweeps m rows alike (a last block of its own length
+// sent its whole warp through the row-by-row path: 20 us of 87 at n = 3e6).
+// The first and last row of each block are its
 // interface unknowns f_k and l_k; the reduced system in (f_0, l_0, f_1, ...)
 // is tridiagonal: row 2k is block k's "first" equation in (l_{k-1}, f_k, l_k)
 // and row 2k+1 its "last" equation in (f_k, l_k, f_{k+1}).
@@ -59,7 +62,7 @@ struct Level {
   const int64_t* bnd;  // batched systems: first rows of systems 1.., sorted (device)
   int64_t nbnd;        // number of such rows (0: one system)
   int32_t m;        // nominal block length
-  int32_t llast;    // length of block p-1, in [2, m+1]
+  int32_t llast;    // rows of block p-1 inside the system, in [1, m]
   int32_t ncap;     // checkpoint slots per block
   int32_t pad;
   // level 0 of fp64 inputs in narrower arithmetic: per system (nbnd + 1
@@ -74,7 +77,8 @@ __device__ __forceinline__ int block_len(const Level& lv, int64_t k) {
 
 // Systems packed back to back are solved as one system whose couplings are
 // cut at every system boundary: a of a system's first row and c of its last
-// row are taken as 0 (they are never read).  A block may straddle
+// row are taken as 0, whatever is stored there: they are overwritten in the
+// chunk's shared-memory slots (cut_chunk).  A block may straddle
 // boundaries; its recurrences then decouple exactly there.  Each lane keeps
 // the boundaries that touch its block, bnd[first .. first+cnt).
 struct Bounds {
@@ -99,19 +103,6 @@ struct Bounds {
     if (lv.nbnd == 0 || !active) return;
     first = lower(lv.bnd, lv.nbnd, start);
     cnt = (int)(lower(lv.bnd, lv.nbnd, start + len + 1) - first);
-  }
-  // a boundary within rows [g0, g0 + rows] (the chunk, or its successor row)
-  __device__ __forceinline__ bool touches(int64_t g0, int rows) const {
-    for (int j = 0; j < cnt; ++j) {
-      const int64_t o = bnd[first + j];
-      if (o >= g0 && o <= g0 + rows) return true;
-    }
-    return false;
-  }
-  __device__ __forceinline__ bool is(int64_t row) const {
-    for (int j = 0; j < cnt; ++j)
-      if (bnd[first + j] == row) return true;
-    return false;
   }
 };
 
@@ -245,9 +236,9 @@ struct RelIO {
   void* rel;  // RelRow<T>
   void* al;   // T
   int* na;    // one per block, used at each warp's first
-  int cap;    // rows per block: m + 1, rounded up to 4 (16-byte chunk starts)
+  int cap;    // rows per block: m, rounded up to 4 (16-byte chunk starts)
 };
-__host__ __device__ constexpr int rel_cap(int m) { return (m + 4) / 4 * 4; }
+__host__ __device__ constexpr int rel_cap(int m) { return (m + 3) / 4 * 4; }
 
 // Pieces of the current x a Stage-1 refinement chunk needs: its R rows and
 // the next piece (the row below the chunk), i.e. kPieces + 1 pieces filling
@@ -295,13 +286,15 @@ struct PieceMap {
   int64_t goff[TL::kPieces];  // element offset of the piece in the arrays (chunk 0)
   int soff[TL::kPieces];      // element offset in a buffer's array
   int row[TL::kPieces];       // first row of the piece within its block (chunk 0)
-  int len[TL::kPieces];       // length of the piece's block, 0 past the last block
+  int len[TL::kPieces];       // rows of the piece's block, 0 past the last block
+  int m;                      // nominal block length (a last block may be shorter)
   __device__ __forceinline__ void init(const Level& lv, int64_t k0, int nb, int lane);
 };
 
 template <class Tin, int R>
 __device__ __forceinline__ void PieceMap<Tin, R>::init(const Level& lv, int64_t k0, int nb,
                                                        int lane) {
+  m = lv.m;
 #pragma unroll
   for (int j = 0; j < TL::kPieces; ++j) {
     const int q = lane + 32 * j;
@@ -317,7 +310,9 @@ __device__ __forceinline__ void PieceMap<Tin, R>::init(const Level& lv, int64_t 
 // Copy rows [row0, row0 + R) of the warp's blocks (clipped to each block's
 // length) of src[0..n_arr) into the buffer's arrays.  kVec16: whole pieces
 // go as one 16-byte copy (arrays 16-byte aligned, m a multiple of kVec);
-// otherwise, and for a block's ragged last piece, element by element.
+// otherwise, and for a block's ragged last piece, element by element.  With
+// n_arr = 4 (a, b, c, d) the rows past a short last block become identity
+// rows of its last row's scale.
 template <class Tin, int R, bool kVec16, class PM>
 __device__ __forceinline__ void load_chunk(Tin* buf, const Tin* const* src, int n_arr,
                                            const PM& pm, int row0) {
@@ -328,14 +323,37 @@ __device__ __forceinline__ void load_chunk(Tin* buf, const Tin* const* src, int 
     const int64_t g = pm.goff[j] + row0;
     if (kVec16 && avail >= TL::kVec) {
       for (int t = 0; t < n_arr; ++t) cp_async<16>(buf + t * TL::kArr + pm.soff[j], src[t] + g);
-    } else if (avail > 0) {
+    } else if (avail > 0 || (pm.len[j] > 0 && pm.len[j] < pm.m)) {
 #pragma unroll
-      for (int v = 0; v < TL::kVec; ++v)
-        if (v < avail)
+      for (int v = 0; v < TL::kVec; ++v) {
+        if (v < avail) {
           for (int t = 0; t < n_arr; ++t)
             cp_async<sizeof(Tin)>(buf + t * TL::kArr + pm.soff[j] + v, src[t] + g + v);
+        } else if (n_arr == 4 && pm.len[j] < pm.m) {
+          Tin* const o = buf + pm.soff[j] + v;
+          o[0] = o[2 * TL::kArr] = o[3 * TL::kArr] = Tin{};
+          cp_async<sizeof(Tin)>(o + TL::kArr, src[1] + (g + avail - 1));
+        }
+      }
     }
   }
+}
+
+// The couplings that leave a system, zeroed in the lane's own slots t of the
+// chunk at row0: a[0], c[n-1] (cut_chunk), and at a boundary `o` rows into
+// the lane's block a of the row and c of the row above it (cut_boundary).
+template <class Tin, int R, int kArr>
+__device__ __forceinline__ void cut_chunk(Tin* t, const Level& lv, int64_t k, int row0) {
+  if (k == 0 && row0 == 0) t[0] = Tin{};
+  if (k == lv.p - 1) {
+    const int r = lv.llast - 1 - row0;
+    if (r >= 0 && r < R) t[2 * kArr + r] = Tin{};
+  }
+}
+template <class Tin, int R, int kArr>
+__device__ __forceinline__ void cut_boundary(Tin* t, int o, int row0) {
+  if (o >= row0 && o < row0 + R) t[o - row0] = Tin{};
+  if (o > row0 && o <= row0 + R) t[2 * kArr + o - 1 - row0] = Tin{};
 }
 
 // Write rows [row0, row0 + R) of the warp's blocks from the buffer's first
@@ -359,8 +377,8 @@ __device__ __forceinline__ void store_chunk(Tin* __restrict__ x, const Tin* buf,
 }
 
 // Rows [row0, row0 + R] of the current x for the warp's blocks: every row up
-// to and including the one below the block (the next block's first row),
-// clipped to the array's n rows.
+// to and including the one below the block (the next block's first row);
+// 0 past the array's n rows.
 template <class Tin, int R, bool kVec16>
 __device__ __forceinline__ void load_xchunk(Tin* buf, const Tin* x, const XPieceMap<Tin, R>& xm,
                                             int row0, int64_t n) {
@@ -372,10 +390,12 @@ __device__ __forceinline__ void load_xchunk(Tin* buf, const Tin* x, const XPiece
     const int64_t avail = min((int64_t)(xm.len[j] + 1 - (row0 + xm.row[j])), n - g);
     if (kVec16 && avail >= TL::kVec) {
       cp_async<16>(buf + xm.soff[j], x + g);
-    } else if (avail > 0) {
+    } else {
 #pragma unroll
-      for (int v = 0; v < TL::kVec; ++v)
+      for (int v = 0; v < TL::kVec; ++v) {
         if (v < avail) cp_async<sizeof(Tin)>(buf + xm.soff[j] + v, x + g + v);
+        else if (g + v >= n) buf[xm.soff[j] + v] = Tin{};
+      }
     }
   }
 }
@@ -398,33 +418,10 @@ __device__ __forceinline__ unsigned long long abs_bits(double v) {
   return ((unsigned long long)hi << 32) | lo;
 }
 
-// chunks the warp iterates: the longest block of the warp decides
-__device__ __forceinline__ int warp_chunks(const Level& lv, int64_t k0, int nb, int R) {
-  const int lmax = (k0 + nb == lv.p) ? max(lv.m, lv.llast) : lv.m;
-  return (lmax + R - 1) / R;
-}
-// shortest block among the warp's active lanes
-__device__ __forceinline__ int warp_lmin(const Level& lv, int64_t k0, int nb) {
-  return (k0 + nb == lv.p) ? min(lv.m, lv.llast) : lv.m;
-}
-// the block length every active lane of the warp has, or 0 if they differ
-__device__ __forceinline__ int warp_luni(const Level& lv, int64_t k0, int nb) {
-  return (k0 + nb == lv.p) ? (lv.llast == lv.m ? lv.m : 0) : lv.m;
-}
-
-// Chunks that every active lane sees the same way run unrolled: all rows
-// interior (kMid), the block's first row f and then interior rows (kFirst,
-// chunk 0), or interior rows and then the block's last row l (kLast, when
-// every lane's block ends with the chunk).  Any other chunk (a ragged last
-// block, a packed-system boundary in or next to the chunk) goes row by row.
-enum ChunkKind : int { kSlow = -1, kMid = 0, kFirst = 1, kLast = 2 };
-__device__ __forceinline__ int chunk_kind(int ch, int row0, int R, int lmin, int luni,
-                                          bool clean) {
-  if (!clean) return kSlow;
-  if (ch >= 1 && row0 + R <= lmin - 1) return kMid;
-  if (ch == 0 && R <= lmin - 1) return kFirst;
-  if (ch >= 1 && luni > 0 && row0 + R == luni) return kLast;
-  return kSlow;
+// Is v +-0, from its bits?  (A coupling that was cut: the x beside it, which
+// may belong to another system, must not reach this one as 0 * inf.)
+__device__ __forceinline__ bool is_zero(double v) {
+  return (((unsigned)__double2hiint(v) & 0x7FFFFFFFu) | (unsigned)__double2loint(v)) == 0u;
 }
 
 // ------------------------------------------------------------------ Stage 1
@@ -470,10 +467,8 @@ __global__ void __launch_bounds__(W * 32)
   const int nb = (int)(lv.k_end - k0 < 32 ? lv.k_end - k0 : 32);
   const int64_t k = k0 + lane;
   const bool active = lane < nb;
-  const int L = active ? block_len(lv, k) : 0;
-  const int nch = warp_chunks(lv, k0, nb, R);
-  const int lmin = warp_lmin(lv, k0, nb);
-  const int luni = warp_luni(lv, k0, nb);
+  const int L = lv.m;
+  const int nch = (L + R - 1) / R;
 
   Tin* tile = reinterpret_cast<Tin*>(smem_raw) + warp * kS1Stages * TL::kBuf;
   const Tin* const srcs[4] = {a, b, c, d};
@@ -495,7 +490,10 @@ __global__ void __launch_bounds__(W * 32)
   for (int c = 0; c < kS1Stages - 1; ++c) fetch(c);
   const int64_t start = k * (int64_t)lv.m;
   Bounds bd;
-  bd.init(lv, start, L, active);
+  bd.init(lv, start, active ? block_len(lv, k) : 0, active);
+  int bj = 0;               // boundaries passed
+  int bnext = 0x7FFFFFFF;   // the next one, in rows from the block's first
+  if (bd.cnt > 0) bnext = (int)(bd.bnd[bd.first] - start);
   // refinement: x of the row above the current one (the previous block's
   // last row before the block's first row)
   Tin xup = Tin{};
@@ -609,13 +607,48 @@ __global__ void __launch_bounds__(W * 32)
     __syncwarp();
     Tin* const tb = tile + (ch % kS1Stages) * TL::kBuf;
     Tin* const t = tb + lane * TL::kStride;
-    const bool clean = !__any_sync(0xffffffffu, bd.cnt > 0 && bd.touches(start + row0, R));
-    const int kind = chunk_kind(ch, row0, R, lmin, luni, clean);
-    // one unrolled body for the three kinds (only row 0 and row R-1 test,
-    // warp-uniformly, whether they are the block's f or l row), compiled
-    // with and without the first unknown's chain
+    cut_chunk<Tin, R, TL::kArr>(t, lv, k, row0);
+    // system boundaries in the lane's rows: the couplings cut, and the codes
+    // of its rows (which belong to two systems or more) taken row by row
+    const bool split = lv.dmax && bnext < row0 + R;
+    unsigned ecode = 0;
+    int rdmax = 0;
+    bool flushed = false;
+    if (bnext <= row0 + R) {
+      int r = 0;
+      while (bnext <= row0 + R) {
+        cut_boundary<Tin, R, TL::kArr>(t, bnext, row0);
+        if (bnext == row0 + R) break;
+        if (split) {
+          for (; r < bnext - row0; ++r) {
+            T av, bv, cv, dv;
+            Ar::template row<true>(t[r], t[TL::kArr + r], t[2 * TL::kArr + r],
+                                   t[3 * TL::kArr + r], av, bv, cv, dv, chk);
+          }
+          codes_raise(lv.dmax, sys, chk.dcode(), chk.ecode, chk.fcode());
+          chk.reset_codes();
+        }
+        ++sys;
+        bnext = ++bj < bd.cnt ? (int)(bd.bnd[bd.first + bj] - start) : 0x7FFFFFFF;
+      }
+      if (split) {
+        for (; r < R && row0 + r < L; ++r) {
+          T av, bv, cv, dv;
+          Ar::template row<true>(t[r], t[TL::kArr + r], t[2 * TL::kArr + r], t[3 * TL::kArr + r],
+                                 av, bv, cv, dv, chk);
+        }
+        ecode = chk.ecode;
+        rdmax = chk.rdmax;
+        flushed = chk.flushed;
+      }
+    }
+    // one unrolled body (only row 0 and row R-1 test, warp-uniformly, whether
+    // they are the block's f or l row), compiled with and without the first
+    // unknown's chain; a last chunk that ends before its R rows (m not a
+    // multiple of R) goes row by row
+    const bool slow = row0 + R > L;
     auto fast_chunk = [&](auto kChain) {
-      const bool first = kind == kFirst, last = kind == kLast;
+      const bool first = ch == 0, last = row0 + R == L;
 #pragma unroll (kRel ? kRelUnroll : R / V)
       for (int r = 0; r < R; r += V) {
         const Vec16<Tin> xa = lds16(t + r), xb = lds16(t + TL::kArr + r),
@@ -623,20 +656,16 @@ __global__ void __launch_bounds__(W * 32)
 #pragma unroll
         for (int v = 0; v < V; ++v) {
           const int rr = r + v;
-          // a of the system's first row and c of its last are never read
-          const bool cut_c = v == V - 1 && rr == R - 1 && last && k == lv.p - 1;
-          const Tin ain = (v == 0 && rr == 0 && first && k == 0) ? Tin{} : xa.v[v];
-          const Tin cin = cut_c ? Tin{} : xc.v[v];
           Tin din = xd.v[v];
           if constexpr (kRef) {  // the residual of the current x
-            const Tin x0 = t[4 * TL::kArr + rr];
-            din = residual_row(ain, xb.v[v], cin, din, xup, x0,
-                               cut_c ? Tin{} : t[4 * TL::kArr + rr + 1]);
+            const Tin x0 = t[4 * TL::kArr + rr], xdn = t[4 * TL::kArr + rr + 1];
+            din = residual_row(xa.v[v], xb.v[v], xc.v[v], din, is_zero(xa.v[v]) ? Tin{} : xup, x0,
+                               is_zero(xc.v[v]) ? Tin{} : xdn);
             xup = x0;
-            t[3 * TL::kArr + rr] = din;
+            if constexpr (!kRel) t[3 * TL::kArr + rr] = din;
           }
           T av, bv, cv, dv;
-          Ar::template row<true>(ain, xb.v[v], cin, din, av, bv, cv, dv, chk);
+          Ar::template row<true>(xa.v[v], xb.v[v], xc.v[v], din, av, bv, cv, dv, chk);
           if (v == 0 && rr == 0 && first) {  // the block's first row: f's equation
             a0 = av; b0 = bv; c0 = cv; d0 = dv;
           } else if (v == V - 1 && rr == R - 1 && last) {  // the block's last row
@@ -654,7 +683,7 @@ __global__ void __launch_bounds__(W * 32)
         }
       }
     };
-    if (kind != kSlow) {
+    if (!slow) {
       if constexpr (kSkip) {
         if (chain) fast_chunk(std::true_type{});
         else fast_chunk(std::false_type{});
@@ -666,29 +695,18 @@ __global__ void __launch_bounds__(W * 32)
       for (int r = 0; r < R; ++r) {
         const int row = row0 + r;
         if (row < L) {
-          // couplings cut at system boundaries (and a[0], c[n-1]) are never read
-          bool cut_a = k == 0 && row == 0, cut_c = k == lv.p - 1 && row == L - 1;
-          if (bd.cnt > 0) {
-            if (bd.is(start + row)) {  // a new packed system starts here
-              cut_a = true;
-              if (lv.dmax) codes_raise(lv.dmax, sys, chk.dcode(), chk.ecode, chk.fcode());
-              chk.reset_codes();
-              ++sys;
-            }
-            cut_c |= bd.is(start + row + 1);
-          }
           Tin din = t[3 * TL::kArr + r];
           if constexpr (kRef) {
-            const Tin x0 = t[4 * TL::kArr + r];
-            din = residual_row(cut_a ? Tin{} : t[r], t[TL::kArr + r],
-                               cut_c ? Tin{} : t[2 * TL::kArr + r], din, cut_a ? Tin{} : xup, x0,
-                               cut_c ? Tin{} : t[4 * TL::kArr + r + 1]);
+            const Tin x0 = t[4 * TL::kArr + r], xdn = t[4 * TL::kArr + r + 1];
+            din = residual_row(t[r], t[TL::kArr + r], t[2 * TL::kArr + r], din,
+                               is_zero(t[r]) ? Tin{} : xup, x0,
+                               is_zero(t[2 * TL::kArr + r]) ? Tin{} : xdn);
             xup = x0;
             t[3 * TL::kArr + r] = din;
           }
           T av, bv, cv, dv;
-          Ar::template row<true>(cut_a ? Tin{} : t[r], t[TL::kArr + r],
-                                 cut_c ? Tin{} : t[2 * TL::kArr + r], din, av, bv, cv, dv, chk);
+          Ar::template row<true>(t[r], t[TL::kArr + r], t[2 * TL::kArr + r], din, av, bv, cv, dv,
+                                 chk);
           if (row == 0) {
             a0 = av; b0 = bv; c0 = cv; d0 = dv;
           } else if (row < L - 1) {
@@ -706,6 +724,11 @@ __global__ void __launch_bounds__(W * 32)
           }
         }
       }
+    }
+    if (split) {  // the body took the chunk's rows together
+      chk.ecode = ecode;
+      chk.rdmax = rdmax;
+      chk.flushed = flushed;
     }
     renorm();
     // the checkpoint at the chunk's end (row0 + R is a multiple of K when
@@ -731,6 +754,8 @@ __global__ void __launch_bounds__(W * 32)
         if constexpr (kRef) xup = active && start > 0 ? rf.x[start - 1] : Tin{};
         chk.reset_codes();  // what was raised stays; the rest is seen again
         sys = lv.nbnd > 0 && active ? bd.first : 0;
+        bj = 0;
+        if (bd.cnt > 0) bnext = (int)(bd.bnd[bd.first] - start);
 #pragma unroll
         for (int c = 0; c < kS1Stages - 1; ++c) fetch(c);
         ch = -1;
@@ -751,29 +776,16 @@ __global__ void __launch_bounds__(W * 32)
   }
   if (active) {
     bad |= Ar::bad_pivot(beta);
-    if (L == 1) {
-      // a one-row block is a one-row system (tails are merged otherwise):
-      // b0 f = d0, and a decoupled identity row for the unused l
-      Ar::to(ra[2 * k], Ar::zero());
-      Ar::to(rb[2 * k], b0);
-      Ar::to(rc[2 * k], Ar::zero());
-      Ar::to(rd[2 * k], d0);
-      Ar::to(ra[2 * k + 1], Ar::zero());
-      Ar::to(rb[2 * k + 1], Ar::one());
-      Ar::to(rc[2 * k + 1], Ar::zero());
-      Ar::to(rd[2 * k + 1], Ar::zero());
-    } else {
-      // first equation of block k, unknowns (l_{k-1}, f_k, l_k)
-      Ar::to(ra[2 * k], k == 0 ? Ar::zero() : a0);
-      Ar::to(rb[2 * k], Ar::sub_mul(b0, c0, Q));
-      Ar::to(rc[2 * k], Ar::neg(Ar::mul(c0, S)));
-      Ar::to(rd[2 * k], Ar::sub_mul(d0, c0, P));
-      // last equation of block k, unknowns (f_k, l_k, f_{k+1})
-      Ar::to(ra[2 * k + 1], al);
-      Ar::to(rb[2 * k + 1], beta);
-      Ar::to(rc[2 * k + 1], k == lv.p - 1 ? Ar::zero() : clast);
-      Ar::to(rd[2 * k + 1], g);
-    }
+    // first equation of block k, unknowns (l_{k-1}, f_k, l_k)
+    Ar::to(ra[2 * k], a0);
+    Ar::to(rb[2 * k], Ar::sub_mul(b0, c0, Q));
+    Ar::to(rc[2 * k], Ar::neg(Ar::mul(c0, S)));
+    Ar::to(rd[2 * k], Ar::sub_mul(d0, c0, P));
+    // last equation of block k, unknowns (f_k, l_k, f_{k+1})
+    Ar::to(ra[2 * k + 1], al);
+    Ar::to(rb[2 * k + 1], beta);
+    Ar::to(rc[2 * k + 1], clast);
+    Ar::to(rd[2 * k + 1], g);
     if (bad || chk.b_bad()) atomicOr(status, ST_BAD_PIVOT);
     if (chk.range_bad()) atomicOr(status, ST_RANGE);
   }
@@ -807,10 +819,9 @@ __global__ void __launch_bounds__(W * 32)
   const int nb = (int)(lv.k_end - k0 < 32 ? lv.k_end - k0 : 32);
   const int64_t k = k0 + lane;
   const bool active = lane < nb;
-  const int L = active ? block_len(lv, k) : 0;
-  const int nch = warp_chunks(lv, k0, nb, R);
-  const int lmin = warp_lmin(lv, k0, nb);
-  const int luni = warp_luni(lv, k0, nb);
+  const int L = lv.m;
+  const int len = active ? block_len(lv, k) : 0;  // rows inside the system
+  const int nch = (L + R - 1) / R;
 
   unsigned char* wbase = smem_raw + warp * TL3::kBytesPerWarp;
   Tin* tile = reinterpret_cast<Tin*>(wbase);
@@ -836,7 +847,7 @@ __global__ void __launch_bounds__(W * 32)
 
   const int64_t start = k * (int64_t)lv.m;
   Bounds bd;
-  bd.init(lv, start, L, active);
+  bd.init(lv, start, len, active);
   T f = Ar::zero(), l = Ar::zero();
   if (active) {
     f = Ar::from(xred[2 * k]);
@@ -870,13 +881,14 @@ __global__ void __launch_bounds__(W * 32)
       gp = Ar::from(ck[lane]);
       zp = Ar::sub_mul(Ar::from(ck[32 + lane]), Ar::from(ck[64 + lane]), f);
     }
-    const bool clean = !__any_sync(0xffffffffu, bd.cnt > 0 && bd.touches(start + row0, R));
-    const int kind = chunk_kind(ch, row0, R, lmin, luni, clean);
-    if (kind != kSlow) {
+    cut_chunk<Tin, R, TL::kArr>(t, lv, k, row0);
+    for (int j = 0; j < bd.cnt; ++j)
+      cut_boundary<Tin, R, TL::kArr>(t, (int)(bd.bnd[bd.first + j] - start), row0);
+    if (row0 + R <= L) {
       // unrolled chunk: forward over the interior rows, back-substitution
-      // from the row below; only row 0 (kFirst: f) and row R-1 (kLast: l)
-      // test their role, warp-uniformly
-      const bool first = kind == kFirst, last = kind == kLast;
+      // from the row below; only row 0 (f) and row R-1 (l) test their role,
+      // warp-uniformly
+      const bool first = ch == 0, last = row0 + R == L;
       T Z[R], G[R];
       Tin xo[R];
 #pragma unroll
@@ -914,9 +926,9 @@ __global__ void __launch_bounds__(W * 32)
       for (int r = 0; r < R; ++r) {
         Ar::to(xo[r], Z[r]);
         oob |= Ar::out_bad(xo[r]);
-        if constexpr (kRef) {  // x += delta (lanes past the level's last block: no rows)
+        if constexpr (kRef) {  // x += delta
           const Tin xn = t[4 * TL::kArr + r] + xo[r];
-          if (active) {
+          if (row0 + r < len) {
             mdel = max(mdel, abs_bits(xo[r]));
             mx = max(mx, abs_bits(xn));
           }
@@ -931,8 +943,9 @@ __global__ void __launch_bounds__(W * 32)
         *reinterpret_cast<float4*>(t + r) = *reinterpret_cast<const float4*>(&w);
       }
     } else {
-      // boundary chunk: the same recurrences, row by row, with the pivots and
-      // right-hand sides parked in the lane's b and c slots
+      // a last chunk that ends before its R rows: the same recurrences, row by
+      // row, with the pivots and right-hand sides parked in the lane's b and c
+      // slots
       T* zs = reinterpret_cast<T*>(t + TL::kArr);
       T* gs = reinterpret_cast<T*>(t + 2 * TL::kArr);
 #pragma unroll 1
@@ -942,10 +955,6 @@ __global__ void __launch_bounds__(W * 32)
           T av, bv, cv, dv;
           Ar::template row<false>(t[r], t[TL::kArr + r], t[2 * TL::kArr + r],
                                   t[3 * TL::kArr + r], av, bv, cv, dv, nochk);
-          if (bd.cnt > 0) {  // couplings cut at system boundaries
-            if (bd.is(start + row)) av = Ar::zero();
-            if (bd.is(start + row + 1)) cv = Ar::zero();
-          }
           const T beta = Ar::sub_mul_dom(bv, av, gp);
           bad |= Ar::bad_pivot(beta);
           const T rbeta = Ar::rcp(beta);
@@ -972,8 +981,10 @@ __global__ void __launch_bounds__(W * 32)
           oob |= Ar::out_bad(t[r]);
           if constexpr (kRef) {  // x += delta
             const Tin xn = t[4 * TL::kArr + r] + t[r];
-            mdel = max(mdel, abs_bits(t[r]));
-            mx = max(mx, abs_bits(xn));
+            if (row < len) {
+              mdel = max(mdel, abs_bits(t[r]));
+              mx = max(mx, abs_bits(xn));
+            }
             t[r] = xn;
           }
         }
@@ -1035,9 +1046,9 @@ __global__ void __launch_bounds__(32)
   const int nb = (int)(lv.k_end - k0 < 32 ? lv.k_end - k0 : 32);
   const int64_t k = k0 + lane;
   const bool active = lane < nb;
-  const int L = active ? block_len(lv, k) : 0;
-  const int nch = warp_chunks(lv, k0, nb, R);
-  const int lmin = warp_lmin(lv, k0, nb);
+  const int L = lv.m;
+  const int len = active ? block_len(lv, k) : 0;  // rows inside the system
+  const int nch = (L + R - 1) / R;
   const RelRow<T>* const rel = static_cast<const RelRow<T>*>(rl.rel) + k0 * rl.cap;
   const T* const rel_al = static_cast<const T*>(rl.al) + k0 * rl.cap;
   const int na = rl.na[k0];
@@ -1104,7 +1115,7 @@ __global__ void __launch_bounds__(32)
       for (int r = R - 1; r >= 0; --r) {
         const int row = row0 + r;
         T xr = Ar::zero();
-        bool in = active;
+        const bool in = row < len;
         if (decltype(kMid)::value || (row >= 1 && row < L - 1)) {
           const RelRow<T> e = w[r * nb];
           T g = e.g;
@@ -1115,8 +1126,6 @@ __global__ void __launch_bounds__(32)
           xr = f;
         } else if (row == L - 1) {
           xr = l;
-        } else {
-          in = false;
         }
         Tin xv;
         Ar::to(xv, xr);
@@ -1138,7 +1147,7 @@ __global__ void __launch_bounds__(32)
         }
       }
     };
-    const bool mid = ch >= 1 && row0 + R <= lmin - 1;
+    const bool mid = ch >= 1 && row0 + R <= L - 1;
     if (mid && ch >= na) chunk(std::true_type{}, std::false_type{});
     else if (mid) chunk(std::true_type{}, std::true_type{});
     else if (ch >= na) chunk(std::false_type{}, std::false_type{});

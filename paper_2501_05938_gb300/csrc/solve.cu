@@ -159,21 +159,15 @@ Level make_level(int64_t n, int m, int R) {
   Level lv{};
   lv.n = n;
   lv.m = m;
-  int64_t p = (n + m - 1) / m;
-  int64_t last = n - (p - 1) * (int64_t)m;
-  if (last == 1 && p > 1) {  // merge a one-row tail into the previous block
-    p -= 1;
-    last = m + 1;
-  }
+  const int64_t p = (n + m - 1) / m;
+  const int64_t last = n - (p - 1) * (int64_t)m;
   lv.p = p;
   lv.k_begin = 0;
   lv.k_end = p;
   lv.bnd = nullptr;
   lv.nbnd = 0;
   lv.llast = (int32_t)last;
-  // checkpoint slots: a block of length L has floor((L - 2) / R) of them;
-  // size for the longest block (m + 1) so the count is monotone in n
-  lv.ncap = (m + 1 - 2) >= R ? (m + 1 - 2) / R : 0;
+  lv.ncap = m - 2 >= R ? (m - 2) / R : 0;  // checkpoint slots of a block
   return lv;
 }
 

@@ -65,22 +65,26 @@ static cudaEvent_t* next_trace(tps_plan_s* P) {
 // Defaults when the caller leaves a parameter at 0 and no predictor is asked
 // for.  Block size: the level-0 kernels run ten warps of 32 blocks on each of
 // 152 SMs at a time (20 KB of shared memory a warp).  A system that cannot
-// fill them twice takes 6.4 warps an SM (the sweeps are serial, so fewer and
-// longer blocks only wait, more and shorter ones cost reduced rows); a larger
-// one the longest blocks of at most 256 rows whose warps fill their last wave.
-// Measured, us a solve, against 128 rows at every size: double-float 2e6 rows
-// 58 (64), fp64 1e8 rows 2033 (2160), double-float 1e8 1208 (1206).
+// fill them twice takes 6.4 warps an SM: the sweeps are serial, so fewer and
+// longer blocks only wait, and more and shorter ones cost reduced rows.  A
+// larger one takes the longest blocks of at most 256 rows whose warps fill
+// their last wave.  Native fp64, bound by its pipe and the cheaper a row the
+// longer the block (decayed terms are skipped), takes up to 384 rows, in one
+// wave if that is enough.  Measured, us a solve, against 128 rows throughout:
+// double-float 3e6 rows 71 (80), 9e6 144 (148), 5e7 619 (625); fp64 3e6
+// 99 (105), 9e6 217 (259), 1.8e7 385 (426), 1e8 1945 (2160); fp32 2e6 28 (31).
 static void default_params(const tps_plan_desc& d, int32_t& m, int32_t& mr, int32_t& S) {
   if (m == 0) {
     const int64_t step = d.dtype == TPS_F32 ? 16 : 8;  // whole chunks
     auto up = [&](int64_t v) { return std::max(step, (v + step - 1) / step * step); };
     constexpr int64_t kWave = 32 * 152 * 10, kSmall = 32 * 152 * 64 / 10;
+    const bool f64 = d.dtype == TPS_F64;
+    const int64_t small_max = f64 ? 104 : 256, cap = f64 ? 384 : 256;
     int64_t v = up((d.n_max + kSmall - 1) / kSmall);
-    for (int64_t k = 2; v > 128; ++k) {
-      const int64_t w = up((d.n_max + kWave * k - 1) / (kWave * k));
-      if (w <= 256) {
-        v = w;
-        break;
+    if (v > small_max) {
+      for (int64_t k = f64 ? 1 : 2;; ++k) {
+        v = up((d.n_max + kWave * k - 1) / (kWave * k));
+        if (v <= cap) break;
       }
     }
     m = (int32_t)v;
@@ -240,6 +244,9 @@ tps_status tps_plan(const tps_plan_desc* desc, tps_plan_t* out) {
   // relations: up to kRelRowsMax rows (25 GB of workspace); above, and where
   // that much memory is not free, Stage 3 works from checkpoints
   P->rel = d.n_max <= kRelRowsMax;
+  // test switch: checkpoints at any size
+  if (const char* t = std::getenv("TPS_TEST_CHECKPOINTS"))
+    if (t[0] == '1') P->rel = false;
   size_workspace();
   P->off_levels = off_levels;
 

@@ -42,8 +42,8 @@ struct LevelPlan {
 };
 
 // Block geometry for n rows and nominal block length m (m >= 2, n > m is
-// not required): p = ceil(n/m) blocks, a one-row tail merged into the block
-// before it so every block has >= 2 rows.
+// not required): p = ceil(n/m) blocks, the last one filled up to m rows with
+// identity rows (see partition_kernels.cuh).
 // Argument checks shared by the entry points: managed memory or device
 // memory of `device`, aligned to `align`; the plan's device is current.
 bool device_ptr_ok(const void* p, size_t align, int device);

@@ -84,6 +84,7 @@ namespace tps {
 // (the same mapping as the level-0 kernels' PieceMap).
 template <class Tin, int R>
 struct WinPieces {
+  static constexpr int m = 0;  // rows past a block are never filled (load_chunk)
   using TL = Tile<Tin, R>;
   int64_t goff[TL::kPieces];  // element offset of the piece in the arrays (chunk 0)
   int soff[TL::kPieces];      // element offset in a buffer's array

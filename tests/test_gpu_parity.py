@@ -645,3 +645,64 @@ def test_relations_with_rows_that_stop_decaying(dtype, kind):
     ref = oracle.thomas(*(np.asarray(s[k], dtype=np.float64) for k in "abcd"))
     ulp = {"f64": 2.0 ** -53, "f64_df": 2.0 ** -46, "f32": 2.0 ** -24}[dtype]
     assert oracle.rel_forward_error(x.double().cpu().numpy(), ref) <= 1e4 * ulp
+
+
+# The last block is filled up with identity rows where n is no multiple of m:
+# one real row, a chunk less or more than whole, all but one; relations and
+# (TPS_TEST_CHECKPOINTS) checkpoints; 16-byte and element-wise loads.
+@pytest.mark.parametrize("checkpoints", [False, True])
+@pytest.mark.parametrize("dtype", ["f64", "f64_df", "f32", "mixed"])
+@pytest.mark.parametrize("m,tail", [(64, 1), (64, 2), (64, 17), (64, 48), (64, 63), (51, 1),
+                                    (51, 40), (12, 5), (6, 1)])
+def test_ragged_last_block(dtype, m, tail, checkpoints, monkeypatch):
+    n = m * 70 + tail
+    monkeypatch.setenv("TPS_TEST_CHECKPOINTS", "1" if checkpoints else "0")
+    plan = binding.Plan(n, dtype=dtype, m=m, flags=binding.NO_ONCHIP)
+    monkeypatch.delenv("TPS_TEST_CHECKPOINTS")
+    s = synth.system(300 + n, n)
+    tdt = torch.float64
+    if dtype == "f32":
+        s, tdt = synth.to_f32(s), torch.float32
+    a, b, c, d = (torch.as_tensor(np.ascontiguousarray(s[k])).to("cuda", tdt) for k in "abcd")
+    a[0] = c[-1] = float("nan")  # not part of the system
+    x = torch.full((n + 1,), float("nan"), dtype=tdt, device="cuda")
+    plan.solve(a, b, c, d, x[:n])
+    torch.cuda.synchronize()
+    info = plan.query()
+    assert info["status"] == 0 and info["refine_fused"] == (dtype == "mixed"), info
+    assert torch.isnan(x[n])
+    ref = oracle.thomas(*(np.asarray(s[k], dtype=np.float64) for k in "abcd"))
+    err = oracle.rel_forward_error(x[:n].double().cpu().numpy(), ref)
+    assert err <= (1e-5 if dtype == "f32" else 1e-10)
+
+
+@pytest.mark.parametrize("checkpoints", [False, True])
+@pytest.mark.parametrize("dtype", ["f64", "f64_df", "f32", "mixed"])
+def test_boundaries_at_every_place_of_a_chunk(dtype, checkpoints, monkeypatch):
+    """Systems of 1 to 40 rows and empty ones: boundaries at every row of a
+    chunk, several in one, on chunk and block edges.  The couplings there hold
+    NaN, and one system's right-hand side spans others' range a thousandfold."""
+    rng = np.random.default_rng(9)
+    sizes = np.concatenate([np.arange(1, 41), rng.integers(0, 9, 300), [64, 128, 0, 63, 500]])
+    off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+    n = int(off[-1])
+    s = {k: np.array(v) for k, v in synth.system(77, n, offsets=off).items()}
+    s["d"][off[30]:off[31]] *= 1e3
+    if dtype == "f32":
+        s = synth.to_f32(s)
+    tdt = torch.float32 if dtype == "f32" else torch.float64
+    ref = oracle.thomas_batched(off, *(np.asarray(s[k], dtype=np.float64) for k in "abcd"))
+    a, b, c, d = (torch.as_tensor(np.ascontiguousarray(s[k])).to("cuda", tdt) for k in "abcd")
+    starts = torch.as_tensor(np.unique(off[:-1][sizes > 0]), device="cuda")
+    ends = torch.as_tensor(np.unique(off[1:][sizes > 0]) - 1, device="cuda")
+    a[starts] = float("nan")
+    c[ends] = float("nan")
+    x = torch.full_like(b, float("nan"))
+    monkeypatch.setenv("TPS_TEST_CHECKPOINTS", "1" if checkpoints else "0")
+    plan = binding.Plan(n, dtype=dtype, m=32, batch_max=len(sizes), flags=binding.NO_ONCHIP)
+    monkeypatch.delenv("TPS_TEST_CHECKPOINTS")
+    plan.solve_batched(torch.as_tensor(off, device="cuda"), a, b, c, d, x, host_offsets=off)
+    torch.cuda.synchronize()
+    assert plan.query()["status"] == 0
+    err = oracle.rel_forward_error(x.double().cpu().numpy(), ref)
+    assert err <= (1e-5 if dtype == "f32" else 1e-10)
