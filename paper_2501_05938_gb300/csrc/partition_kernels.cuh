@@ -540,7 +540,7 @@ __global__ void __launch_bounds__(W * 32)
     g = Ar::sub_mul(dv, ratio, g);
     if constexpr (!kRel || decltype(kChain)::value) al = Ar::mul_neg_nn(ratio, al);
     bad |= Ar::bad_pivot(beta);
-    const T rbeta = Ar::rcp(beta);
+    const T rbeta = Ar::rcp_bulk(beta);
     if constexpr (kRel) {
       T gp;
       if constexpr (sizeof(Tin) == 4) {  // bound by memory: round the quotients once
@@ -903,7 +903,7 @@ __global__ void __launch_bounds__(W * 32)
           Ar::template row<false>(xa.v[v], xb.v[v], xc.v[v], xd.v[v], av, bv, cv, dv, nochk);
           const T beta = Ar::sub_mul_dom(bv, av, gp);
           bad |= Ar::bad_pivot(beta);
-          const T rbeta = Ar::rcp(beta);
+          const T rbeta = Ar::rcp_bulk(beta);
           zp = Ar::mul_nn(Ar::sub_mul(dv, av, zp), rbeta);
           gp = Ar::mul_nn(cv, rbeta);
           Z[rr] = zp;
@@ -957,7 +957,7 @@ __global__ void __launch_bounds__(W * 32)
                                   t[3 * TL::kArr + r], av, bv, cv, dv, nochk);
           const T beta = Ar::sub_mul_dom(bv, av, gp);
           bad |= Ar::bad_pivot(beta);
-          const T rbeta = Ar::rcp(beta);
+          const T rbeta = Ar::rcp_bulk(beta);
           zp = Ar::mul_nn(Ar::sub_mul(dv, av, zp), rbeta);
           gp = Ar::mul_nn(cv, rbeta);
           zs[r] = zp;
