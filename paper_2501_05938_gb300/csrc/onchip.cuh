@@ -397,6 +397,7 @@ __global__ void __launch_bounds__(kOcThreads, 1)
   const Tin* const src[4] = {a, b, c, d};
   constexpr int V = 16 / (int)sizeof(Tin);
   const int nv = vec16 ? rows / V : 0;
+  chain_wait();
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     for (int i = tid; i < nv; i += B) cp_async<16>(s0[k] + i * V, src[k] + r0 + i * V);

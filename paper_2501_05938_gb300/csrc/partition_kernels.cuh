@@ -106,6 +106,17 @@ struct Bounds {
   }
 };
 
+// Every kernel of a solve is launched with programmatic stream serialization
+// (launch_chained) and starts with this wait, so it is set up while the kernel
+// before it in the stream still runs, and goes on once that one has completed
+// and its writes are visible: the stream's order as ever, but a boundary
+// between two kernels costs about 0.5 us where an ordinary one costs 1.5 us
+// and is then rounded up to the next 2.048 us (measured back to back: 1 us of
+// work a kernel takes 1.5 against 4.1 us, 5 us of work 5.4 against 8.2).
+__device__ __forceinline__ void chain_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // Status bits written into the device status word.
 enum : int { ST_BAD_PIVOT = 1, ST_NO_CONVERGENCE = 2, ST_TIMEOUT = 4, ST_RANGE = 8 };
 
@@ -153,6 +164,7 @@ __device__ __forceinline__ void codes_raise_warp(unsigned* dmax, int64_t sys, bo
 // codes for the next solve.  One CTA.
 static __global__ void __launch_bounds__(256)
     k_dcode_check(unsigned* __restrict__ dmax, int64_t count, int* __restrict__ status) {
+  chain_wait();
   bool bad = false;
   for (int64_t i = threadIdx.x; i < count; i += blockDim.x) {
     unsigned* p = dmax + kCodes * i;
@@ -476,6 +488,7 @@ __global__ void __launch_bounds__(W * 32)
   pm.init(lv, k0, nb, lane);
   XPieceMap<Tin, R> xpm;
   if constexpr (kRef) xpm.init(lv, k0, nb, lane);
+  chain_wait();
   // chunk c goes to buffer c % kS1Stages, one commit group per chunk
   auto fetch = [&](int c) {
     if (c < nch) {
@@ -839,6 +852,7 @@ __global__ void __launch_bounds__(W * 32)
       cp_async<sizeof(Tred)>(dst + 64 + lane, ck_v + slot);
     }
   };
+  chain_wait();
   load_chunk<Tin, R, kVec16>(tile, srcs, 4, pm, (nch - 1) * R);
   if constexpr (kRef) load_chunk<Tin, R, kVec16>(tile + 4 * TL::kArr, xsrc, 1, pm, (nch - 1) * R);
   load_ck(ckbuf, nch - 1);
@@ -1051,9 +1065,10 @@ __global__ void __launch_bounds__(32)
   const int nch = (L + R - 1) / R;
   const RelRow<T>* const rel = static_cast<const RelRow<T>*>(rl.rel) + k0 * rl.cap;
   const T* const rel_al = static_cast<const T*>(rl.al) + k0 * rl.cap;
-  const int na = rl.na[k0];
   PieceMap<Tin, R> pm;
   pm.init(lv, k0, nb, lane);
+  chain_wait();
+  const int na = rl.na[k0];
   const Tin* const xsrc[1] = {x};
   auto rows_of = [&](int st) {
     return reinterpret_cast<RelRow<T>*>(smem_raw + st * BT::kStage);
@@ -1191,6 +1206,7 @@ __global__ void __launch_bounds__(32)
   const int lane = threadIdx.x;
   const int nn = (int)n;
   bool bad = false, oob = false;
+  chain_wait();
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     const int i = lane + 32 * h;

@@ -117,6 +117,12 @@ static cudaError_t launch_onchip_raw(int64_t n, const Tin* a, const Tin* b, cons
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
+  // one CTA has no barrier, so it need not be a cooperative launch, which
+  // cannot be chained
+  if (g.G == 1 && !extra_arrival) {
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+  }
   const OcShared sh{bar, (unsigned)g.G + (extra_arrival ? 1u : 0u), status, report,
                     own_status ? 1 : 0};
   const cudaError_t e =
@@ -151,8 +157,7 @@ unsigned* level0_dmax(tps_plan_s* P) {
 cudaError_t dcode_check(tps_plan_s* P, int64_t count, cudaStream_t s) {
   unsigned* dmax = level0_dmax(P);
   if (!dmax) return cudaSuccess;
-  k_dcode_check<<<1, 256, 0, s>>>(dmax, count, P->d_status);
-  return cudaGetLastError();
+  return launch_chained(k_dcode_check, 1, 256, 0, s, dmax, count, P->d_status);
 }
 
 Level make_level(int64_t n, int m, int R) {
@@ -286,9 +291,8 @@ static cudaError_t launch_stage1(const Level& lv, const Tin* a, const Tin* b, co
     auto k = k_stage1<Ar, Tin, Tred, R, K, W, decltype(vec)::value, kRef, decltype(rl)::value>;
     const cudaError_t e = set_smem(k, smem, done);
     if (e != cudaSuccess) return e;
-    k<<<grid, 32 * W, smem, s>>>(lv, a, b, c, d, B.red[0], B.red[1], B.red[2], B.red[3], B.ck[0],
-                                 B.ck[1], B.ck[2], status, rf, B.rl);
-    return cudaGetLastError();
+    return launch_chained(k, grid, 32 * W, smem, s, lv, a, b, c, d, B.red[0], B.red[1], B.red[2],
+                          B.red[3], B.ck[0], B.ck[1], B.ck[2], status, rf, B.rl);
   };
   const bool vec = vec16_ok<Tin>(lv.m, ptrs, kRef ? 6 : 4);
   if (rel) return vec ? go(std::true_type{}, std::true_type{})
@@ -311,8 +315,7 @@ static cudaError_t launch_stage3(const Level& lv, const Tin* a, const Tin* b, co
       constexpr size_t bytes = BackTile<Ar, Tin, R, kRef>::kBytes;
       const cudaError_t e = set_smem(k, bytes, done);
       if (e != cudaSuccess) return e;
-      k<<<(unsigned)warps, 32, bytes, s>>>(lv, B.red[4], x, status, B.rl, rf);
-      return cudaGetLastError();
+      return launch_chained(k, (unsigned)warps, 32, bytes, s, lv, B.red[4], x, status, B.rl, rf);
     };
     return vec16_ok<Tin>(lv.m, xp, 1) ? go(std::true_type{}) : go(std::false_type{});
   }
@@ -325,9 +328,8 @@ static cudaError_t launch_stage3(const Level& lv, const Tin* a, const Tin* b, co
     auto k = k_stage3<Ar, Tin, Tred, R, W, decltype(vec)::value, kRef>;
     const cudaError_t e = set_smem(k, smem, done);
     if (e != cudaSuccess) return e;
-    k<<<grid, 32 * W, smem, s>>>(lv, a, b, c, d, B.red[4], B.ck[0], B.ck[1], B.ck[2], x, status,
-                                 rf);
-    return cudaGetLastError();
+    return launch_chained(k, grid, 32 * W, smem, s, lv, a, b, c, d, B.red[4], B.ck[0], B.ck[1],
+                          B.ck[2], x, status, rf);
   };
   return vec16_ok<Tin>(lv.m, ptrs, 5) ? go(std::true_type{}) : go(std::false_type{});
 }
@@ -338,8 +340,8 @@ static cudaError_t run_levels(tps_plan_s* P, const std::vector<LevelPlan>& level
                               Tin* x, cudaStream_t s) {
   if (idx == levels.size()) {
     if (n <= 0) return cudaSuccess;
-    k_base<Ar, Tin, Tin><<<1, 32, 0, s>>>(n, a, b, c, d, x, nullptr, 0, P->d_status, nullptr);
-    return cudaGetLastError();
+    return launch_chained(k_base<Ar, Tin, Tin>, 1, 32, 0, s, n, a, b, c, d, x, nullptr, 0,
+                          P->d_status, nullptr);
   }
   bool used = false;
   cudaError_t eo = launch_onchip<Ar, Tin>(P, n, a, b, c, d, x, s, used, false);
@@ -498,10 +500,9 @@ cudaError_t base_solve(tps_plan_s* P, int64_t n, const void* a, const void* b, c
     using Ar = decltype(ar);
     using Tin = std::remove_pointer_t<decltype(tin)>;
     (void)tred;
-    k_base<Ar, Tin, Tin><<<1, 32, 0, s>>>(n, (const Tin*)a, (const Tin*)b, (const Tin*)c,
-                                          (const Tin*)d, (Tin*)x, bnd, nbnd, P->d_status,
-                                          level0_dmax(P));
-    return cudaGetLastError();
+    return launch_chained(k_base<Ar, Tin, Tin>, 1, 32, 0, s, n, (const Tin*)a, (const Tin*)b,
+                          (const Tin*)c, (const Tin*)d, (Tin*)x, bnd, nbnd, P->d_status,
+                          level0_dmax(P));
   });
 }
 

@@ -12,6 +12,24 @@
 
 namespace tps {
 
+// A kernel launch chained to the kernel before it in the stream (chain_wait):
+// only for kernels that call chain_wait before they touch memory.
+template <class... P, class... A>
+inline cudaError_t launch_chained(void (*k)(P...), unsigned grid, unsigned block, size_t smem,
+                                  cudaStream_t s, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k, static_cast<P>(args)...);
+}
+
 constexpr size_t kAlign = 256;
 inline size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
 
