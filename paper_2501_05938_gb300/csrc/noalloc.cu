@@ -28,7 +28,7 @@ constexpr int kM0 = 64;           // rows per block at the top level
 constexpr int kMr = 32;           // rows per block at the reduced levels
 constexpr int kMaxLevels = 8;
 constexpr size_t kScratchBytes = size_t(2) << 20;  // 2 MiB per GPU
-constexpr size_t kHeadOnchip = 128;  // the on-chip launch's status word and two counters
+constexpr size_t kHeadOnchip = 128;  // the on-chip solve's status word and three counters
 
 // The scratch array.  In host code `g_scratch` names a host-side shadow,
 // not device memory: its device address comes from cudaGetSymbolAddress.
@@ -180,7 +180,7 @@ extern "C" tps_status tps_solve_noalloc(int32_t dtype, int64_t n, const void* a,
   tps_status ts = scratch_address(&ws);
   if (ts != TPS_OK) return ts;
   cudaStream_t s = (cudaStream_t)stream;
-  // the whole system in one on-chip launch where it fits, which reports and
+  // the whole system on chip where it fits, which reports and
   // clears its own status word (its words of the header, kHeadOnchip, are
   // zero between launches; its exchange rows sit where the levels would go);
   // a test switch (TPS_TEST_NOALLOC_LEVELS=1) keeps the level-by-level route

@@ -1,8 +1,8 @@
 // Single-pass, on-chip partition solve for systems that fit in the GPU's
 // shared memory (the same method as the multi-launch path: Sec. 1 and
 // Sec. 2.2 of the paper, blocks eliminated onto their first and last rows,
-// a reduced interface system, per-block recovery), as ONE cooperative
-// launch that reads a, b, c, d from HBM once and writes x once.
+// a reduced interface system, per-block recovery), in one pass that reads a,
+// b, c, d from HBM once and writes x once.
 //
 //   CTA c owns the consecutive level-0 blocks [c*B, (c+1)*B) of mt rows (one
 //   block per thread; mt odd, so a thread's rows start on a different bank
@@ -14,8 +14,8 @@
 //   eliminated), in the warp by shuffles and then across the warps (every
 //   warp the same), until the CTA's own two equations are left; they go to
 //   global memory, divided by their diagonals.
-//   One grid barrier (bounded wait; a timeout sets ST_TIMEOUT and every CTA
-//   returns); a system that fits one CTA has none.
+//   One grid barrier (bounded wait, see OcMode); a system that fits one CTA
+//   has none.
 //   Stage 2: every warp solves for its CTA's two values by parallel cyclic
 //   reduction over the interface rows around them, which ends once their
 //   couplings are negligible; where they do not decay in time, the CTA
@@ -335,18 +335,36 @@ __device__ __forceinline__ void red_release_add(unsigned* p, unsigned v) {
   asm volatile("red.release.gpu.global.add.u32 [%0], %1;\n" ::"l"(p), "r"(v) : "memory");
 }
 
+// How a system of several CTAs is launched.  A cooperative launch keeps all
+// CTAs resident for the barrier, but cannot be chained (launch_chained), which
+// costs up to 3 us.  The other way is two chained launches: in kFirst a
+// CTA that has waited long enough for the others (they may not all be
+// resident: another stream's kernel holds SMs) leaves without its x; kFinish,
+// one CTA, returns at once if none did, else does those CTAs' rows again, by
+// when every interface equation is there.  No CTA waits for one that cannot
+// run.  (launch_onchip_raw chooses.)
+enum OcMode : int { kCoop = 0, kFirst = 1, kFinish = 2 };
+constexpr unsigned kOcPatience = 512;  // kFirst: polls of about 0.3 us
+
 // What the CTAs of one launch share.
 struct OcShared {
-  unsigned* bar;      // [0] arrivals at the barrier, [1] CTAs done; both zero
-                      // between launches (the last CTA clears them)
+  unsigned* bar;      // [0] arrivals at the barrier, [1] CTAs done, [2] CTAs that gave up;
+                      // all zero between solves (the last CTA clears them)
   unsigned arrivals;  // what the barrier waits for: G (more only to exercise the timeout)
   int* status;
-  int32_t* report;    // with own_status: the launch's tps_status, or null
-  int own_status;     // the status word belongs to this launch: cleared at its end
+  int32_t* report;    // with own_status: the solve's tps_status, or null
+  int own_status;     // the status word belongs to this solve: cleared at its end
+  int mode;           // OcMode
 };
 
+__device__ __forceinline__ void oc_report(const OcShared& sh) {
+  if (sh.own_status) {
+    const int w = atomicExch(sh.status, 0);
+    if (sh.report) *sh.report = status_code(w);
+  }
+}
 // The CTA is done with everything it shares: the last one clears the
-// barrier for the next launch and, with own_status, reports the status.
+// barrier for the next launch and, at the end of the solve, reports.
 __device__ __forceinline__ void oc_leave(const OcShared& sh, unsigned G) {
   __syncthreads();
   if (threadIdx.x != 0) return;
@@ -355,21 +373,18 @@ __device__ __forceinline__ void oc_leave(const OcShared& sh, unsigned G) {
   __threadfence();
   sh.bar[0] = 0u;
   sh.bar[1] = 0u;
-  if (sh.own_status) {
-    const int w = atomicExch(sh.status, 0);
-    if (sh.report) *sh.report = status_code(w);
-  }
+  if (sh.mode == kCoop) oc_report(sh);
 }
 
 // n rows, level-0 blocks of mt rows (p blocks, the last of length in
-// [2, mt + 1]), blockDim.x of them per CTA (64, 128 or 256), all CTAs
-// co-resident (cooperative launch).  xch: 3 x 2G values of T (the interface
-// equations), then 3 x G range codes.  vec16: a, b, c, d, x 16-byte aligned.
+// [2, mt + 1]), blockDim.x of them per CTA (64, 128 or 256), G CTAs.  xch: 3 x 2G
+// values of T (the interface equations), then 3 x G range codes and G flags
+// (1: the CTA gave up).  vec16: a, b, c, d, x 16-byte aligned.
 // codes: judge the system's range (level 0 of fp64 inputs in narrower
 // arithmetic).
 template <class Ar, class Tin>
 __global__ void __launch_bounds__(kOcThreads, 1)
-    k_onchip(int64_t n, int mt, int64_t p, const Tin* __restrict__ a,
+    k_onchip(int64_t n, int mt, int64_t p, int G, const Tin* __restrict__ a,
              const Tin* __restrict__ b, const Tin* __restrict__ c, const Tin* __restrict__ d,
              Tin* __restrict__ x, typename Ar::T* __restrict__ xch, OcShared sh, int vec16,
              int codes) {
@@ -384,203 +399,224 @@ __global__ void __launch_bounds__(kOcThreads, 1)
   for (int k = 0; k < 4; ++k) s0[k] = reinterpret_cast<Tin*>(smem_raw + k * Lay::kL0);
   EndEq<T>* const weq = reinterpret_cast<EndEq<T>*>(smem_raw + 4 * Lay::kL0);
   T* const pc = reinterpret_cast<T*>(smem_raw + 4 * Lay::kL0 + Lay::kEq);
-  const int G = (int)gridDim.x, cta = (int)blockIdx.x, tid = (int)threadIdx.x;
-  const int B = (int)blockDim.x, nw = B >> 5, lane = tid & 31;
-  const int64_t kb = (int64_t)cta * B;
-  const int64_t ke = kb + B < p ? kb + B : p;
-  const int nb = (int)(ke - kb);
-  const int64_t r0 = kb * mt;
-  const int64_t r1 = ke == p ? n : ke * mt;
-  const int rows = (int)(r1 - r0);
-
-  // ---- load the CTA's rows (r0 * sizeof(Tin) is a multiple of 16)
+  const int tid = (int)threadIdx.x, B = (int)blockDim.x, nw = B >> 5, lane = tid & 31;
+  const int M = 2 * G, last = 2 * nw - 1;
+  unsigned* const xcode = reinterpret_cast<unsigned*>(xch + 3 * M);
+  unsigned* const xgave = xcode + 3 * G;
   const Tin* const src[4] = {a, b, c, d};
   constexpr int V = 16 / (int)sizeof(Tin);
-  const int nv = vec16 ? rows / V : 0;
+  const bool fin = sh.mode == kFinish;
   chain_wait();
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    for (int i = tid; i < nv; i += B) cp_async<16>(s0[k] + i * V, src[k] + r0 + i * V);
-    for (int i = nv * V + tid; i < rows; i += B)
-      cp_async<sizeof(Tin)>(s0[k] + i, src[k] + r0 + i);
+  if (fin && ld_l2(sh.bar + 2) == 0u) {
+    if (tid == 0) oc_report(sh);
+    return;
   }
-  cp_async_commit();
-  if (tid < 6) code_s[tid / 3][tid % 3] = 0u;
-  cp_async_wait<0>();
-  __syncthreads();
-  // a[0] and c[n-1] are not part of the system
-  if (tid == 0 && cta == 0) s0[0][0] = Tin{};
-  if (tid == 0 && ke == p) s0[2][rows - 1] = Tin{};
-  __syncthreads();
-
-  // ---- Stage 1: one block per thread (past the last block: identity rows)
-  bool bad = false;
-  int L0len = 0;
-  RowChk chk;
-  EndEq<T> F{Ar::zero(), Ar::one(), Ar::zero(), Ar::zero()}, E = F;
-  if (tid < nb) {
-    const int64_t k = kb + tid;
-    L0len = k == p - 1 ? (int)(n - k * mt) : mt;
-    const AccL0<Ar, Tin> A{{s0[0], s0[1], s0[2], s0[3]}, (int)(k * mt - r0)};
-    oc_fwd<Ar>(A, L0len, F, E, bad, chk);
-  }
-  // the rows' range: a, c, d too large or b invalid; the codes of the
-  // system's range are collected per CTA and judged after the barrier
-  if (codes) {
-    const unsigned dc = __reduce_max_sync(0xffffffffu, chk.dcode());
-    const unsigned ec = __reduce_max_sync(0xffffffffu, chk.ecode);
-    const unsigned fc = __reduce_max_sync(0xffffffffu, chk.fcode());
-    if ((tid & 31) == 0) {
-      atomicMax(&code_s[0][0], dc);
-      atomicMax(&code_s[0][1], ec);
-      atomicMax(&code_s[0][2], fc);
-    }
-  }
-  if (chk.range_bad()) atomicOr(sh.status, ST_RANGE);
-  bad |= chk.b_bad();
-
-  // ---- the CTA's own two interface equations, divided by their diagonals:
-  // f = p - u l_prev - v l (lane 0),  l = p - u f - v f_next (lane 2 nw - 1)
-  OcMerge<Ar> mg;
-  mg.up(F, E, weq, nw, tid, bad);
-  const T rown = Ar::rcp(mg.own.b);
-  const T wn = Ar::mul(mg.own.w, rown), in = Ar::mul(mg.own.i, rown);
-  T pv = Ar::mul(mg.own.d, rown), uv = lane == 0 ? wn : in, vv = lane == 0 ? in : wn;
-  const int M = 2 * G, last = 2 * nw - 1;
-  if (lane == 0 || lane == last) bad |= Ar::bad_pivot(mg.own.b);
-  unsigned* const xcode = reinterpret_cast<unsigned*>(xch + 3 * M);
-  if (G > 1 && (tid == 0 || tid == last)) {
-    const int i = 2 * cta + (tid != 0);
-    xch[i] = pv;
-    xch[M + i] = uv;
-    xch[2 * M + i] = vv;
-  }
-  if (codes && G > 1 && tid == 0) {
-#pragma unroll
-    for (int q = 0; q < 3; ++q) xcode[q * G + cta] = code_s[0][q];
-  }
-  if (bad) atomicOr(sh.status, ST_BAD_PIVOT);
-  if (tid < 32) __syncwarp();  // lane `last`'s stores before lane 0's release
-
-  // ---- grid barrier (every CTA is resident: cooperative launch); warp 0
-  // wrote all that the other CTAs read
-  if (sh.arrivals > 1) {
-    if (tid == 0) {
-      red_release_add(sh.bar, 1u);
-      int ok = 1;
-      unsigned it = 0;
-      while (ld_acquire_u32(sh.bar) < sh.arrivals) {
-        if (++it > kOcSpinLimit) {
-          ok = 0;
-          atomicOr(sh.status, ST_TIMEOUT);
-          break;
-        }
-        if (it > 64) __nanosleep(100);
-      }
-      ok_s = ok;
-    }
-    __syncthreads();
-    if (!ok_s) {
-      oc_leave(sh, (unsigned)G);
-      return;
-    }
-  }
-
-  // ---- Stage 2.  Lane j takes interface row 2 cta - 15 + j, so the CTA's
-  // own rows are lanes 15 and 16 and four strides (1, 2, 4, 8) reach no
-  // further than the warp.  Every stride squares the couplings' order; between
-  // CTAs of many rows these have decayed already, and one or two strides
-  // leave the own rows with negligible ones: below 2^-103 of the diagonal
-  // (what split_row takes as 0) in single-precision parts, 2^-160 in fp64.
-  if (G > 1) {
-    const int i = 2 * cta - 15 + lane;
-    const bool in_sys = i >= 0 && i < M;
-    pv = in_sys ? ld_l2(xch + i) : Ar::zero();
-    uv = in_sys ? ld_l2(xch + M + i) : Ar::zero();
-    vv = in_sys ? ld_l2(xch + 2 * M + i) : Ar::zero();
-  } else {
-    const int src = lane == 16 ? last : 0;
-    const T p1 = shfl_v(pv, src), u1 = shfl_v(uv, src), v1 = shfl_v(vv, src);
-    const bool own = lane == 15 || lane == 16;
-    pv = own ? p1 : Ar::zero();
-    uv = own ? u1 : Ar::zero();
-    vv = own ? v1 : Ar::zero();
-  }
-  if (codes && cta == 0 && G > 1) {  // every CTA's codes are in
-    for (int i = tid; i < G; i += B) {
-#pragma unroll
-      for (int q = 0; q < 3; ++q) atomicMax(&code_s[1][q], ld_l2(xcode + q * G + i));
-    }
-  }
-  bool badr = false;
-  auto settled = [&]() {
-    const unsigned q = __ballot_sync(0xffffffffu, Ar::negligible(uv) && Ar::negligible(vv));
-    return ((q >> 15) & 3u) == 3u;
-  };
-  bool done = settled();
 #pragma unroll 1
-  for (int s = 1; s <= 8 && !done; s <<= 1) {
-    const T z = Ar::zero();
-    const bool lo = lane >= s, hi = lane + s < 32;
-    const T pm = shfl_v(pv, lane - s), um = shfl_v(uv, lane - s), vm = shfl_v(vv, lane - s);
-    const T pq = shfl_v(pv, lane + s), uq = shfl_v(uv, lane + s), vq = shfl_v(vv, lane + s);
-    oc_pcr<Ar>(pv, uv, vv, lo ? pm : z, lo ? um : z, lo ? vm : z, hi ? pq : z, hi ? uq : z,
-               hi ? vq : z, badr);
-    done = settled();
-  }
-  T fc = shfl_v(pv, 15), lc = shfl_v(pv, 16);
-  if (!done) {  // the same in every warp of the CTA: weakly coupled nowhere near
-    T* cur = pc;
-    T* nxt = pc + 3 * M;
-    for (int i = tid; i < 3 * M; i += B) cur[i] = ld_l2(xch + i);
-    __syncthreads();
-    bool stop = false;
-    for (int s = 1; s < M && !stop; s <<= 1) {
-      bool quiet = true;
-      for (int i = tid; i < M; i += B) {
-        const T z = Ar::zero();
-        const int im = i - s, iq = i + s;
-        const bool lo = im >= 0, hi = iq < M;
-        T pi = cur[i], ui = cur[M + i], vi = cur[2 * M + i];
-        oc_pcr<Ar>(pi, ui, vi, lo ? cur[im] : z, lo ? cur[M + im] : z, lo ? cur[2 * M + im] : z,
-                   hi ? cur[iq] : z, hi ? cur[M + iq] : z, hi ? cur[2 * M + iq] : z, badr);
-        nxt[i] = pi;
-        nxt[M + i] = ui;
-        nxt[2 * M + i] = vi;
-        quiet &= Ar::negligible(ui) && Ar::negligible(vi);
-      }
-      stop = __syncthreads_and(quiet);
-      T* const t = cur;
-      cur = nxt;
-      nxt = t;
+  for (int cta = fin ? 0 : (int)blockIdx.x; cta < (fin ? G : (int)blockIdx.x + 1); ++cta) {
+    if (fin && ld_l2(xgave + cta) == 0u) continue;
+    const int64_t kb = (int64_t)cta * B;
+    const int64_t ke = kb + B < p ? kb + B : p;
+    const int nb = (int)(ke - kb);
+    const int64_t r0 = kb * mt;
+    const int64_t r1 = ke == p ? n : ke * mt;
+    const int rows = (int)(r1 - r0);
+
+    // ---- load the CTA's rows (r0 * sizeof(Tin) is a multiple of 16)
+    const int nv = vec16 ? rows / V : 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      for (int i = tid; i < nv; i += B) cp_async<16>(s0[k] + i * V, src[k] + r0 + i * V);
+      for (int i = nv * V + tid; i < rows; i += B)
+        cp_async<sizeof(Tin)>(s0[k] + i, src[k] + r0 + i);
     }
-    fc = cur[2 * cta];
-    lc = cur[2 * cta + 1];
-  }
-  if (badr) atomicOr(sh.status, ST_BAD_PIVOT);
+    cp_async_commit();
+    if (tid < 6) code_s[tid / 3][tid % 3] = 0u;
+    cp_async_wait<0>();
+    __syncthreads();
+    // a[0] and c[n-1] are not part of the system
+    if (tid == 0 && cta == 0) s0[0][0] = Tin{};
+    if (tid == 0 && ke == p) s0[2][rows - 1] = Tin{};
+    __syncthreads();
 
-  // ---- Stage 3 down the merges, then the block
-  T f, l;
-  mg.down(lane == 0 ? fc : lc, nw, tid, f, l);
-  if (tid < nb) {
-    const int64_t k = kb + tid;
-    const AccL0<Ar, Tin> A{{s0[0], s0[1], s0[2], s0[3]}, (int)(k * mt - r0)};
-    oc_bwd<Ar>(A, L0len, f, l);
-  }
-  __syncthreads();
+    // ---- Stage 1: one block per thread (past the last block: identity rows)
+    bool bad = false;
+    int L0len = 0;
+    RowChk chk;
+    EndEq<T> F{Ar::zero(), Ar::one(), Ar::zero(), Ar::zero()}, E = F;
+    if (tid < nb) {
+      const int64_t k = kb + tid;
+      L0len = k == p - 1 ? (int)(n - k * mt) : mt;
+      const AccL0<Ar, Tin> A{{s0[0], s0[1], s0[2], s0[3]}, (int)(k * mt - r0)};
+      oc_fwd<Ar>(A, L0len, F, E, bad, chk);
+    }
+    // the rows' range: a, c, d too large or b invalid; the codes of the
+    // system's range are collected per CTA and judged after the barrier
+    if (codes) {
+      const unsigned dc = __reduce_max_sync(0xffffffffu, chk.dcode());
+      const unsigned ec = __reduce_max_sync(0xffffffffu, chk.ecode);
+      const unsigned fc = __reduce_max_sync(0xffffffffu, chk.fcode());
+      if ((tid & 31) == 0) {
+        atomicMax(&code_s[0][0], dc);
+        atomicMax(&code_s[0][1], ec);
+        atomicMax(&code_s[0][2], fc);
+      }
+    }
+    if (chk.range_bad()) atomicOr(sh.status, ST_RANGE);
+    bad |= chk.b_bad();
 
-  // ---- x out of the d slots
-  for (int i = tid; i < nv; i += B)
-    *reinterpret_cast<float4*>(x + r0 + i * V) = *reinterpret_cast<const float4*>(s0[3] + i * V);
-  for (int i = nv * V + tid; i < rows; i += B) x[r0 + i] = s0[3][i];
-  bool oob = false;
-  for (int i = tid; i < rows; i += B) oob |= Ar::out_bad(s0[3][i]);
-  if (codes && cta == 0 && tid == 0) {
-    const unsigned* q = code_s[G > 1 ? 1 : 0];
-    oob |= range_codes_bad(q[0], q[1], q[2]);
+    // ---- the CTA's own two interface equations, divided by their diagonals:
+    // f = p - u l_prev - v l (lane 0),  l = p - u f - v f_next (lane 2 nw - 1)
+    OcMerge<Ar> mg;
+    mg.up(F, E, weq, nw, tid, bad);
+    const T rown = Ar::rcp(mg.own.b);
+    const T wn = Ar::mul(mg.own.w, rown), in = Ar::mul(mg.own.i, rown);
+    T pv = Ar::mul(mg.own.d, rown), uv = lane == 0 ? wn : in, vv = lane == 0 ? in : wn;
+    if (lane == 0 || lane == last) bad |= Ar::bad_pivot(mg.own.b);
+    const bool publish = G > 1 && !fin;
+    if (publish && (tid == 0 || tid == last)) {
+      const int i = 2 * cta + (tid != 0);
+      xch[i] = pv;
+      xch[M + i] = uv;
+      xch[2 * M + i] = vv;
+    }
+    if (codes && publish && tid == 0) {
+#pragma unroll
+      for (int q = 0; q < 3; ++q) xcode[q * G + cta] = code_s[0][q];
+    }
+    if (bad) atomicOr(sh.status, ST_BAD_PIVOT);
+    if (tid < 32) __syncwarp();  // lane `last`'s stores before lane 0's release
+
+    // ---- grid barrier; warp 0 wrote all that the other CTAs read
+    if (sh.arrivals > 1 && !fin) {
+      if (tid == 0) {
+        red_release_add(sh.bar, 1u);
+        int ok = 1;
+        unsigned it = 0;
+        const unsigned limit = sh.mode == kFirst ? kOcPatience : kOcSpinLimit;
+        while (ld_acquire_u32(sh.bar) < sh.arrivals) {
+          if (++it > limit) {
+            ok = 0;
+            if (sh.mode == kFirst) atomicAdd(sh.bar + 2, 1u);
+            else atomicOr(sh.status, ST_TIMEOUT);
+            break;
+          }
+          if (sh.mode == kCoop && it > 64) __nanosleep(100);
+        }
+        xgave[cta] = ok ? 0u : 1u;
+        ok_s = ok;
+      }
+      __syncthreads();
+      if (!ok_s) {
+        oc_leave(sh, (unsigned)G);
+        return;
+      }
+    }
+
+    // ---- Stage 2.  Lane j takes interface row 2 cta - 15 + j, so the CTA's
+    // own rows are lanes 15 and 16 and four strides (1, 2, 4, 8) reach no
+    // further than the warp.  Every stride squares the couplings' order; between
+    // CTAs of many rows these have decayed already, and one or two strides
+    // leave the own rows with negligible ones: below 2^-103 of the diagonal
+    // (what split_row takes as 0) in single-precision parts, 2^-160 in fp64.
+    if (G > 1) {
+      const int i = 2 * cta - 15 + lane;
+      const bool in_sys = i >= 0 && i < M;
+      pv = in_sys ? ld_l2(xch + i) : Ar::zero();
+      uv = in_sys ? ld_l2(xch + M + i) : Ar::zero();
+      vv = in_sys ? ld_l2(xch + 2 * M + i) : Ar::zero();
+    } else {
+      const int src = lane == 16 ? last : 0;
+      const T p1 = shfl_v(pv, src), u1 = shfl_v(uv, src), v1 = shfl_v(vv, src);
+      const bool own = lane == 15 || lane == 16;
+      pv = own ? p1 : Ar::zero();
+      uv = own ? u1 : Ar::zero();
+      vv = own ? v1 : Ar::zero();
+    }
+    if (codes && cta == 0 && G > 1) {  // every CTA's codes are in
+      for (int i = tid; i < G; i += B) {
+#pragma unroll
+        for (int q = 0; q < 3; ++q) atomicMax(&code_s[1][q], ld_l2(xcode + q * G + i));
+      }
+    }
+    bool badr = false;
+    auto settled = [&]() {
+      const unsigned q = __ballot_sync(0xffffffffu, Ar::negligible(uv) && Ar::negligible(vv));
+      return ((q >> 15) & 3u) == 3u;
+    };
+    bool done = settled();
+#pragma unroll 1
+    for (int s = 1; s <= 8 && !done; s <<= 1) {
+      const T z = Ar::zero();
+      const bool lo = lane >= s, hi = lane + s < 32;
+      const T pm = shfl_v(pv, lane - s), um = shfl_v(uv, lane - s), vm = shfl_v(vv, lane - s);
+      const T pq = shfl_v(pv, lane + s), uq = shfl_v(uv, lane + s), vq = shfl_v(vv, lane + s);
+      oc_pcr<Ar>(pv, uv, vv, lo ? pm : z, lo ? um : z, lo ? vm : z, hi ? pq : z, hi ? uq : z,
+                 hi ? vq : z, badr);
+      done = settled();
+    }
+    T fc = shfl_v(pv, 15), lc = shfl_v(pv, 16);
+    if (!done) {  // the same in every warp of the CTA: weakly coupled nowhere near
+      T* cur = pc;
+      T* nxt = pc + 3 * M;
+      for (int i = tid; i < 3 * M; i += B) cur[i] = ld_l2(xch + i);
+      __syncthreads();
+      bool stop = false;
+      for (int s = 1; s < M && !stop; s <<= 1) {
+        bool quiet = true;
+        for (int i = tid; i < M; i += B) {
+          const T z = Ar::zero();
+          const int im = i - s, iq = i + s;
+          const bool lo = im >= 0, hi = iq < M;
+          T pi = cur[i], ui = cur[M + i], vi = cur[2 * M + i];
+          oc_pcr<Ar>(pi, ui, vi, lo ? cur[im] : z, lo ? cur[M + im] : z, lo ? cur[2 * M + im] : z,
+                     hi ? cur[iq] : z, hi ? cur[M + iq] : z, hi ? cur[2 * M + iq] : z, badr);
+          nxt[i] = pi;
+          nxt[M + i] = ui;
+          nxt[2 * M + i] = vi;
+          quiet &= Ar::negligible(ui) && Ar::negligible(vi);
+        }
+        stop = __syncthreads_and(quiet);
+        T* const t = cur;
+        cur = nxt;
+        nxt = t;
+      }
+      fc = cur[2 * cta];
+      lc = cur[2 * cta + 1];
+    }
+    if (badr) atomicOr(sh.status, ST_BAD_PIVOT);
+
+    // ---- Stage 3 down the merges, then the block
+    T f, l;
+    mg.down(lane == 0 ? fc : lc, nw, tid, f, l);
+    if (tid < nb) {
+      const int64_t k = kb + tid;
+      const AccL0<Ar, Tin> A{{s0[0], s0[1], s0[2], s0[3]}, (int)(k * mt - r0)};
+      oc_bwd<Ar>(A, L0len, f, l);
+    }
+    __syncthreads();
+
+    // ---- x out of the d slots
+    for (int i = tid; i < nv; i += B)
+      *reinterpret_cast<float4*>(x + r0 + i * V) = *reinterpret_cast<const float4*>(s0[3] + i * V);
+    for (int i = nv * V + tid; i < rows; i += B) x[r0 + i] = s0[3][i];
+    bool oob = false;
+    for (int i = tid; i < rows; i += B) oob |= Ar::out_bad(s0[3][i]);
+    if (codes && cta == 0 && tid == 0) {
+      const unsigned* q = code_s[G > 1 ? 1 : 0];
+      oob |= range_codes_bad(q[0], q[1], q[2]);
+    }
+    if (oob) atomicOr(sh.status, ST_RANGE);
+    if (fin) __syncthreads();  // the next CTA's rows take this one's place
   }
-  if (oob) atomicOr(sh.status, ST_RANGE);
-  if (sh.arrivals > 1 || sh.own_status) oc_leave(sh, (unsigned)G);
+  if (fin) {
+    if (tid == 0) {
+      __threadfence();
+      sh.bar[2] = 0u;
+      oc_report(sh);
+    }
+  } else if (sh.arrivals > 1 || sh.own_status) {
+    oc_leave(sh, (unsigned)G);
+  }
 }
 
 }  // namespace tps

@@ -93,12 +93,15 @@ static int oc_ctas_max() {
 }
 
 // Solve the system on chip if it fits (used = true), else leave it.  xch:
-// onchip_exchange_bytes() of device memory; bar: the launch's two counters,
-// zero between launches; report: see OcShared (own_status where given).
+// onchip_exchange_bytes() of device memory; bar: the solve's three counters,
+// zero between solves; extra_arrival:
+// 0, or to exercise the barrier one CTA more awaited than launched, in a
+// cooperative launch (1: it times out) or a chained one (2: every CTA gives
+// up and is done again); report: see OcShared (own_status where given).
 template <class Ar, class Tin>
 static cudaError_t launch_onchip_raw(int64_t n, const Tin* a, const Tin* b, const Tin* c,
                                      const Tin* d, Tin* x, void* xch, unsigned* bar,
-                                     int* status, bool extra_arrival, cudaStream_t s,
+                                     int* status, int extra_arrival, cudaStream_t s,
                                      bool& used, bool codes, bool own_status = false,
                                      int32_t* report = nullptr) {
   used = false;
@@ -107,27 +110,44 @@ static cudaError_t launch_onchip_raw(int64_t n, const Tin* a, const Tin* b, cons
   using T = typename Ar::T;
   const uintptr_t al = (uintptr_t)a | (uintptr_t)b | (uintptr_t)c | (uintptr_t)d | (uintptr_t)x;
   const int vec16 = (al % 16) == 0;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)g.G);
-  cfg.blockDim = dim3((unsigned)g.B);
-  cfg.dynamicSmemBytes = OcLayout<Ar, Tin>::kBytes;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeCooperative;
-  attr[0].val.cooperative = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  // one CTA has no barrier, so it need not be a cooperative launch, which
-  // cannot be chained
-  if (g.G == 1 && !extra_arrival) {
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
+  // Two chained launches or one cooperative one: the chained pair starts sooner
+  // but has a boundary more.  Measured back to back, us a solve, chained
+  // against cooperative: fp64 10007 rows 12.1 / 14.3 and 65536 14.7 / 16.4,
+  // double-float 800000 19.9 / 20.5, but fp32 1000003 12.7 / 12.3 and as
+  // Stage 2 of 256 fp32 systems 115.5 / 113.8 a batch: fp32 stays cooperative.
+  const bool coop = extra_arrival == 1 ||
+                    (std::is_same<Ar, ArF32>::value && g.G > 1 && extra_arrival == 0);
+  OcShared sh{bar, (unsigned)g.G + (extra_arrival ? 1u : 0u), status, report,
+              own_status ? 1 : 0, kFirst};
+  constexpr size_t smem = OcLayout<Ar, Tin>::kBytes;
+  cudaError_t e;
+  if (coop) {
+    sh.mode = kCoop;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)g.G);
+    cfg.blockDim = dim3((unsigned)g.B);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    e = cudaLaunchKernelEx(&cfg, k_onchip<Ar, Tin>, n, g.mt, g.p, g.G, a, b, c, d, x,
+                           reinterpret_cast<T*>(xch), sh, vec16, codes ? 1 : 0);
+  } else {
+    if (g.G == 1) sh.mode = kCoop;  // no barrier, nothing to finish
+    auto go = [&](int ctas) {
+      return launch_chained(k_onchip<Ar, Tin>, (unsigned)ctas, (unsigned)g.B, smem, s, n, g.mt,
+                            g.p, g.G, a, b, c, d, x, reinterpret_cast<T*>(xch), sh, vec16,
+                            codes ? 1 : 0);
+    };
+    e = go(g.G);
+    if (e == cudaSuccess && g.G > 1) {
+      sh.mode = kFinish;
+      e = go(1);
+    }
   }
-  const OcShared sh{bar, (unsigned)g.G + (extra_arrival ? 1u : 0u), status, report,
-                    own_status ? 1 : 0};
-  const cudaError_t e =
-      cudaLaunchKernelEx(&cfg, k_onchip<Ar, Tin>, n, g.mt, g.p, a, b, c, d, x,
-                         reinterpret_cast<T*>(xch), sh, vec16, codes ? 1 : 0);
   if (e == cudaSuccess) used = true;
   return e;
 }
@@ -140,7 +160,7 @@ static cudaError_t launch_onchip(tps_plan_s* P, int64_t n, const Tin* a, const T
   used = false;
   if (P->desc.flags & TPS_NO_ONCHIP) return cudaSuccess;
   if (P->desc.flags & TPS_EXTERNAL_WORKSPACE) {  // the caller may have used it in between
-    const cudaError_t e = cudaMemsetAsync(P->ws + 32, 0, 2 * sizeof(unsigned), s);
+    const cudaError_t e = cudaMemsetAsync(P->ws + 32, 0, 3 * sizeof(unsigned), s);
     if (e != cudaSuccess) return e;
   }
   return launch_onchip_raw<Ar, Tin>(n, a, b, c, d, x, P->ws + P->off_xch,
@@ -735,7 +755,7 @@ cudaError_t onchip_solve(int dtype, int64_t n, const void* a, const void* b, con
     using Tin = std::remove_pointer_t<decltype(tin)>;
     (void)tred;
     return launch_onchip_raw<Ar, Tin>(n, (const Tin*)a, (const Tin*)b, (const Tin*)c,
-                                      (const Tin*)d, (Tin*)x, xch, bar, status, false, s, used,
+                                      (const Tin*)d, (Tin*)x, xch, bar, status, 0, s, used,
                                       dtype == TPS_F64_DF, true, report);
   });
 }

@@ -251,7 +251,9 @@ tps_status tps_plan(const tps_plan_desc* desc, tps_plan_t* out) {
   P->off_levels = off_levels;
 
   if (const char* t = std::getenv("TPS_TEST_ONCHIP_TIMEOUT"))
-    P->test_barrier_extra = t[0] == '1';
+    P->test_barrier_extra = t[0] == '1' ? 1 : 0;
+  if (const char* t = std::getenv("TPS_TEST_ONCHIP_GIVE_UP"))
+    if (t[0] == '1') P->test_barrier_extra = 2;
   // test switch: the mixed solve's corrections as three separate passes
   // on every route (to compare them with the fused step)
   if (const char* t = std::getenv("TPS_TEST_UNFUSED_REFINE"))

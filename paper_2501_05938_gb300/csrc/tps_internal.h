@@ -131,10 +131,11 @@ struct tps_plan_s {
   int32_t last_onchip = 0;
   int32_t graph_onchip = 0;  // last_onchip and last_levels of the captured Stage 2
   int32_t graph_levels = 0;
-  // test hook (TPS_TEST_ONCHIP_TIMEOUT=1 at plan creation): the on-chip
-  // solve's grid barrier waits for one CTA more than it launches, so the
-  // bounded wait runs out and the solve reports TPS_ERR_TIMEOUT
-  bool test_barrier_extra = false;
+  // test hooks at plan creation: the on-chip solve's grid barrier waits for
+  // one CTA more than it launches, so the bounded wait runs out and the solve
+  // reports TPS_ERR_TIMEOUT (1, TPS_TEST_ONCHIP_TIMEOUT=1) or does every CTA
+  // again (2, TPS_TEST_ONCHIP_GIVE_UP=1)
+  int test_barrier_extra = 0;
   bool test_unfused_refine = false;  // TPS_TEST_UNFUSED_REFINE=1 at plan time
   int32_t last_refine_fused = 0;     // the last mixed solve used refine_step
   // batched work list (device) and its capacity in entries
@@ -183,8 +184,8 @@ cudaError_t refine_step(tps_plan_s* P, const std::vector<LevelPlan>& levels, con
 size_t onchip_exchange_bytes();
 // The single-launch on-chip solve of one system if it fits on this device
 // (used = true), else nothing.  xch: onchip_exchange_bytes() of device
-// memory; bar: two device counters, status: a status word, all three zero
-// between launches; report: the solve's tps_status, or null.
+// memory; bar: three device counters, status: a status word, all zero
+// between solves; report: the solve's tps_status, or null.
 cudaError_t onchip_solve(int dtype, int64_t n, const void* a, const void* b, const void* c,
                          const void* d, void* x, void* xch, unsigned* bar, int* status,
                          int32_t* report, cudaStream_t s, bool& used);

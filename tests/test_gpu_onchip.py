@@ -157,3 +157,23 @@ def test_couplings_that_do_not_decay(dtype, ulp, n):
     assert info["status"] == 0 and info["onchip"] == 1, info
     ref = oracle.thomas(*(np.asarray(s[k], dtype=np.float64) for k in "abcd"))
     assert oracle.rel_forward_error(x, ref) <= 16 * (4.0 / delta) * ulp
+
+
+@pytest.mark.parametrize("dtype", ["f64", "f64_df", "f32"])
+@pytest.mark.parametrize("n", [6000, 100003, 800001])
+def test_ctas_that_gave_up_are_done_again(dtype, n, monkeypatch):
+    """The barrier waits for one CTA more than there are, so every CTA gives up
+    and the second launch does it again; a solve after it, undisturbed, finds
+    the counters as they should be."""
+    monkeypatch.setenv("TPS_TEST_ONCHIP_GIVE_UP", "1")
+    plan = binding.Plan(n, dtype=dtype)
+    monkeypatch.delenv("TPS_TEST_ONCHIP_GIVE_UP")
+    s = synth.system(33 + n, n)
+    tdt = torch.float64
+    if dtype == "f32":
+        s, tdt = synth.to_f32(s), torch.float32
+    x0, info0 = solve(binding.Plan(n, dtype=dtype), s, tdt)
+    for _ in range(2):
+        x, info = solve(plan, s, tdt)
+        assert info["status"] == 0 and info["onchip"] == 1, info
+        assert np.array_equal(x, x0)
