@@ -99,11 +99,17 @@ def _ptr(t):
 
 
 def _stream(stream):
+    """The raw handle of `stream`, or of the current stream.  (The raw getters
+    that torch's own stream object is made from: building that object takes
+    longer than the launch of a small solve.)"""
     import torch
 
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    try:
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    except AttributeError:  # a torch without them, or without CUDA
+        return torch.cuda.current_stream().cuda_stream
 
 
 class Plan:
@@ -116,6 +122,7 @@ class Plan:
                              streams=int(streams), max_iters=int(max_iters), chunk=int(chunk),
                              tol=float(tol), flags=int(flags), reserved=0)
         self.dtype = dtype
+        self._want = None  # the arrays' torch dtype
         self._h = ctypes.c_void_p()
         check(lib().tps_plan(ctypes.byref(self.desc), ctypes.byref(self._h)), "tps_plan")
 
@@ -147,9 +154,11 @@ class Plan:
         """a, b, c, d, x: contiguous tensors of the plan's I/O type (float32
         for "f32", float64 otherwise), n elements each (the library checks
         where they live)."""
-        import torch
+        want = self._want
+        if want is None:
+            import torch
 
-        want = torch.float32 if self.dtype == "f32" else torch.float64
+            want = self._want = torch.float32 if self.dtype == "f32" else torch.float64
         for t in ts:
             if t.dtype != want or not t.is_contiguous() or t.numel() != n:
                 raise TpsError(1, f"arrays must be contiguous {want} tensors of {n} elements")
@@ -170,8 +179,10 @@ class Plan:
         """Device-resident solve; a..x are CUDA tensors of n elements."""
         n = b.numel()
         self._arrays(n, a, b, c, d, x)
-        check(lib().tps_solve(self._h, n, _ptr(a), _ptr(b), _ptr(c), _ptr(d), _ptr(x),
-                              _stream(stream)), "tps_solve")
+        st = lib().tps_solve(self._h, n, a.data_ptr(), b.data_ptr(), c.data_ptr(), d.data_ptr(),
+                             x.data_ptr(), _stream(stream))
+        if st:
+            raise TpsError(st, "tps_solve")
         return x
 
     def solve_batched(self, offsets, a, b, c, d, x, host_offsets=None, stream=None):
