@@ -160,18 +160,24 @@ __device__ __forceinline__ void codes_raise_warp(unsigned* dmax, int64_t sys, bo
 }
 
 // After every row of the level-0 system has been loaded: flag ST_RANGE for
-// each system whose codes are out of range (range_codes_bad), and clear the
-// codes for the next solve.  One CTA.
-static __global__ void __launch_bounds__(256)
-    k_dcode_check(unsigned* __restrict__ dmax, int64_t count, int* __restrict__ status) {
-  chain_wait();
+// each system i, i + step, .. < count whose codes are out of range
+// (range_codes_bad), and clear the codes for the next solve.
+__device__ __forceinline__ void judge_codes(unsigned* dmax, int64_t i, int64_t step,
+                                            int64_t count, int* status) {
   bool bad = false;
-  for (int64_t i = threadIdx.x; i < count; i += blockDim.x) {
+  for (; i < count; i += step) {
     unsigned* p = dmax + kCodes * i;
     bad |= range_codes_bad(p[0], p[1], p[2]);
     p[0] = p[1] = p[2] = 0u;
   }
   if (bad) atomicOr(status, ST_RANGE);
+}
+// The same as a launch of its own, one CTA (k_back does it where it follows
+// in the same stream: 2 to 3 us less a solve).
+static __global__ void __launch_bounds__(256)
+    k_dcode_check(unsigned* __restrict__ dmax, int64_t count, int* __restrict__ status) {
+  chain_wait();
+  judge_codes(dmax, threadIdx.x, blockDim.x, count, status);
 }
 
 // ------------------------------------------------------------------ cp.async
@@ -1031,6 +1037,7 @@ __global__ void __launch_bounds__(W * 32)
 // out; fp32 12) where k_stage3 moves 40.  Bound by those bytes, so what
 // counts is how many are on their way: a chunk's relations are one contiguous
 // piece of memory, copied with cp.async kBackStages - 1 chunks ahead.
+// Where lv.dmax is given, the range codes Stage 1 raised are judged on the way.
 // kRef: the result is added to x in place and the maxima go to rf.max2.
 #ifndef TPS_BACK_STAGES
 #define TPS_BACK_STAGES 3
@@ -1173,6 +1180,9 @@ __global__ void __launch_bounds__(32)
     st = st == kBackStages - 1 ? 0 : st + 1;
   }
   if (oob) atomicOr(status, ST_RANGE);
+  if (lv.dmax)
+    judge_codes(lv.dmax, (int64_t)blockIdx.x * 32 + lane, (int64_t)gridDim.x * 32, lv.nbnd + 1,
+                status);
   if constexpr (kRef) {
     for (int o = 16; o > 0; o >>= 1) {
       mdel = max(mdel, __shfl_xor_sync(0xffffffffu, mdel, o));

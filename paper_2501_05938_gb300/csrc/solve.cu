@@ -456,7 +456,7 @@ cudaError_t stage1_range(tps_plan_s* P, const LevelPlan& L, int64_t kb, int64_t 
 
 cudaError_t stage3_range(tps_plan_s* P, const LevelPlan& L, int64_t kb, int64_t ke,
                          const void* a, const void* b, const void* c, const void* d, void* x,
-                         cudaStream_t s) {
+                         cudaStream_t s, bool judge) {
   return dispatch(P->desc.dtype, [&](auto ar, auto* tin, auto* tred) -> cudaError_t {
     using Ar = decltype(ar);
     using Tin = std::remove_pointer_t<decltype(tin)>;
@@ -465,6 +465,7 @@ cudaError_t stage3_range(tps_plan_s* P, const LevelPlan& L, int64_t kb, int64_t 
     Level lv = L.lv;
     lv.k_begin = kb;
     lv.k_end = ke;
+    lv.dmax = judge ? level0_dmax(P) : nullptr;
     return launch_stage3<Ar, Tin, Tred, R>(lv, (const Tin*)a, (const Tin*)b, (const Tin*)c,
                                            (const Tin*)d, LevelBufs<Tred>(P, L), (Tin*)x,
                                            P->d_status, s);
@@ -658,7 +659,8 @@ static tps_status run_solve_direct(tps_plan_s* P, int64_t n, const void* a, cons
     if (e == cudaSuccess && ev) e = cudaEventRecord(ev[2], s);
   } else {
     if (e == cudaSuccess) e = stage1_range(P, lv[0], 0, lv[0].lv.p, a, b, c, d, s);
-    if (e == cudaSuccess) e = dcode_check(P, nbnd + 1, s);
+    const bool judge = lv[0].rel;  // k_back judges the range codes
+    if (e == cudaSuccess && !judge) e = dcode_check(P, nbnd + 1, s);
     if (e == cudaSuccess && ev) e = cudaEventRecord(ev[1], s);
     // with stage events (TPS_TRACE) TPS_GRAPH captures Stage 2 alone; without
     // them the whole solve is one graph already (run_solve_graph)
@@ -666,7 +668,7 @@ static tps_status run_solve_direct(tps_plan_s* P, int64_t n, const void* a, cons
       e = ((P->desc.flags & TPS_GRAPH) && ev) ? reduced_solve_graph(P, lv, s)
                                               : reduced_solve(P, lv, s);
     if (e == cudaSuccess && ev) e = cudaEventRecord(ev[2], s);
-    if (e == cudaSuccess) e = stage3_range(P, lv[0], 0, lv[0].lv.p, a, b, c, d, x, s);
+    if (e == cudaSuccess) e = stage3_range(P, lv[0], 0, lv[0].lv.p, a, b, c, d, x, s, judge);
   }
   if (e == cudaSuccess && ev) e = cudaEventRecord(ev[3], s);
   return e == cudaSuccess ? TPS_OK : TPS_ERR_CUDA;

@@ -163,14 +163,15 @@ tps_status run_solve(tps_plan_s* P, int64_t n, const void* a, const void* b, con
                      cudaEvent_t* ev, const int64_t* bnd = nullptr, int64_t nbnd = 0);
 
 // Level-0 pieces of the solve for the chunked host pipeline: Stage 1 and
-// Stage 3 on blocks [kb, ke), Stage 2 on the whole reduced system, and the
+// Stage 3 on blocks [kb, ke) (judge: k_back also judges the range codes, as
+// dcode_check does), Stage 2 on the whole reduced system, and the
 // one-warp solve for n <= kBaseMax.
 cudaError_t stage1_range(tps_plan_s* P, const LevelPlan& L, int64_t kb, int64_t ke,
                          const void* a, const void* b, const void* c, const void* d,
                          cudaStream_t s);
 cudaError_t stage3_range(tps_plan_s* P, const LevelPlan& L, int64_t kb, int64_t ke,
                          const void* a, const void* b, const void* c, const void* d, void* x,
-                         cudaStream_t s);
+                         cudaStream_t s, bool judge = false);
 cudaError_t reduced_solve(tps_plan_s* P, const std::vector<LevelPlan>& levels, cudaStream_t s);
 // One correction step of the mixed solve fused into level 0's sweeps
 // (levels non-empty): r = d - A x (fp64) formed in Stage 1, the fp32 solve
