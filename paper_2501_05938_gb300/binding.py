@@ -122,7 +122,6 @@ class Plan:
                              streams=int(streams), max_iters=int(max_iters), chunk=int(chunk),
                              tol=float(tol), flags=int(flags), reserved=0)
         self.dtype = dtype
-        self._want = None  # the arrays' torch dtype
         self._h = ctypes.c_void_p()
         check(lib().tps_plan(ctypes.byref(self.desc), ctypes.byref(self._h)), "tps_plan")
 
@@ -154,11 +153,9 @@ class Plan:
         """a, b, c, d, x: contiguous tensors of the plan's I/O type (float32
         for "f32", float64 otherwise), n elements each (the library checks
         where they live)."""
-        want = self._want
-        if want is None:
-            import torch
+        import torch
 
-            want = self._want = torch.float32 if self.dtype == "f32" else torch.float64
+        want = torch.float32 if self.dtype == "f32" else torch.float64
         for t in ts:
             if t.dtype != want or not t.is_contiguous() or t.numel() != n:
                 raise TpsError(1, f"arrays must be contiguous {want} tensors of {n} elements")
