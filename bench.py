@@ -27,7 +27,7 @@ Stage 2, Stage 3).
   batched  4096 packed systems, n_i log-uniform in [2^8, 2^20], each solve
            one graph launch (--no-extra skips this and the next)
   mixed    the refinement workload (b = 1.01 (|a| + |c|)) in every arithmetic
-  midsize_f64_df  n = 65536 and 800000: the single-launch on-chip solve
+  midsize_f64_df  n = 65536 and 800000: the on-chip solve
            against the level-by-level route (L2-warm)
   truncated_f64_df  the headline system by truncated decoupling (windows with
            halos, an approximation with a per-window error bound), one pass
@@ -573,7 +573,7 @@ def extra_workloads(binding, synth, world, rank, stream, a):
             us = max_over_ranks(e0.elapsed_time(e1) / steps, world) * 1e3
             q = plan.query()
             err = ((x - g["x_true"]).abs().max() / g["x_true"].abs().max()).item()
-            row[name] = {"us_per_solve": us, "value": world * n / (us * 1e-6), "launches": 2 * q["levels"] + 1,
+            row[name] = {"us_per_solve": us, "value": world * n / (us * 1e-6), "launches": 2 * q["levels"] + (2 if q["onchip"] else 1),
                          "onchip": q["onchip"], "rel_fwd_vs_x_true": err}
         row["speedup"] = row["levels"]["us_per_solve"] / row["onchip"]["us_per_solve"]
         mid[str(n)] = row
@@ -744,7 +744,7 @@ def main():
     # (the committed ncu count per row) over its event time, against this
     # GPU's measured fp64 FMA rate
     s1p = infop["stage_ms"][0]
-    f64t = fp64_table().get(f"k_stage1_f64_m{infop['m']}")
+    f64t = fp64_table().get(f"k_stage1_f64_m{infop['m']}", fp64_table().get("k_stage1_f64"))
     plain_roof = {"bound": "fp64", "kernel": "k_stage1", "peak": fp64_peak / 1e9,
                   "unit": "G fp64-pipe thread-inst/s",
                   "peak_kind": "measured: the fastest of fp64 fma / mul / add chains "
@@ -756,17 +756,20 @@ def main():
     plain_roof["frac"] = (plain_roof["achieved"] / plain_roof["peak"]
                           if plain_roof["achieved"] else None)
     plain_roof["frac_step_hbm"] = 40 * n / (msp * 1e-3) / 1e9 / hbm_peak
-    dominant = "k_stage1" if s1 >= s3 else "k_stage3"
+    # Stage 1 reads a, b, c, d and writes a relation a row (32 + 16 bytes), Stage 3
+    # reads it and writes x (16 + 8); above 2^30 rows, from checkpoints, 32 and 40
+    rel = n <= 1 << 30
+    dominant = "k_stage1" if s1 >= s3 else ("k_back" if rel else "k_stage3")
     dom_ms = max(s1, s3)
-    alg_bytes = (32 if dominant == "k_stage1" else 40) * n
+    alg_bytes = {"k_stage1": 48 if rel else 32, "k_back": 24, "k_stage3": 40}[dominant] * n
     achieved = alg_bytes / (dom_ms * 1e-3) / 1e9
     tt = traffic_table()
     traffic = tt.get(f"{dominant}_f64_df_m{info['m']}", tt.get(f"{dominant}_f64_df"))
     kernel_hash = kernel_source_hash()
     levels = info["levels"]
-    # Stage 1 and Stage 3 per level, the base solve, and the range-code check
-    # after level 0's Stage 1 (double-float only)
-    launches_per_step = 2 * levels + 2
+    # Stage 1 and Stage 3 per level and the on-chip solve's two launches (above
+    # 2^30 rows the range-code check besides)
+    launches_per_step = 2 * levels + (2 if rel else 3)
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": a.steps,
         "warmup": a.warmup, "ms_per_step": ms, "higher_is_better": True, "scaling": "weak",

@@ -98,7 +98,7 @@ typedef enum {
 #define TPS_GRAPH 16u             /* replay the solve as one CUDA graph launch    */
 #define TPS_ZERO_COPY 32u         /* host residency: kernels, not copy engines,   */
                                   /* move host data (see tps_solve_host_async)    */
-#define TPS_NO_ONCHIP 64u         /* never use the single-launch on-chip solve    */
+#define TPS_NO_ONCHIP 64u         /* never use the on-chip solve                  */
 #define TPS_TRUNCATE 128u         /* approximate windowed solve (see tps_solve)   */
 #define TPS_HOST_OVERLAP 256u     /* host residency: a second buffer set so that  */
                                   /* tps_solve_host_many_async overlaps systems   */
@@ -187,24 +187,28 @@ tps_status tps_set_workspace(tps_plan_t plan, void* dev_ptr, size_t bytes);
  *
  * A system that fits in the GPU's shared memory (up to ~0.89 M rows in
  * fp64 and double-float, ~1.8 M in fp32 on 152 SMs; not for packed batches)
- * is solved by a single cooperative launch that reads a, b, c, d once and
- * writes x once: each CTA eliminates its rows on chip, one grid barrier,
- * every CTA solves the small system of CTA interface rows, and recovers its
- * rows on chip.  The reduced system of a larger solve takes the same path
+ * is solved in one pass that reads a, b, c, d once and writes x once: each
+ * CTA eliminates its rows on chip, one grid barrier, every CTA solves for
+ * its own interface rows, and recovers its rows on chip.  The reduced system of a larger solve takes the same path
  * once it fits.  TPS_NO_ONCHIP keeps every level on separate launches.
- * The grid barrier waits a bounded time: if the launch's CTAs cannot all
- * become resident (another such launch from another stream, or other
- * long-running work holding the SMs), the wait ends, the solve reports
- * TPS_ERR_TIMEOUT through tps_plan_query and the context stays usable; run
- * on-chip solves of different streams one after the other, or use
- * TPS_NO_ONCHIP for plans that run concurrently.
+ * The grid barrier waits a bounded time for CTAs that are not resident
+ * (another such solve on another stream, or other long-running work holding
+ * the SMs).  In fp64 and double-float a second launch then does the rows of
+ * the CTAs that gave up.  In fp32 the launch is cooperative, so the CTAs are
+ * resident together; should the wait end all the same, the solve reports
+ * TPS_ERR_TIMEOUT through tps_plan_query and the context stays usable.
+ *
+ * Larger systems run level by level.  Up to 2^30 rows the workspace holds a
+ * relation per row (24 bytes, fp32 12), from which Stage 3 recovers x without
+ * reading a, b, c, d again; for more rows, or where tps_plan cannot allocate
+ * that much, it repeats the elimination from checkpoints (1.2 bytes a row).
  *
  * TPS_MIXED_F32_F64: x0 from an fp32 elimination of the fp64 inputs, then
  * corrections until ||delta||/||x|| <= tol or max_iters.  Where the system
  * is solved level by level, each correction is one fused pass of the
  * partition method: Stage 1 forms r = d - A x in fp64 from the rows and the
- * current x (writing r to the workspace), Stage 3 adds the fp32 solution of
- * A delta = r to x in place (tps_info.refine_fused = 1); the single-launch
+ * current x, Stage 3 adds the fp32 solution of
+ * A delta = r to x in place (tps_info.refine_fused = 1); the
  * on-chip route keeps a separate residual pass, solve and update pass.
  *
  * TPS_TRUNCATE (device plans, fp64 / double-float / fp32; not the paper's
@@ -316,7 +320,7 @@ tps_status tps_solve_host_many_async(tps_plan_t plan, int64_t count, int64_t n,
  *               the solve has run (NULL: not reported)
  *   stream      cudaStream_t as void*
  * A system that fits in shared memory (every accepted size on a 152-SM
- * GB300) is solved by the single-launch on-chip solve (see tps_solve);
+ * GB300) is solved by the on-chip solve (see tps_solve);
  * otherwise fixed parameters m = 64 at the top level, 32 below.  The first
  * call on a device looks up the scratch array's device address
  * (cudaGetSymbolAddress) with that device current.  Every call overwrites

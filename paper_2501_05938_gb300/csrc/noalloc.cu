@@ -5,9 +5,8 @@
 // where a cudaMalloc (which may synchronise the device) is not acceptable.
 // Instead of a plan and its workspace, this entry point keeps
 // its scratch (the reduced systems, the Stage-1 checkpoints and a status
-// word; or, when the system fits on chip and is solved by one cooperative
-// launch, that launch's barrier counter and exchange rows) in one
-// fixed-size array in device global memory, declared at file scope below.  Every GPU that loads the library holds that array
+// word; or, when the system fits on chip, that solve's counters and
+// exchange rows) in one fixed-size array in device global memory, declared at file scope below.  Every GPU that loads the library holds that array
 // (kScratchBytes) until the process exits.  All calls share it, and it keeps
 // whatever the last call left there; so two calls whose work overlaps on
 // the GPU (different streams, or different host threads) race on it and
@@ -147,8 +146,8 @@ cudaError_t run(unsigned char* ws, const Layout& L, int idx, int64_t n, const Ti
 // Translate the status bits into a tps_status for the caller's output.
 __global__ void k_report(const int* st, int32_t* out) { *out = status_code(*st); }
 
-// A cooperative launch the device refuses for its size or resources (fewer
-// SMs than the cached occupancy assumed, e.g. under an SM partition):
+// A cooperative launch (fp32) the device refuses for its size or resources
+// (fewer SMs than the cached occupancy assumed, e.g. under an SM partition):
 // the level-by-level route serves instead.
 bool launch_refused(cudaError_t e) {
   return e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorLaunchOutOfResources ||
@@ -182,7 +181,7 @@ extern "C" tps_status tps_solve_noalloc(int32_t dtype, int64_t n, const void* a,
   cudaStream_t s = (cudaStream_t)stream;
   // the whole system on chip where it fits, which reports and
   // clears its own status word (its words of the header, kHeadOnchip, are
-  // zero between launches; its exchange rows sit where the levels would go);
+  // zero between solves; its exchange rows sit where the levels would go);
   // a test switch (TPS_TEST_NOALLOC_LEVELS=1) keeps the level-by-level route
   bool onchip = false;
   const char* lvl = std::getenv("TPS_TEST_NOALLOC_LEVELS");

@@ -33,14 +33,23 @@
 // (f_k, l_k, f_{k+1}).  The first reduced equation needs the first interior
 // unknown as a function of f_k and l_k; instead of a second, bottom-up
 // sweep, the sweep carries x_1 = P - Q f - S x_{j+1} along, which costs four
-// multiply-adds per row and no extra reciprocal.  At every chunk boundary
-// the normalised relation x_j = (g_j - alpha_j f - c_j x_{j+1}) / beta_j is
-// written out as a checkpoint (c/beta, g/beta, alpha/beta).
+// multiply-adds per row and no extra reciprocal.
 //
-// Stage 3 walks each block's chunks bottom-up.  A chunk restarts the forward
-// elimination from its checkpoint (with f now known), keeps the R pivots and
-// right-hand sides in registers, and back-substitutes from the x of the row
-// below it (l_k for the last chunk).  The chunk's x goes back through the
+// Stage 3, the ordinary way (kRel, k_back): Stage 1 writes the normalised
+// relation x_j = g_j - alpha_j f - c_j x_{j+1} of every interior row, lane by
+// lane as it makes them, and Stage 3 back-substitutes from these.  Terms in f
+// and the chain for x_1 are left out once they have decayed below rounding.
+// Both sweeps are bound by memory: 49 and 25 bytes a row, at n = 2^25 in
+// double-float 260 and 131 us, 94% of the copy rate (k_stage1 with
+// checkpoints 215 us, k_stage3 218 us).  Native fp64 Stage 1 is bound by the
+// fp64 pipe: 480 us (k_stage3's half of that work is gone: 490 -> 129 us).
+//
+// Without the workspace that takes (24 bytes a row), Stage 1 writes the
+// relation only at every chunk boundary, as a checkpoint, and k_stage3 walks
+// each block's chunks bottom-up: a chunk restarts the forward elimination
+// from its checkpoint (with f now known), keeps the R pivots and right-hand
+// sides in registers, and back-substitutes from the x of the row below it
+// (l_k for the last chunk).  The chunk's x goes back through the
 // shared-memory slots and out with the same coalesced piece mapping.
 #pragma once
 #include <cuda_runtime.h>
@@ -448,6 +457,10 @@ __device__ __forceinline__ bool is_zero(double v) {
 #ifndef TPS_STAGE1_STAGES
 #define TPS_STAGE1_STAGES 2
 #endif
+// kRel compiles its row body twice (with and without the chain), so it is
+// unrolled by pairs of 16-byte row groups only: at n = 2^25 in double-float the
+// whole chunk unrolled takes 384 us (instruction fetch), four groups 308, two
+// 260, one 268.
 #ifndef TPS_REL_UNROLL
 #define TPS_REL_UNROLL 2
 #endif
@@ -559,7 +572,7 @@ __global__ void __launch_bounds__(W * 32)
     g = Ar::sub_mul(dv, ratio, g);
     if constexpr (!kRel || decltype(kChain)::value) al = Ar::mul_neg_nn(ratio, al);
     bad |= Ar::bad_pivot(beta);
-    const T rbeta = Ar::rcp_bulk(beta);
+    const T rbeta = Ar::rcp(beta);
     if constexpr (kRel) {
       T gp;
       if constexpr (sizeof(Tin) == 4) {  // bound by memory: round the quotients once
@@ -923,7 +936,7 @@ __global__ void __launch_bounds__(W * 32)
           Ar::template row<false>(xa.v[v], xb.v[v], xc.v[v], xd.v[v], av, bv, cv, dv, nochk);
           const T beta = Ar::sub_mul_dom(bv, av, gp);
           bad |= Ar::bad_pivot(beta);
-          const T rbeta = Ar::rcp_bulk(beta);
+          const T rbeta = Ar::rcp(beta);
           zp = Ar::mul_nn(Ar::sub_mul(dv, av, zp), rbeta);
           gp = Ar::mul_nn(cv, rbeta);
           Z[rr] = zp;
@@ -977,7 +990,7 @@ __global__ void __launch_bounds__(W * 32)
                                   t[3 * TL::kArr + r], av, bv, cv, dv, nochk);
           const T beta = Ar::sub_mul_dom(bv, av, gp);
           bad |= Ar::bad_pivot(beta);
-          const T rbeta = Ar::rcp_bulk(beta);
+          const T rbeta = Ar::rcp(beta);
           zp = Ar::mul_nn(Ar::sub_mul(dv, av, zp), rbeta);
           gp = Ar::mul_nn(cv, rbeta);
           zs[r] = zp;

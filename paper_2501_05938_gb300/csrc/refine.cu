@@ -12,12 +12,13 @@
 // iteration.
 //
 // Where the system is solved level by level (every size but those the
-// single-launch on-chip solve takes), a correction is one pass of the
-// partition method over the rows (refine_step): Stage 1 forms the residual
-// from the rows and x as it streams them and writes it out, Stage 3 reads
-// the residual back as its right-hand side and adds its result to x.  Per
-// row that moves a, b, c, d, x in and r out, then a, b, c, r, x in and x
-// out: 96 bytes against 144 for a residual pass, a solve and an update pass.
+// on-chip solve takes), a correction is one pass of the partition method over
+// the rows (refine_step): Stage 1 forms the residual from the rows and x as
+// it streams them, and its fp32 relations go out; Stage 3 adds its result to
+// x.  Per row that moves a, b, c, d, x in and a relation out, then the
+// relation and x in and x out: 72 bytes against 128 for a residual pass, a
+// solve and an update pass.  (From checkpoints: r out, and a, b, c, r in
+// again, 96 bytes.)
 // The on-chip route keeps the three separate passes below.
 #include <cuda_runtime.h>
 

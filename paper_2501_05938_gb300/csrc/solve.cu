@@ -1,6 +1,6 @@
 // Recursive device-resident partition solve: Stage 1 on the input, the same
 // method on the reduced interface system (Stage 2) until it fits one warp
-// or the GPU's shared memory (the single-launch on-chip solve), then Stage 3
+// or the GPU's shared memory (the on-chip solve), then Stage 3
 // back up the levels.
 #include <cuda_runtime.h>
 
