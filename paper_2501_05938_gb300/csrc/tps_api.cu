@@ -74,6 +74,13 @@ static cudaEvent_t* next_trace(tps_plan_s* P) {
 // double-float 3e6 rows 71 (80), 9e6 144 (148), 5e7 619 (625); fp64 3e6
 // 99 (105), 9e6 217 (259), 1.8e7 385 (426), 1e8 1945 (2160); fp32 2e6 28 (31).
 static void default_params(const tps_plan_desc& d, int32_t& m, int32_t& mr, int32_t& S) {
+  if (m == 0 && d.residency == TPS_HOST_PINNED) {
+    // bound by the link: 128 rows, shorter where that leaves few blocks (n =
+    // 2^23 double-float, two systems overlapped: 3240 us, 256 rows 3290, and
+    // the rule below, 88 rows, which do not divide into four chunks, 3467)
+    m = 128;
+    while (m > 8 && d.n_max / m < 152 * 32 * 4) m /= 2;
+  }
   if (m == 0) {
     const int64_t step = d.dtype == TPS_F32 ? 16 : 8;  // whole chunks
     auto up = [&](int64_t v) { return std::max(step, (v + step - 1) / step * step); };

@@ -405,6 +405,11 @@ def paper_rule_streams(n, coeffs):
 def default_params(n, residency, dtype=0):
     """The library's defaults (tps_plan with zero parameters, no predictor; its
     fp64 rule apart, which the timings do not cover)."""
+    if residency:
+        m = 128
+        while m > 8 and n // m < 152 * 32 * 4:
+            m //= 2
+        return m, 4, 0
     step = 16 if dtype == 1 else 8
 
     def up(v):
@@ -417,7 +422,7 @@ def default_params(n, residency, dtype=0):
         while m > 256:
             k += 1
             m = up(-(-n // (wave * k)))
-    return m, (4 if residency else 1), 0
+    return m, 1, 0
 
 
 def evaluate(rows, weights_path):
