@@ -744,7 +744,7 @@ def main():
     # (the committed ncu count per row) over its event time, against this
     # GPU's measured fp64 FMA rate
     s1p = infop["stage_ms"][0]
-    f64t = fp64_table().get(f"k_stage1_f64_m{infop['m']}", fp64_table().get("k_stage1_f64"))
+    f64t = fp64_table().get(f"k_stage1_f64_m{infop['m']}")
     plain_roof = {"bound": "fp64", "kernel": "k_stage1", "peak": fp64_peak / 1e9,
                   "unit": "G fp64-pipe thread-inst/s",
                   "peak_kind": "measured: the fastest of fp64 fma / mul / add chains "
