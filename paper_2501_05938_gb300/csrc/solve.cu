@@ -584,7 +584,7 @@ static tps_status run_solve_graph(tps_plan_s* P, int64_t n, const void* a, const
                                   int64_t nbnd) {
   const int64_t key[16] = {n, (int64_t)a, (int64_t)b, (int64_t)c, (int64_t)d, (int64_t)x,
                            (int64_t)bnd, nbnd, P->m, P->m_reduced, (int64_t)lv.size(),
-                           (int64_t)P->ws, P->desc.dtype, (int64_t)P->desc.flags, 0, 0};
+                           (int64_t)P->ws, P->desc.dtype, (int64_t)P->desc.flags, P->rel, 0};
   bool same = P->solve_graph != nullptr;
   for (int i = 0; i < 16 && same; ++i) same = P->sgkey[i] == key[i];
   if (!same) {

@@ -134,6 +134,26 @@ static size_t workspace_for(tps_plan_s* P, size_t* off_levels_out, size_t* off_d
   return off;
 }
 
+// The plan's workspace with or without relations (P->rel): its size and the
+// buffers' offsets.
+static void size_workspace(tps_plan_s* P) {
+  if (P->desc.flags & TPS_TUNE_EXHAUSTIVE) {
+    // the autotuner's smallest block size needs the largest workspace
+    const int32_t keep = P->m;
+    P->m = kTuneMin;
+    P->ws_needed = workspace_for(P, &P->off_levels, &P->off_dev);
+    P->m = keep;
+    size_t o2 = 0, d2 = 0;
+    const size_t own = workspace_for(P, &o2, &d2);
+    if (own > P->ws_needed) {
+      P->ws_needed = own;
+      P->off_dev = d2;
+    }
+  } else {
+    P->ws_needed = workspace_for(P, &P->off_levels, &P->off_dev);
+  }
+}
+
 }  // namespace tps
 
 using namespace tps;
@@ -230,32 +250,14 @@ tps_status tps_plan(const tps_plan_desc* desc, tps_plan_t* out) {
   }
   default_params(d, P->m, P->m_reduced, P->streams);
 
-  size_t off_levels = 0, off_dev = 0;
-  auto size_workspace = [&]() {
-    if (d.flags & TPS_TUNE_EXHAUSTIVE) {
-      // the autotuner's smallest block size needs the largest workspace
-      const int32_t keep = P->m;
-      P->m = kTuneMin;
-      P->ws_needed = workspace_for(P, &off_levels, &off_dev);
-      P->m = keep;
-      size_t o2 = 0, d2 = 0;
-      const size_t own = workspace_for(P, &o2, &d2);
-      if (own > P->ws_needed) {
-        P->ws_needed = own;
-        off_dev = d2;
-      }
-    } else {
-      P->ws_needed = workspace_for(P, &off_levels, &off_dev);
-    }
-  };
   // relations: up to kRelRowsMax rows (25 GB of workspace); above, and where
   // that much memory is not free, Stage 3 works from checkpoints
-  P->rel = d.n_max <= kRelRowsMax;
+  // (a caller's workspace: if it is large enough, see tps_set_workspace)
+  P->rel = d.n_max <= kRelRowsMax && !(d.flags & TPS_EXTERNAL_WORKSPACE);
   // test switch: checkpoints at any size
   if (const char* t = std::getenv("TPS_TEST_CHECKPOINTS"))
     if (t[0] == '1') P->rel = false;
-  size_workspace();
-  P->off_levels = off_levels;
+  size_workspace(P);
 
   if (const char* t = std::getenv("TPS_TEST_ONCHIP_TIMEOUT"))
     P->test_barrier_extra = t[0] == '1' ? 1 : 0;
@@ -302,7 +304,7 @@ tps_status tps_plan(const tps_plan_desc* desc, tps_plan_t* out) {
     if (e != cudaSuccess && P->rel) {
       cudaGetLastError();
       P->rel = false;
-      size_workspace();
+      size_workspace(P);
       e = cudaMalloc(&ws, P->ws_needed);
     }
     if (e != cudaSuccess) {
@@ -321,7 +323,7 @@ tps_status tps_plan(const tps_plan_desc* desc, tps_plan_t* out) {
       return TPS_ERR_CUDA;
     }
   }
-  if (P->pipe) P->pipe->off_dev = off_dev;
+  if (P->pipe) P->pipe->off_dev = P->off_dev;
   if (d.flags & TPS_HOST_OVERLAP) {
     // the twin: the same plan with the parameters chosen above, fixed
     tps_plan_desc t = P->desc;
@@ -391,8 +393,20 @@ tps_status tps_workspace_size(tps_plan_t P, size_t* bytes) {
 tps_status tps_set_workspace(tps_plan_t P, void* dev_ptr, size_t bytes) {
   if (!P || !dev_ptr) return TPS_ERR_INVALID_ARG;
   if (!(P->desc.flags & TPS_EXTERNAL_WORKSPACE)) return TPS_ERR_INVALID_ARG;
-  if (bytes < P->ws_needed || ((uintptr_t)dev_ptr % kAlign) != 0) return TPS_ERR_INVALID_ARG;
+  if (((uintptr_t)dev_ptr % kAlign) != 0) return TPS_ERR_INVALID_ARG;
   if (!on_plan_device(P) || !device_ptr_ok(dev_ptr, kAlign, P->device)) return TPS_ERR_INVALID_ARG;
+  // with relations if the buffer holds them; tps_workspace_size asks for
+  // what the solve cannot do without
+  const size_t least = P->ws_needed;
+  if (bytes < least) return TPS_ERR_INVALID_ARG;
+  P->rel = P->desc.n_max <= kRelRowsMax;
+  size_workspace(P);
+  if (bytes < P->ws_needed) {
+    P->rel = false;
+    size_workspace(P);
+  }
+  P->ws_needed = least;
+  if (P->pipe) P->pipe->off_dev = P->off_dev;
   P->ws = (unsigned char*)dev_ptr;
   P->ws_bytes = bytes;
   P->ws_owned = false;

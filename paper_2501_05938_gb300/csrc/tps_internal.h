@@ -98,6 +98,7 @@ struct tps_plan_s {
   bool codes_off = false;
   double* d_scalars = nullptr; // refinement reductions (next bytes of ws)
   size_t off_levels = 0;       // first level buffer offset
+  size_t off_dev = 0;          // host residency: device copies of a, b, c, d, x
   bool rel = false;            // the levels keep relations (see build_levels)
   size_t off_refine = 0;       // refinement residual and correction vectors
   cudaStream_t last_stream = nullptr;

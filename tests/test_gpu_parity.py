@@ -706,3 +706,36 @@ def test_boundaries_at_every_place_of_a_chunk(dtype, checkpoints, monkeypatch):
     assert plan.query()["status"] == 0
     err = oracle.rel_forward_error(x.double().cpu().numpy(), ref)
     assert err <= (1e-5 if dtype == "f32" else 1e-10)
+
+
+@pytest.mark.parametrize("dtype", ["f64", "f64_df", "f32", "mixed"])
+def test_external_workspace_with_and_without_relations(dtype):
+    """The size asked for holds no relations; a buffer that holds them makes the
+    plan use them (both give the same answer to rounding, not to the bit)."""
+    n = 100003
+    s = synth.system(41, n)
+    tdt = torch.float64
+    if dtype == "f32":
+        s, tdt = synth.to_f32(s), torch.float32
+    a, b, c, d = (torch.as_tensor(np.ascontiguousarray(s[k])).to("cuda", tdt) for k in "abcd")
+    ref = oracle.thomas(*(np.asarray(s[k], dtype=np.float64) for k in "abcd"))
+    plan = binding.Plan(n, dtype=dtype, m=32,
+                        flags=binding.NO_ONCHIP | binding.EXTERNAL_WORKSPACE | binding.GRAPH)
+    least = plan.workspace_size()
+    with pytest.raises(binding.TpsError):
+        plan.set_workspace(torch.empty(least - 1, dtype=torch.uint8, device="cuda"))
+    more = (1 << 20) + n * (14 if dtype in ("f32", "mixed") else 27)
+    ws = torch.empty(least + more, dtype=torch.uint8, device="cuda")
+    xs = []
+    for size in (least + more, least, least + more):
+        plan.set_workspace(ws[:size])
+        assert plan.workspace_size() == least
+        x = torch.full_like(b, float("nan"))
+        plan.solve(a, b, c, d, x)
+        torch.cuda.synchronize()
+        assert plan.query()["status"] == 0
+        err = oracle.rel_forward_error(x.double().cpu().numpy(), ref)
+        assert err <= (1e-5 if dtype == "f32" else 1e-10)
+        xs.append(x)
+    assert torch.equal(xs[0], xs[2])
+    assert dtype == "mixed" or not torch.equal(xs[0], xs[1])  # the other route ran
