@@ -64,15 +64,17 @@ static cudaEvent_t* next_trace(tps_plan_s* P) {
 
 // Defaults when the caller leaves a parameter at 0 and no predictor is asked
 // for.  Block size: the level-0 kernels run ten warps of 32 blocks on each of
-// 152 SMs at a time (20 KB of shared memory a warp).  A system that cannot
-// fill them twice takes 6.4 warps an SM: the sweeps are serial, so fewer and
-// longer blocks only wait, and more and shorter ones cost reduced rows.  A
-// larger one takes the longest blocks of at most 256 rows whose warps fill
+// 152 SMs at a time (20 KB of shared memory a warp).  Up to 256 rows a block,
+// the shortest blocks whose warps are at most eight an SM, two on each of its
+// quarters: the sweeps are serial, so longer blocks only wait, and with
+// shorter ones some quarters have three warps to the others' two.  A
+// larger system takes the longest blocks of at most 256 rows whose warps fill
 // their last wave.  Native fp64, bound by its pipe and the cheaper a row the
-// longer the block (decayed terms are skipped), takes up to 384 rows, in one
-// wave if that is enough.  Measured, us a solve, against 128 rows throughout:
-// double-float 3e6 rows 71 (80), 9e6 144 (148), 5e7 619 (625); fp64 3e6
-// 99 (105), 9e6 217 (259), 1.8e7 385 (426), 1e8 1945 (2160); fp32 2e6 28 (31).
+// longer the block (decayed terms are skipped), takes up to 384 rows there, in
+// one wave if that is enough.  Measured, us a solve, against 6.4 warps an SM:
+// double-float 1.5e6 rows 35 (39), 3e6 56 (61), 6e6 91 (100), fp32 3e6 26 (27),
+// fp64 3e6 89 (90); against 128 rows: double-float 3e6 56 (80), 5e7 619 (625),
+// fp64 1.8e7 385 (426), 1e8 1945 (2160) before its reciprocal was changed.
 static void default_params(const tps_plan_desc& d, int32_t& m, int32_t& mr, int32_t& S) {
   if (m == 0 && d.residency == TPS_HOST_PINNED) {
     // bound by the link: 128 rows, shorter where that leaves few blocks (n =
@@ -84,11 +86,11 @@ static void default_params(const tps_plan_desc& d, int32_t& m, int32_t& mr, int3
   if (m == 0) {
     const int64_t step = d.dtype == TPS_F32 ? 16 : 8;  // whole chunks
     auto up = [&](int64_t v) { return std::max(step, (v + step - 1) / step * step); };
-    constexpr int64_t kWave = 32 * 152 * 10, kSmall = 32 * 152 * 64 / 10;
+    constexpr int64_t kWave = 32 * 152 * 10, kSmall = 32 * 152 * 8;
     const bool f64 = d.dtype == TPS_F64;
-    const int64_t small_max = f64 ? 104 : 256, cap = f64 ? 384 : 256;
+    const int64_t cap = f64 ? 384 : 256;
     int64_t v = up((d.n_max + kSmall - 1) / kSmall);
-    if (v > small_max) {
+    if (v > 256) {
       for (int64_t k = f64 ? 1 : 2;; ++k) {
         v = up((d.n_max + kWave * k - 1) / (kWave * k));
         if (v <= cap) break;

@@ -402,27 +402,14 @@ def paper_rule_streams(n, coeffs):
                                            bg.ctypes.data, 1e6))
 
 
-def default_params(n, residency, dtype=0):
-    """The library's defaults (tps_plan with zero parameters, no predictor; its
-    fp64 rule apart, which the timings do not cover)."""
-    if residency:
-        m = 128
-        while m > 8 and n // m < 152 * 32 * 4:
-            m //= 2
-        return m, 4, 0
-    step = 16 if dtype == 1 else 8
-
-    def up(v):
-        return max(step, -(-v // step) * step)
-
-    wave, small = 32 * 152 * 10, 32 * 152 * 64 // 10
-    m, k = up(-(-n // small)), 2
-    if m > 256:
-        m = up(-(-n // (wave * k)))
-        while m > 256:
-            k += 1
-            m = up(-(-n // (wave * k)))
-    return m, 1, 0
+def default_params(n, residency):
+    """The fixed defaults the predictor is compared with: 128 rows a block, halved
+    while that leaves fewer than four warps an SM.  (tps_plan's own default for
+    device plans follows the number of warps more closely.)"""
+    m = 128
+    while m > 8 and n // m < 152 * 32 * 4:
+        m //= 2
+    return m, (4 if residency else 1), 0
 
 
 def evaluate(rows, weights_path):
@@ -440,7 +427,7 @@ def evaluate(rows, weights_path):
         tbest = min(r["ms"] for r in recs)
         pm, pS, pc = _predict(dict(n_max=n, batch_max=batch if batch > 1 else 0,
                                    dtype=(1 if dt == 1 else 3), residency=resid))
-        dm, dS, dc = default_params(n, resid, dt)
+        dm, dS, dc = default_params(n, resid)
         if kind == "host":
             t_mlp = _lookup(recs, S=pS, chunk=pc)
             t_def = _lookup(recs, S=dS, chunk=dc)
