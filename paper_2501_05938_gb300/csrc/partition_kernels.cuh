@@ -772,7 +772,9 @@ __global__ void __launch_bounds__(W * 32)
         if (!keep && __all_sync(0xffffffffu, !active || Ar::decayed(S, alp, cp))) {
           chain = false;
           na = ch + 1;
-          al = Ar::zero();
+          // not even the decayed S: it belongs to the row below this chunk,
+          // not to l, which may be another packed system's
+          al = S = Ar::zero();
         }
       } else if (__any_sync(0xffffffffu, active && !dom)) {  // start over, skip nothing
         cp_async_wait<0>();
@@ -794,7 +796,10 @@ __global__ void __launch_bounds__(W * 32)
         continue;
       }
     } else if constexpr (Ar::kSkipChain) {
-      if (chain && __all_sync(0xffffffffu, !active || Ar::chain_small(S))) chain = false;
+      if (chain && __all_sync(0xffffffffu, !active || Ar::chain_small(S))) {
+        chain = false;
+        S = Ar::zero();  // as above
+      }
     }
     if constexpr (kRef && !kRel) {  // the chunk's residual (in the d slots) out
       __syncwarp();
