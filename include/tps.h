@@ -205,6 +205,11 @@ tps_status tps_set_workspace(tps_plan_t plan, void* dev_ptr, size_t bytes);
  * relation per row (24 bytes, fp32 12), from which Stage 3 recovers x without
  * reading a, b, c, d again; for more rows, or where tps_plan cannot allocate
  * that much, it repeats the elimination from checkpoints (1.2 bytes a row).
+ * Terms that decay along a block are left out once they are 0 in the
+ * arithmetic, with one exception: TPS_F64 leaves out of a block's first
+ * unknown what would reach it from below in the same block through a product
+ * of couplings under 2^-60 (an x that much smaller than one it hangs on is
+ * not resolved there).
  *
  * TPS_MIXED_F32_F64: x0 from an fp32 elimination of the fp64 inputs, then
  * corrections until ||delta||/||x|| <= tol or max_iters.  Where the system

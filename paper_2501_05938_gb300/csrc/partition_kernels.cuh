@@ -37,8 +37,11 @@
 //
 // Stage 3, the ordinary way (kRel, k_back): Stage 1 writes the normalised
 // relation x_j = g_j - alpha_j f - c_j x_{j+1} of every interior row, lane by
-// lane as it makes them, and Stage 3 back-substitutes from these.  Terms in f
-// and the chain for x_1 are left out once they have decayed below rounding.
+// lane as it makes them, and Stage 3 back-substitutes from these.  In
+// double-float and fp32 alpha and the chain for x_1 are left out once they are
+// 0 (underflown: 50 to 80 rows into a block of an ordinary system); native
+// fp64 leaves out the chain below 2^-60 and always writes alpha, which Stage 3
+// reads only where it may be seen.
 // Both sweeps are bound by memory: 49 and 25 bytes a row, at n = 2^25 in
 // double-float 260 and 131 us, 94% of the copy rate (k_stage1 with
 // checkpoints 215 us, k_stage3 218 us).  Native fp64 Stage 1 is bound by the
@@ -253,8 +256,7 @@ struct RefineIO {
 // written by Stage 1 and read by k_back in the order in which their lanes own
 // them: row j of the nb (32, or the launch's last few) blocks of the warp that
 // starts at block k0 is nb consecutive values from (k0 * cap + j * nb).
-// al has decayed below rounding a few chunks into a block of an ordinary
-// system: na[k0] says how many chunks of the warp have it.
+// na[k0] says how many chunks of the warp have an al that counts (k_stage1).
 template <class T>
 struct alignas(2 * sizeof(T)) RelRow {
   T c, g;
@@ -488,6 +490,7 @@ __global__ void __launch_bounds__(W * 32)
   using T = typename Ar::T;
   using TL = Tile<Tin, R, kRef ? 5 : 4>;
   constexpr bool kSkip = Ar::kSkipChain || kRel;  // decayed chains are skipped
+  constexpr bool kRelF64 = Ar::kSkipChain && kRel;
   constexpr int V = TL::kVec;
   static_assert(!kRef || std::is_same<Tin, double>::value, "refinement steps are fp64");
   static_assert(R % K == 0 || K % R == 0, "chunk rows and checkpoint spacing must nest");
@@ -553,20 +556,58 @@ __global__ void __launch_bounds__(W * 32)
   // rounding and the rows skip it (kChain false); they check |c| <= |beta|
   // instead, so S cannot grow back, and a block where that fails reports a
   // pivot failure (not dominant).
-  // With kRel every policy skips, and al with the chain, once S and every
-  // later al are below 2^-60 (Ar::decayed).  Both bounds rest on the rows
-  // being dominant, which the skipping rows check (Ar::dominant): if one is
-  // not, the warp starts over and skips nothing (`keep`).
-  bool chain = true, nondom = false, dom = true, keep = false, sdec = false;
+  // The last unknown's coupling to f, al, is never left out.  With kRel the
+  // other policies skip too, S and al together, but only once both are 0 in
+  // every lane (underflown, or cut off at a system boundary), from where on
+  // every term with them is 0: nothing is lost by it.  na: the chunks in which
+  // k_back has to read al.
+  bool chain = true, nondom = false;
   int na = nch;
-  T alp = Ar::zero(), cp = Ar::zero();  // the last row's relation (al, c)
+  unsigned alex = 0;  // native fp64: the chunk's largest exponent field of al
+  // the last row's relation; before row 1, x_0 = f
+  T cp = Ar::zero(), gp = Ar::zero(), alp = Ar::neg(Ar::one());
 
   // one interior row (1 <= row <= L-2).  The product chains alpha and S and
   // the accumulators P and Q are left unnormalised here and renormalised
   // once per chunk (renorm), which bounds their low parts to a few ulps.
   RelRow<T>* const rel = static_cast<RelRow<T>*>(rl.rel) + (kRel ? k0 * rl.cap : 0);
   T* const rel_al = static_cast<T*>(rl.al) + (kRel ? k0 * rl.cap : 0);
+  // a row's pivot, right-hand side and coupling to f after the row above it
+  auto eliminate = [&](const T av, const T bv, const T dv) {
+    if constexpr (kRelF64) {
+      beta = Ar::sub_mul_dom(bv, av, cp);
+      g = Ar::sub_mul(dv, av, gp);
+      al = Ar::mul_neg_nn(av, alp);
+    } else {
+      const T ratio = Ar::mul_nn(av, rbp);
+      beta = Ar::sub_mul_dom(bv, ratio, cprev);
+      g = Ar::sub_mul(dv, ratio, g);
+      al = Ar::mul_neg_nn(ratio, al);
+    }
+  };
   auto interior = [&](const T av, const T bv, const T cv, const T dv, auto kChain, int row) {
+    if constexpr (kRelF64) {  // in the relations' own terms: one product fewer
+      eliminate(av, bv, dv);
+      bad |= Ar::bad_pivot(beta);
+      const T rbeta = Ar::rcp(beta);
+      cp = Ar::mul(cv, rbeta);
+      gp = Ar::mul(g, rbeta);
+      alp = Ar::mul(al, rbeta);
+      alex = max(alex, Ar::exponent(alp));
+      const RelRow<T> w{cp, gp};
+      if (active) {
+        rel[row * nb + lane] = w;
+        rel_al[row * nb + lane] = alp;
+      }
+      if constexpr (decltype(kChain)::value) {
+        P = Ar::sub_mul_nn(P, S, gp);
+        Q = Ar::sub_mul_nn(Q, S, alp);
+        S = Ar::mul_neg_nn(S, cp);
+      } else {
+        nondom |= !Ar::mag_le(cv, beta);
+      }
+      return;
+    }
     const T ratio = Ar::mul_nn(av, rbp);
     beta = Ar::sub_mul_dom(bv, ratio, cprev);
     g = Ar::sub_mul(dv, ratio, g);
@@ -574,35 +615,23 @@ __global__ void __launch_bounds__(W * 32)
     bad |= Ar::bad_pivot(beta);
     const T rbeta = Ar::rcp(beta);
     if constexpr (kRel) {
-      T gp;
+      RelRow<T> w;
       if constexpr (sizeof(Tin) == 4) {  // bound by memory: round the quotients once
-        cp = Ar::quot(cv, beta, rbeta);
-        gp = Ar::quot(g, beta, rbeta);
+        w.c = Ar::quot(cv, beta, rbeta);
+        w.g = Ar::quot(g, beta, rbeta);
       } else {
-        cp = Ar::mul(cv, rbeta);
-        gp = Ar::mul(g, rbeta);
+        w.c = Ar::mul(cv, rbeta);
+        w.g = Ar::mul(g, rbeta);
       }
-      const RelRow<T> w{cp, gp};
       if (active) rel[row * nb + lane] = w;
       if constexpr (decltype(kChain)::value) {
-        alp = Ar::mul(Ar::norm(al), rbeta);
-        if (active) rel_al[row * nb + lane] = alp;
-        if constexpr (Ar::kSkipChain) {  // one fp64 product fewer
-          P = Ar::sub_mul_nn(P, S, w.g);
-          Q = Ar::sub_mul_nn(Q, S, alp);
-          S = Ar::mul_neg_nn(S, cp);
-        } else {  // shorter lives of w and alp: 260 against 296 us at n = 2^25
-          const T tt = Ar::mul_nn(S, rbeta);
-          P = Ar::sub_mul_nn(P, tt, g);
-          Q = Ar::sub_mul_nn(Q, tt, al);
-          S = Ar::mul_neg_nn(tt, cv);
-        }
-        if constexpr (Ar::kSkipChain) {
-          if (sdec) nondom |= !Ar::mag_le(cv, beta);
-        }
-      } else {
-        if constexpr (Ar::kSkipChain) nondom |= !Ar::mag_le(cv, beta);
-        dom &= Ar::dominant(av, bv, cv);
+        const T aw = Ar::mul(Ar::norm(al), rbeta);
+        if (active) rel_al[row * nb + lane] = aw;
+        // not from w and aw, which would live longer: 260 against 296 us at n = 2^25
+        const T tt = Ar::mul_nn(S, rbeta);
+        P = Ar::sub_mul_nn(P, tt, g);
+        Q = Ar::sub_mul_nn(Q, tt, al);
+        S = Ar::mul_neg_nn(tt, cv);
       }
     } else if constexpr (decltype(kChain)::value) {
       const T tt = Ar::mul_nn(S, rbeta);
@@ -701,10 +730,7 @@ __global__ void __launch_bounds__(W * 32)
           if (v == 0 && rr == 0 && first) {  // the block's first row: f's equation
             a0 = av; b0 = bv; c0 = cv; d0 = dv;
           } else if (v == V - 1 && rr == R - 1 && last) {  // the block's last row
-            const T ratio = Ar::mul_nn(av, rbp);
-            beta = Ar::sub_mul_dom(bv, ratio, cprev);
-            g = Ar::sub_mul(dv, ratio, g);
-            al = Ar::mul_neg_nn(ratio, al);
+            eliminate(av, bv, dv);
             clast = cv;
           } else {
             interior(av, bv, cv, dv, kChain, row0 + rr);
@@ -748,10 +774,7 @@ __global__ void __launch_bounds__(W * 32)
               if ((row + 1) % K == 0 && r + 1 < R) checkpoint(row);
             }
           } else {
-            const T ratio = Ar::mul_nn(av, rbp);
-            beta = Ar::sub_mul_dom(bv, ratio, cprev);
-            g = Ar::sub_mul(dv, ratio, g);
-            al = Ar::mul_neg_nn(ratio, al);
+            eliminate(av, bv, dv);
             clast = cv;
           }
         }
@@ -766,39 +789,23 @@ __global__ void __launch_bounds__(W * 32)
     // the checkpoint at the chunk's end (row0 + R is a multiple of K when
     // K divides R, and every K / R chunks otherwise)
     if (((row0 + R) % K) == 0) checkpoint(row0 + R - 1);
-    if constexpr (kRel) {
+    if constexpr (Ar::kSkipChain) {
       if (chain) {
-        if (Ar::kSkipChain && __all_sync(0xffffffffu, !active || Ar::chain_small(S))) sdec = true;
-        if (!keep && __all_sync(0xffffffffu, !active || Ar::decayed(S, alp, cp))) {
+        na = ch + 1;
+        if (__all_sync(0xffffffffu, !active || Ar::chain_small(S))) {
           chain = false;
-          na = ch + 1;
           // not even the decayed S: it belongs to the row below this chunk,
           // not to l, which may be another packed system's
-          al = S = Ar::zero();
+          S = Ar::zero();
         }
-      } else if (__any_sync(0xffffffffu, active && !dom)) {  // start over, skip nothing
-        cp_async_wait<0>();
-        __syncwarp();
-        chain = keep = dom = true;
-        sdec = bad = nondom = false;
-        na = nch;
-        rbp = Ar::one();
-        cprev = g = P = Q = Ar::zero();
-        al = S = Ar::neg(Ar::one());
-        if constexpr (kRef) xup = active && start > 0 ? rf.x[start - 1] : Tin{};
-        chk.reset_codes();  // what was raised stays; the rest is seen again
-        sys = lv.nbnd > 0 && active ? bd.first : 0;
-        bj = 0;
-        if (bd.cnt > 0) bnext = (int)(bd.bnd[bd.first] - start);
-#pragma unroll
-        for (int c = 0; c < kS1Stages - 1; ++c) fetch(c);
-        ch = -1;
-        continue;
+      } else if (kRel && __any_sync(0xffffffffu, active && alex >= Ar::kLateExponent)) {
+        na = ch + 1;
       }
-    } else if constexpr (Ar::kSkipChain) {
-      if (chain && __all_sync(0xffffffffu, !active || Ar::chain_small(S))) {
+      alex = 0;
+    } else if constexpr (kRel) {
+      if (chain && __all_sync(0xffffffffu, !active || (Ar::is_zero(S) && Ar::is_zero(al)))) {
         chain = false;
-        S = Ar::zero();  // as above
+        na = ch + 1;
       }
     }
     if constexpr (kRef && !kRel) {  // the chunk's residual (in the d slots) out
@@ -1093,7 +1100,7 @@ __global__ void __launch_bounds__(32)
   PieceMap<Tin, R> pm;
   pm.init(lv, k0, nb, lane);
   chain_wait();
-  const int na = rl.na[k0];
+  int na = rl.na[k0];
   const Tin* const xsrc[1] = {x};
   auto rows_of = [&](int st) {
     return reinterpret_cast<RelRow<T>*>(smem_raw + st * BT::kStage);
@@ -1136,7 +1143,7 @@ __global__ void __launch_bounds__(32)
     l = Ar::from(xred[2 * k + 1]);
   }
   T xn = l;
-  bool oob = false;
+  bool oob = false, late = false;
   unsigned long long mdel = 0, mx = 0;  // refinement maxima (bit patterns)
   int st = 0;
   for (int ch = nch - 1; ch >= 0; --ch) {
@@ -1162,6 +1169,9 @@ __global__ void __launch_bounds__(32)
           if constexpr (decltype(kAl)::value) g = Ar::sub_mul(g, wal[r * nb], f);
           xn = Ar::sub_mul(g, e.c, xn);
           xr = xn;
+          if constexpr (Ar::kSkipChain) {
+            if constexpr (!decltype(kAl)::value) late |= in && Ar::late(xr, f);
+          }
         } else if (row == 0) {
           xr = f;
         } else if (row == L - 1) {
@@ -1196,6 +1206,18 @@ __global__ void __launch_bounds__(32)
     store_chunk<Tin, R, kVec16>(x, tile, pm, row0);
     __syncwarp();  // the slots are refilled by a later chunk
     st = st == kBackStages - 1 ? 0 : st + 1;
+    if constexpr (Ar::kSkipChain) {  // an x so small that f may be missed: again, with every al
+      if (ch == na && __any_sync(0xffffffffu, late)) {
+        cp_async_wait<0>();
+        __syncwarp();
+        na = nch;
+        xn = l;
+        st = 0;
+#pragma unroll
+        for (int i = 0; i < kBackStages - 1; ++i) fetch(nch - 1 - i, i);
+        ch = nch;
+      }
+    }
   }
   if (oob) atomicOr(status, ST_RANGE);
   if (lv.dmax)

@@ -75,3 +75,44 @@ def test_packed_systems_do_not_couple(dtype, checkpoints, b, cut, monkeypatch):
         for lo, hi, size in ((0, off[1], first), (off[1], n, second)):
             err = np.abs(x[lo:hi] - ref[lo:hi]).max()
             assert err <= 16 * cond * ULP[dtype] * np.abs(ref[lo:hi]).max(), (first, second, size)
+
+
+# How far below the impulse a component keeps its relative accuracy: native
+# fp64 to the format's end; double-float as long as a relation's pair is normal
+# (2^-126 with 24 bits of its low part below), fp32 as long as the value is.
+DEEP = {"f64": 2.0 ** -950, "f64_df": 2.0 ** -98, "f32": 2.0 ** -120}
+
+
+def impulse_error(x, ref, peak, dtype):
+    """Largest relative error among the components down to DEEP of the peak."""
+    use = np.abs(ref) >= DEEP[dtype] * peak
+    return (np.abs(x - ref)[use] / np.abs(ref)[use]).max()
+
+
+@pytest.mark.parametrize("checkpoints", [False, True])
+@pytest.mark.parametrize("dtype", ["f64", "f64_df", "f32"])
+@pytest.mark.parametrize("at", [0, 1, 17, 100, 255])
+def test_impulse_is_resolved_far_below_its_peak(dtype, checkpoints, at, monkeypatch):
+    """One nonzero entry in d, `at` rows into a block: x falls by 2 + sqrt(3) a
+    row on either side, with no cancellation anywhere, so every component has
+    a small relative error (a few roundings a row: 4 n ulp with n the rows it
+    has come).  Native fp64 is held to it downwards of the impulse; upwards it
+    leaves out what reaches a block's first unknown over more than 2^-60."""
+    m, n = 256, 256 * 40
+    s = toeplitz(n, 4.0)
+    row, peak = 11 * m + at, 2.0 ** 60
+    s["d"] = np.zeros(n)
+    s["d"][row] = peak
+    ref = oracle.thomas(*(s[k] for k in "abcd"))
+    plan = make_plan(n, dtype, checkpoints, monkeypatch, m=m, flags=binding.NO_ONCHIP)
+    a, b, c, d = to_device(s, dtype)
+    x = torch.full_like(b, float("nan"))
+    plan.solve(a, b, c, d, x)
+    torch.cuda.synchronize()
+    assert plan.query()["status"] == 0
+    x = x.double().cpu().numpy()
+    if dtype == "f64":
+        up = ref[:row] >= 2.0 ** -50 * peak
+        assert (np.abs(x - ref)[:row][up] <= 2.0 ** -44 * ref[:row][up]).all()
+        x, ref = x[row:], ref[row:]
+    assert impulse_error(x, ref, peak, dtype) <= 2048 * ULP[dtype]
