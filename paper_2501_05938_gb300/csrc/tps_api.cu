@@ -102,58 +102,65 @@ static void default_params(const tps_plan_desc& d, int32_t& m, int32_t& mr, int3
   if (S == 0) S = (d.residency == TPS_HOST_PINNED) ? 4 : 1;
 }
 
-static size_t workspace_for(tps_plan_s* P, size_t* off_levels_out, size_t* off_dev_out) {
+// The buffers of a plan's workspace with block size m, with or without
+// relations, and its size.
+struct WsLayout {
+  size_t dmax, xch, win, levels, refine, dev, end;
+};
+static WsLayout workspace_layout(const tps_plan_s* P, int32_t m, bool rel) {
+  WsLayout W = {};
   size_t off = 0;
   off = align_up(off + 64);  // status word, refinement maxima, grid-barrier counters
-  P->off_dmax = off;         // per-system range codes (zero between solves)
+  W.dmax = off;              // per-system range codes (zero between solves)
   off = align_up(off + 4 * kCodes * (size_t)std::max<int64_t>(1, P->desc.batch_max));
-  P->off_xch = off;          // interface rows of the on-chip solve
+  W.xch = off;               // interface rows of the on-chip solve
   off = align_up(off + onchip_exchange_bytes());
-  *off_levels_out = off;
   if (P->desc.flags & TPS_TRUNCATE) {  // windows are solved on their own: no levels
-    P->off_rel = off;
-    off = align_up(off + truncate_rel_bytes(P->desc.n_max, P->m, P->m_reduced, P->desc.dtype));
-    *off_levels_out = off;
-    *off_dev_out = off;
-    return off;
+    W.win = off;
+    off = align_up(off + truncate_rel_bytes(P->desc.n_max, m, P->m_reduced, P->desc.dtype));
+    W.levels = W.refine = W.dev = W.end = off;
+    return W;
   }
+  W.levels = off;
   std::vector<LevelPlan> lv;
   const size_t eio = elem_bytes_io(P->desc.dtype);
   const size_t ered = elem_bytes_red(P->desc.dtype);
   int64_t nmax = P->desc.n_max;
-  size_t end = build_levels(nmax, P->m, P->m_reduced, eio, ered, P->rel, off, lv);
+  off = build_levels(nmax, m, P->m_reduced, eio, ered, rel, off, lv);
+  W.refine = off;
   if (P->desc.dtype == TPS_MIXED_F32_F64) {
     // residual r and correction delta (fp64)
-    P->off_refine = end;
-    end = align_up(end + (size_t)nmax * 8);
-    end = align_up(end + (size_t)nmax * 8);
+    off = align_up(off + (size_t)nmax * 8);
+    off = align_up(off + (size_t)nmax * 8);
   }
-  off = end;
-  *off_dev_out = off;
+  W.dev = off;
   if (P->desc.residency == TPS_HOST_PINNED) {
     for (int i = 0; i < 5; ++i) off = align_up(off + (size_t)nmax * eio);
   }
-  return off;
+  W.end = off;
+  return W;
 }
 
-// The plan's workspace with or without relations (P->rel): its size and the
-// buffers' offsets.
-static void size_workspace(tps_plan_s* P) {
-  if (P->desc.flags & TPS_TUNE_EXHAUSTIVE) {
-    // the autotuner's smallest block size needs the largest workspace
-    const int32_t keep = P->m;
-    P->m = kTuneMin;
-    P->ws_needed = workspace_for(P, &P->off_levels, &P->off_dev);
-    P->m = keep;
-    size_t o2 = 0, d2 = 0;
-    const size_t own = workspace_for(P, &o2, &d2);
-    if (own > P->ws_needed) {
-      P->ws_needed = own;
-      P->off_dev = d2;
-    }
-  } else {
-    P->ws_needed = workspace_for(P, &P->off_levels, &P->off_dev);
-  }
+// What the plan needs with block size m; the autotuner's smallest block size
+// needs the most.
+static size_t workspace_size(const tps_plan_s* P, int32_t m, bool rel) {
+  size_t v = workspace_layout(P, m, rel).end;
+  if (P->desc.flags & TPS_TUNE_EXHAUSTIVE)
+    v = std::max(v, workspace_layout(P, kTuneMin, rel).end);
+  return v;
+}
+
+// The plan takes block size m, with or without relations.
+static void place(tps_plan_s* P, int32_t m, bool rel) {
+  const WsLayout W = workspace_layout(P, m, rel);
+  P->m = m;
+  P->rel = rel;
+  P->off_dmax = W.dmax;
+  P->off_xch = W.xch;
+  P->off_rel = W.win;
+  P->off_levels = W.levels;
+  P->off_refine = W.refine;
+  if (P->pipe) P->pipe->off_dev = W.dev;
 }
 
 }  // namespace tps
@@ -255,11 +262,12 @@ tps_status tps_plan(const tps_plan_desc* desc, tps_plan_t* out) {
   // relations: up to kRelRowsMax rows (25 GB of workspace); above, and where
   // that much memory is not free, Stage 3 works from checkpoints
   // (a caller's workspace: if it is large enough, see tps_set_workspace)
-  P->rel = d.n_max <= kRelRowsMax && !(d.flags & TPS_EXTERNAL_WORKSPACE);
+  bool rel = d.n_max <= kRelRowsMax && !(d.flags & TPS_EXTERNAL_WORKSPACE);
   // test switch: checkpoints at any size
   if (const char* t = std::getenv("TPS_TEST_CHECKPOINTS"))
-    if (t[0] == '1') P->rel = false;
-  size_workspace(P);
+    if (t[0] == '1') rel = false;
+  P->m_plan = P->m;
+  P->ws_needed = workspace_size(P, P->m, rel);
 
   if (const char* t = std::getenv("TPS_TEST_ONCHIP_TIMEOUT"))
     P->test_barrier_extra = t[0] == '1' ? 1 : 0;
@@ -303,10 +311,10 @@ tps_status tps_plan(const tps_plan_desc* desc, tps_plan_t* out) {
   if (!(d.flags & TPS_EXTERNAL_WORKSPACE)) {
     void* ws = nullptr;
     cudaError_t e = cudaMalloc(&ws, P->ws_needed);
-    if (e != cudaSuccess && P->rel) {
+    if (e != cudaSuccess && rel) {
       cudaGetLastError();
-      P->rel = false;
-      size_workspace(P);
+      rel = false;
+      P->ws_needed = workspace_size(P, P->m, rel);
       e = cudaMalloc(&ws, P->ws_needed);
     }
     if (e != cudaSuccess) {
@@ -319,13 +327,13 @@ tps_status tps_plan(const tps_plan_desc* desc, tps_plan_t* out) {
     P->ws_owned = true;
     P->d_status = (int*)P->ws;
     P->d_scalars = (double*)(P->ws + 8);
+    place(P, P->m, rel);
     e = cudaMemset(P->ws, 0, P->off_xch);  // header and range codes
     if (e != cudaSuccess) {
       tps_plan_destroy(P);
       return TPS_ERR_CUDA;
     }
   }
-  if (P->pipe) P->pipe->off_dev = P->off_dev;
   if (d.flags & TPS_HOST_OVERLAP) {
     // the twin: the same plan with the parameters chosen above, fixed
     tps_plan_desc t = P->desc;
@@ -397,18 +405,12 @@ tps_status tps_set_workspace(tps_plan_t P, void* dev_ptr, size_t bytes) {
   if (!(P->desc.flags & TPS_EXTERNAL_WORKSPACE)) return TPS_ERR_INVALID_ARG;
   if (((uintptr_t)dev_ptr % kAlign) != 0) return TPS_ERR_INVALID_ARG;
   if (!on_plan_device(P) || !device_ptr_ok(dev_ptr, kAlign, P->device)) return TPS_ERR_INVALID_ARG;
-  // with relations if the buffer holds them; tps_workspace_size asks for
-  // what the solve cannot do without
-  const size_t least = P->ws_needed;
-  if (bytes < least) return TPS_ERR_INVALID_ARG;
-  P->rel = P->desc.n_max <= kRelRowsMax;
-  size_workspace(P);
-  if (bytes < P->ws_needed) {
-    P->rel = false;
-    size_workspace(P);
-  }
-  P->ws_needed = least;
-  if (P->pipe) P->pipe->off_dev = P->off_dev;
+  if (bytes < P->ws_needed) return TPS_ERR_INVALID_ARG;
+  // with relations if the buffer holds them; a block size that tps_autotune
+  // chose on a larger buffer and that needs more than this one goes back to the
+  // plan's, for which ws_needed suffices
+  const bool rel = P->desc.n_max <= kRelRowsMax && workspace_size(P, P->m, true) <= bytes;
+  place(P, rel || workspace_size(P, P->m, false) <= bytes ? P->m : P->m_plan, rel);
   P->ws = (unsigned char*)dev_ptr;
   P->ws_bytes = bytes;
   P->ws_owned = false;
@@ -791,9 +793,8 @@ tps_status tps_autotune(tps_plan_t P, int64_t n, int64_t count, const int64_t* o
   float best_t = -1.0f;
   tps_status st = TPS_OK;
   for (int32_t m = kTuneMin; m <= kTuneMax && st == TPS_OK; m *= 2) {
-    P->m = m;
-    size_t o1 = 0, o2 = 0;
-    if (workspace_for(P, &o1, &o2) > P->ws_bytes) continue;  // does not fit this plan
+    if (workspace_layout(P, m, P->rel).end > P->ws_bytes) continue;  // does not fit this plan
+    place(P, m, P->rel);
     st = solve();  // warm-up
     if (st != TPS_OK) break;
     if (cudaEventRecord(e0, s) != cudaSuccess) { st = TPS_ERR_CUDA; break; }

@@ -84,6 +84,7 @@ struct tps_plan_s {
   tps_plan_desc desc;
   int32_t device = -1;  // the device current at tps_plan; every call must use it
   int32_t m = 0, m_reduced = 0, streams = 1;
+  int32_t m_plan = 0;  // m when the plan was made (tps_autotune may change m)
   int64_t chunk = 0;
   unsigned char* ws = nullptr;
   size_t ws_bytes = 0, ws_needed = 0;
@@ -98,7 +99,6 @@ struct tps_plan_s {
   bool codes_off = false;
   double* d_scalars = nullptr; // refinement reductions (next bytes of ws)
   size_t off_levels = 0;       // first level buffer offset
-  size_t off_dev = 0;          // host residency: device copies of a, b, c, d, x
   bool rel = false;            // the levels keep relations (see build_levels)
   size_t off_refine = 0;       // refinement residual and correction vectors
   cudaStream_t last_stream = nullptr;

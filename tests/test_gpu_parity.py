@@ -739,3 +739,30 @@ def test_external_workspace_with_and_without_relations(dtype):
         xs.append(x)
     assert torch.equal(xs[0], xs[2])
     assert dtype == "mixed" or not torch.equal(xs[0], xs[1])  # the other route ran
+
+
+@pytest.mark.parametrize("dtype", ["f64", "mixed"])
+def test_workspace_of_the_size_asked_for_after_autotune(dtype):
+    """tps_autotune on a large buffer picks blocks shorter than the plan's, whose
+    levels take more than tps_workspace_size; a buffer of that size given
+    afterwards is still enough: nothing beyond it is written."""
+    n = 100003
+    s = synth.system(43, n)
+    a, b, c, d = (dev(s[k]) for k in "abcd")
+    plan = binding.Plan(n, dtype=dtype, m=1024,
+                        flags=binding.NO_ONCHIP | binding.EXTERNAL_WORKSPACE)
+    least = plan.workspace_size()
+    buf = torch.zeros(least + 64 * n, dtype=torch.uint8, device="cuda")
+    plan.set_workspace(buf)
+    x = torch.full_like(b, float("nan"))
+    m, _ = plan.autotune(a, b, c, d, x, reps=1)
+    assert m < 1024 and plan.workspace_size() == least
+    plan.set_workspace(buf[:least])
+    buf[least:] = 0xA5
+    x.fill_(float("nan"))
+    plan.solve(a, b, c, d, x)
+    torch.cuda.synchronize()
+    assert plan.query()["status"] == 0
+    assert bool((buf[least:] == 0xA5).all())
+    ref = oracle.thomas(s["a"], s["b"], s["c"], s["d"])
+    assert oracle.rel_forward_error(x.cpu().numpy(), ref) <= F64_FWD
