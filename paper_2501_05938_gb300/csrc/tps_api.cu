@@ -814,7 +814,8 @@ tps_status tps_autotune(tps_plan_t P, int64_t n, int64_t count, const int64_t* o
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
-  P->m = (st == TPS_OK && best_t >= 0.0f) ? best : keep;
+  // also the buffers that lie behind the levels of this block size
+  place(P, (st == TPS_OK && best_t >= 0.0f) ? best : keep, P->rel);
   if (best_m) *best_m = P->m;
   if (best_ms) *best_ms = best_t;
   return st;

@@ -138,3 +138,24 @@ def test_autotune_picks_a_block_size_and_stays_correct():
     torch.cuda.synchronize()
     ref = oracle.thomas(s["a"], s["b"], s["c"], s["d"])
     assert oracle.rel_forward_error(x.cpu().numpy(), ref) <= 1e-10
+
+
+def test_autotuned_mixed_plan_from_checkpoints(monkeypatch):
+    """The residual's buffer lies behind the levels of the block size chosen, not
+    of the last one timed, in which it would be written over them."""
+    n = 100003
+    s = synth.system(47, n, kind=synth.KIND_RATIO, ratio=1.01)
+    a, b, c, d = (torch.as_tensor(np.ascontiguousarray(s[k])).cuda() for k in "abcd")
+    monkeypatch.setenv("TPS_TEST_CHECKPOINTS", "1")
+    plan = binding.Plan(n, dtype="mixed", flags=binding.NO_ONCHIP | binding.TUNE_EXHAUSTIVE)
+    monkeypatch.delenv("TPS_TEST_CHECKPOINTS")
+    x = torch.full_like(b, float("nan"))
+    m, _ = plan.autotune(a, b, c, d, x, reps=1)
+    assert m < 1024
+    x.fill_(float("nan"))
+    plan.solve(a, b, c, d, x)
+    torch.cuda.synchronize()
+    info = plan.query()
+    assert info["status"] == 0 and info["refine_fused"], info
+    ref = oracle.thomas(s["a"], s["b"], s["c"], s["d"])
+    assert oracle.rel_forward_error(x.cpu().numpy(), ref) <= 1e-12
