@@ -397,9 +397,9 @@ int tps_predict_load(const char* path);
 
 /* Exhaustive search: time tps_solve (count == 0: one system of n rows) or
  * tps_solve_batched (count > 0, offsets as there) on the caller's data for
- * every block size m in {16, 32, ..., 1024} whose workspace fits the plan,
- * `reps` timed solves each after one warm-up, and keep the fastest m in the
- * plan.  A plan created with TPS_TUNE_EXHAUSTIVE sizes its workspace for the
+ * the plan's block size and every m in {16, 32, ..., 1024} whose workspace
+ * fits the plan, `reps` timed solves each after one warm-up, and keep the
+ * fastest m in the plan.  A plan created with TPS_TUNE_EXHAUSTIVE sizes its workspace for the
  * whole grid.  Synchronises `stream`; x is overwritten.  *best_m and
  * *best_ms (may be NULL) receive the choice and its mean time.
  * For a host-residency plan (count must be 0, a..x pinned or, with

@@ -792,7 +792,10 @@ tps_status tps_autotune(tps_plan_t P, int64_t n, int64_t count, const int64_t* o
   int32_t best = keep;
   float best_t = -1.0f;
   tps_status st = TPS_OK;
-  for (int32_t m = kTuneMin; m <= kTuneMax && st == TPS_OK; m *= 2) {
+  // the plan's own block size first, then the grid
+  for (int32_t i = 0; (kTuneMin << i) / 2 <= kTuneMax && st == TPS_OK; ++i) {
+    const int32_t m = i == 0 ? keep : (kTuneMin << i) / 2;
+    if (i > 0 && m == keep) continue;
     if (workspace_layout(P, m, P->rel).end > P->ws_bytes) continue;  // does not fit this plan
     place(P, m, P->rel);
     st = solve();  // warm-up

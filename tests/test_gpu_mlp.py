@@ -159,3 +159,15 @@ def test_autotuned_mixed_plan_from_checkpoints(monkeypatch):
     assert info["status"] == 0 and info["refine_fused"], info
     ref = oracle.thomas(s["a"], s["b"], s["c"], s["d"])
     assert oracle.rel_forward_error(x.cpu().numpy(), ref) <= 1e-12
+
+
+def test_autotune_times_the_plans_own_block_size(monkeypatch):
+    """Here the only one: from checkpoints shorter blocks need more workspace."""
+    n, m = 200003, 2048
+    s = synth.system(48, n)
+    a, b, c, d = (torch.as_tensor(np.ascontiguousarray(s[k])).cuda() for k in "abcd")
+    monkeypatch.setenv("TPS_TEST_CHECKPOINTS", "1")
+    plan = binding.Plan(n, dtype="f64", m=m, flags=binding.NO_ONCHIP)
+    monkeypatch.delenv("TPS_TEST_CHECKPOINTS")
+    best, ms = plan.autotune(a, b, c, d, torch.empty_like(b), reps=1)
+    assert best == m and ms > 0
