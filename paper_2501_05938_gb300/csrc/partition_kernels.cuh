@@ -429,13 +429,14 @@ __device__ __forceinline__ void load_xchunk(Tin* buf, const Tin* x, const XPiece
   }
 }
 
-// r = d - (a x_{i-1} + b x_i + c x_{i+1}) in fp64 (a and c already cut to
-// zero where a coupling does not exist, and the matching x passed as 0).
+// r = d - (a x_{i-1} + b x_i + c x_{i+1}) in fp64.  Where a or c is 0 (cut at
+// a boundary) the x beside it, which may belong to another system, is left out:
+// it must not reach this one as 0 * inf.
 __device__ __forceinline__ double residual_row(double a, double b, double c, double d, double xm,
                                                double x0, double xp) {
   double r = fma(-b, x0, d);
-  r = fma(-a, xm, r);
-  return fma(-c, xp, r);
+  r = fma(-a, ArF64::is_zero(a) ? 0.0 : xm, r);
+  return fma(-c, ArF64::is_zero(c) ? 0.0 : xp, r);
 }
 // |v|'s bit pattern from integer operations on the two halves (masking the
 // sign of the 64-bit pattern is compiled as an fp64 absolute value, an
@@ -445,12 +446,6 @@ __device__ __forceinline__ unsigned long long abs_bits(double v) {
   const unsigned hi = (unsigned)__double2hiint(v) & 0x7FFFFFFFu;
   const unsigned lo = (unsigned)__double2loint(v);
   return ((unsigned long long)hi << 32) | lo;
-}
-
-// Is v +-0, from its bits?  (A coupling that was cut: the x beside it, which
-// may belong to another system, must not reach this one as 0 * inf.)
-__device__ __forceinline__ bool is_zero(double v) {
-  return (((unsigned)__double2hiint(v) & 0x7FFFFFFFu) | (unsigned)__double2loint(v)) == 0u;
 }
 
 // ------------------------------------------------------------------ Stage 1
@@ -720,8 +715,7 @@ __global__ void __launch_bounds__(W * 32)
           Tin din = xd.v[v];
           if constexpr (kRef) {  // the residual of the current x
             const Tin x0 = t[4 * TL::kArr + rr], xdn = t[4 * TL::kArr + rr + 1];
-            din = residual_row(xa.v[v], xb.v[v], xc.v[v], din, is_zero(xa.v[v]) ? Tin{} : xup, x0,
-                               is_zero(xc.v[v]) ? Tin{} : xdn);
+            din = residual_row(xa.v[v], xb.v[v], xc.v[v], din, xup, x0, xdn);
             xup = x0;
             if constexpr (!kRel) t[3 * TL::kArr + rr] = din;
           }
@@ -756,9 +750,7 @@ __global__ void __launch_bounds__(W * 32)
           Tin din = t[3 * TL::kArr + r];
           if constexpr (kRef) {
             const Tin x0 = t[4 * TL::kArr + r], xdn = t[4 * TL::kArr + r + 1];
-            din = residual_row(t[r], t[TL::kArr + r], t[2 * TL::kArr + r], din,
-                               is_zero(t[r]) ? Tin{} : xup, x0,
-                               is_zero(t[2 * TL::kArr + r]) ? Tin{} : xdn);
+            din = residual_row(t[r], t[TL::kArr + r], t[2 * TL::kArr + r], din, xup, x0, xdn);
             xup = x0;
             t[3 * TL::kArr + r] = din;
           }

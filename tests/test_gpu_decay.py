@@ -116,3 +116,23 @@ def test_impulse_is_resolved_far_below_its_peak(dtype, checkpoints, at, monkeypa
         assert (np.abs(x - ref)[:row][up] <= 2.0 ** -44 * ref[:row][up]).all()
         x, ref = x[row:], ref[row:]
     assert impulse_error(x, ref, peak, dtype) <= 2048 * ULP[dtype]
+
+
+@pytest.mark.parametrize("dtype,n", [("f64", 5000), ("f64", 20011), ("f64_df", 5000),
+                                     ("f64_df", 100003), ("f32", 20011), ("f32", 300007)])
+def test_impulse_on_chip(dtype, n):
+    """The same on chip, where the interface rows of the CTAs around decide."""
+    s = toeplitz(n, 4.0)
+    peak = 2.0 ** 60
+    for row in (n // 2, n // 3 + 5, 0, n - 1):
+        s["d"] = np.zeros(n)
+        s["d"][row] = peak
+        ref = oracle.thomas(*(s[k] for k in "abcd"))
+        plan = binding.Plan(n, dtype=dtype)
+        a, b, c, d = to_device(s, dtype)
+        x = torch.full_like(b, float("nan"))
+        plan.solve(a, b, c, d, x)
+        torch.cuda.synchronize()
+        info = plan.query()
+        assert info["status"] == 0 and info["onchip"] == 1, info
+        assert impulse_error(x.double().cpu().numpy(), ref, peak, dtype) <= 2048 * ULP[dtype]
