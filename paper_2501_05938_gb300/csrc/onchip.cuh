@@ -404,6 +404,7 @@ __global__ void __launch_bounds__(kOcThreads, 1)
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ unsigned code_s[2][3];  // this CTA's range codes; CTA 0: the system's
   __shared__ int ok_s;
+  __shared__ bool gave_s[kOcMaxCtas];
   Tin* s0[4];
 #pragma unroll
   for (int k = 0; k < 4; ++k) s0[k] = reinterpret_cast<Tin*>(smem_raw + k * Lay::kL0);
@@ -417,13 +418,17 @@ __global__ void __launch_bounds__(kOcThreads, 1)
   constexpr int V = 16 / (int)sizeof(Tin);
   const bool fin = sh.mode == kFinish;
   chain_wait();
-  if (fin && ld_l2(sh.bar + 2) == 0u) {
-    if (tid == 0) oc_report(sh);
-    return;
+  if (fin) {  // which CTAs gave up, read once for all threads
+    const bool any = tid == 0 && ld_l2(sh.bar + 2) != 0u;
+    for (int i = tid; i < G; i += B) gave_s[i] = ld_l2(xgave + i) != 0u;
+    if (!__syncthreads_or(any)) {
+      if (tid == 0) oc_report(sh);
+      return;
+    }
   }
 #pragma unroll 1
   for (int cta = fin ? 0 : (int)blockIdx.x; cta < (fin ? G : (int)blockIdx.x + 1); ++cta) {
-    if (fin && ld_l2(xgave + cta) == 0u) continue;
+    if (fin && !gave_s[cta]) continue;
     const int64_t kb = (int64_t)cta * B;
     const int64_t ke = kb + B < p ? kb + B : p;
     const int nb = (int)(ke - kb);
@@ -571,7 +576,10 @@ __global__ void __launch_bounds__(kOcThreads, 1)
       done = settled();
     }
     T fc = shfl_v(pv, 15), lc = shfl_v(pv, 16);
-    if (!done) {  // the same in every warp of the CTA: weakly coupled nowhere near
+    // the same in every warp, of which each has read the rows by itself: made
+    // so, since the barriers below need it even if another solve on the same
+    // exchange rows (a misuse) changed them in between
+    if (!(G > 1 ? __syncthreads_and(done) : done)) {  // not weakly coupled nearby
       T* cur = pc;
       T* nxt = pc + 3 * M;
       for (int i = tid; i < 3 * M; i += B) cur[i] = ld_l2(xch + i);

@@ -329,6 +329,13 @@ tps_status tps_plan(const tps_plan_desc* desc, tps_plan_t* out) {
     P->d_scalars = (double*)(P->ws + 8);
     place(P, P->m, rel);
     e = cudaMemset(P->ws, 0, P->off_xch);  // header and range codes
+    // test switch: the on-chip barrier's counters as two solves on one plan at
+    // once (a misuse) may leave them
+    if (const char* t = std::getenv("TPS_TEST_ONCHIP_RESIDUE")) {
+      const unsigned one[2] = {1u, 1u};
+      if (t[0] == '1' && e == cudaSuccess)
+        e = cudaMemcpy(P->ws + 32, one, sizeof(one), cudaMemcpyHostToDevice);
+    }
     if (e != cudaSuccess) {
       tps_plan_destroy(P);
       return TPS_ERR_CUDA;

@@ -177,3 +177,21 @@ def test_ctas_that_gave_up_are_done_again(dtype, n, monkeypatch):
         x, info = solve(plan, s, tdt)
         assert info["status"] == 0 and info["onchip"] == 1, info
         assert np.array_equal(x, x0)
+
+
+@pytest.mark.parametrize("dtype,n", [("f64", 10007), ("f64_df", 40009), ("f64_df", 800001),
+                                     ("f32", 40009), ("f32", 1000003)])
+def test_barrier_that_opened_early(dtype, n, monkeypatch):
+    """A count left at the barrier (by two solves on one plan at once, a misuse)
+    lets CTAs read interface rows that others are still writing.  That solve
+    is spoiled, but its warps stay together and the context survives."""
+    monkeypatch.setenv("TPS_TEST_ONCHIP_RESIDUE", "1")
+    plan = binding.Plan(n, dtype=dtype)
+    monkeypatch.delenv("TPS_TEST_ONCHIP_RESIDUE")
+    s = synth.system(53, n)
+    tdt = torch.float64
+    if dtype == "f32":
+        s, tdt = synth.to_f32(s), torch.float32
+    for _ in range(3):
+        solve(plan, s, tdt)
+    check(dtype, n, 53, 1)
