@@ -353,13 +353,14 @@ __device__ __forceinline__ void red_release_add(unsigned* p, unsigned v) {
 // one CTA, returns at once if none did, else does those CTAs' rows again, by
 // when every interface equation is there.  No CTA waits for one that cannot
 // run.  (launch_onchip_raw chooses.)
-enum OcMode : int { kCoop = 0, kFirst = 1, kFinish = 2 };
+enum OcMode : int { kSolo = 0, kCoop = 1, kFirst = 2, kFinish = 3 };
 constexpr unsigned kOcPatience = 512;  // kFirst: polls of about 0.3 us
 
-// What the CTAs of one launch share.
+// What the CTAs of one solve share.
 struct OcShared {
-  unsigned* bar;      // [0] arrivals at the barrier, [1] CTAs done, [2] CTAs that gave up;
-                      // all zero between solves (the last CTA clears them)
+  unsigned* bar;      // arrivals at the barrier; 0 between solves: whatever they
+                      // left there, the solve's last launch clears it (kFinish,
+                      // k_onchip_end), so that no solve can spoil a later one
   unsigned arrivals;  // what the barrier waits for: G (more only to exercise the timeout)
   int* status;
   int32_t* report;    // with own_status: the solve's tps_status, or null
@@ -373,23 +374,17 @@ __device__ __forceinline__ void oc_report(const OcShared& sh) {
     if (sh.report) *sh.report = status_code(w);
   }
 }
-// The CTA is done with everything it shares: the last one clears the
-// barrier for the next launch and, at the end of the solve, reports.
-__device__ __forceinline__ void oc_leave(const OcShared& sh, unsigned G) {
-  __syncthreads();
-  if (threadIdx.x != 0) return;
-  __threadfence();
-  if (G > 1 && atomicAdd(sh.bar + 1, 1u) != G - 1) return;
-  __threadfence();
-  sh.bar[0] = 0u;
-  sh.bar[1] = 0u;
-  if (sh.mode == kCoop) oc_report(sh);
+// After a cooperative launch: the barrier's counter and the solve's report.
+static __global__ void k_onchip_end(OcShared sh) {
+  chain_wait();
+  *sh.bar = 0u;
+  oc_report(sh);
 }
 
 // n rows, level-0 blocks of mt rows (p blocks, the last of length in
 // [2, mt + 1]), blockDim.x of them per CTA (64, 128 or 256), G CTAs.  xch: 3 x 2G
 // values of T (the interface equations), then 3 x G range codes and G flags
-// (1: the CTA gave up).  vec16: a, b, c, d, x 16-byte aligned.
+// (1: the CTA gave up; kFirst).  vec16: a, b, c, d, x 16-byte aligned.
 // codes: judge the system's range (level 0 of fp64 inputs in narrower
 // arithmetic).
 template <class Ar, class Tin>
@@ -419,8 +414,9 @@ __global__ void __launch_bounds__(kOcThreads, 1)
   const bool fin = sh.mode == kFinish;
   chain_wait();
   if (fin) {  // which CTAs gave up, read once for all threads
-    const bool any = tid == 0 && ld_l2(sh.bar + 2) != 0u;
-    for (int i = tid; i < G; i += B) gave_s[i] = ld_l2(xgave + i) != 0u;
+    if (tid == 0) *sh.bar = 0u;
+    bool any = false;
+    for (int i = tid; i < G; i += B) any |= gave_s[i] = ld_l2(xgave + i) != 0u;
     if (!__syncthreads_or(any)) {
       if (tid == 0) oc_report(sh);
       return;
@@ -502,7 +498,7 @@ __global__ void __launch_bounds__(kOcThreads, 1)
     if (tid < 32) __syncwarp();  // lane `last`'s stores before lane 0's release
 
     // ---- grid barrier; warp 0 wrote all that the other CTAs read
-    if (sh.arrivals > 1 && !fin) {
+    if (publish) {
       if (tid == 0) {
         red_release_add(sh.bar, 1u);
         int ok = 1;
@@ -511,8 +507,7 @@ __global__ void __launch_bounds__(kOcThreads, 1)
         while (ld_acquire_u32(sh.bar) < sh.arrivals) {
           if (++it > limit) {
             ok = 0;
-            if (sh.mode == kFirst) atomicAdd(sh.bar + 2, 1u);
-            else atomicOr(sh.status, ST_TIMEOUT);
+            if (sh.mode == kCoop) atomicOr(sh.status, ST_TIMEOUT);
             break;
           }
           if (sh.mode == kCoop && it > 64) __nanosleep(100);
@@ -521,10 +516,7 @@ __global__ void __launch_bounds__(kOcThreads, 1)
         ok_s = ok;
       }
       __syncthreads();
-      if (!ok_s) {
-        oc_leave(sh, (unsigned)G);
-        return;
-      }
+      if (!ok_s) return;
     }
 
     // ---- Stage 2.  Lane j takes interface row 2 cta - 15 + j, so the CTA's
@@ -632,14 +624,9 @@ __global__ void __launch_bounds__(kOcThreads, 1)
     if (oob) atomicOr(sh.status, ST_RANGE);
     if (fin) __syncthreads();  // the next CTA's rows take this one's place
   }
-  if (fin) {
-    if (tid == 0) {
-      __threadfence();
-      sh.bar[2] = 0u;
-      oc_report(sh);
-    }
-  } else if (sh.arrivals > 1 || sh.own_status) {
-    oc_leave(sh, (unsigned)G);
+  if (sh.own_status && (fin || sh.mode == kSolo)) {
+    __syncthreads();
+    if (tid == 0) oc_report(sh);
   }
 }
 

@@ -93,8 +93,8 @@ static int oc_ctas_max() {
 }
 
 // Solve the system on chip if it fits (used = true), else leave it.  xch:
-// onchip_exchange_bytes() of device memory; bar: the solve's three counters,
-// zero between solves; extra_arrival:
+// onchip_exchange_bytes() of device memory; bar: the barrier's counter, zero
+// between solves; extra_arrival:
 // 0, or to exercise the barrier one CTA more awaited than launched, in a
 // cooperative launch (1: it times out) or a chained one (2: every CTA gives
 // up and is done again); report: see OcShared (own_status where given).
@@ -135,8 +135,12 @@ static cudaError_t launch_onchip_raw(int64_t n, const Tin* a, const Tin* b, cons
     cfg.numAttrs = 1;
     e = cudaLaunchKernelEx(&cfg, k_onchip<Ar, Tin>, n, g.mt, g.p, g.G, a, b, c, d, x,
                            reinterpret_cast<T*>(xch), sh, vec16, codes ? 1 : 0);
+    if (e == cudaSuccess) {
+      e = launch_chained(k_onchip_end, 1, 1, 0, s, sh);
+      if (e != cudaSuccess) cudaMemsetAsync(bar, 0, sizeof(unsigned), s);
+    }
   } else {
-    if (g.G == 1) sh.mode = kCoop;  // no barrier, nothing to finish
+    if (g.G == 1) sh.mode = kSolo;  // no barrier, nothing to finish
     auto go = [&](int ctas) {
       return launch_chained(k_onchip<Ar, Tin>, (unsigned)ctas, (unsigned)g.B, smem, s, n, g.mt,
                             g.p, g.G, a, b, c, d, x, reinterpret_cast<T*>(xch), sh, vec16,
@@ -146,6 +150,7 @@ static cudaError_t launch_onchip_raw(int64_t n, const Tin* a, const Tin* b, cons
     if (e == cudaSuccess && g.G > 1) {
       sh.mode = kFinish;
       e = go(1);
+      if (e != cudaSuccess) cudaMemsetAsync(bar, 0, sizeof(unsigned), s);
     }
   }
   if (e == cudaSuccess) used = true;
@@ -160,7 +165,7 @@ static cudaError_t launch_onchip(tps_plan_s* P, int64_t n, const Tin* a, const T
   used = false;
   if (P->desc.flags & TPS_NO_ONCHIP) return cudaSuccess;
   if (P->desc.flags & TPS_EXTERNAL_WORKSPACE) {  // the caller may have used it in between
-    const cudaError_t e = cudaMemsetAsync(P->ws + 32, 0, 3 * sizeof(unsigned), s);
+    const cudaError_t e = cudaMemsetAsync(P->ws + 32, 0, sizeof(unsigned), s);
     if (e != cudaSuccess) return e;
   }
   return launch_onchip_raw<Ar, Tin>(n, a, b, c, d, x, P->ws + P->off_xch,

@@ -110,7 +110,7 @@ struct WsLayout {
 static WsLayout workspace_layout(const tps_plan_s* P, int32_t m, bool rel) {
   WsLayout W = {};
   size_t off = 0;
-  off = align_up(off + 64);  // status word, refinement maxima, grid-barrier counters
+  off = align_up(off + 64);  // status word, refinement maxima, grid-barrier counter
   W.dmax = off;              // per-system range codes (zero between solves)
   off = align_up(off + 4 * kCodes * (size_t)std::max<int64_t>(1, P->desc.batch_max));
   W.xch = off;               // interface rows of the on-chip solve
@@ -329,12 +329,12 @@ tps_status tps_plan(const tps_plan_desc* desc, tps_plan_t* out) {
     P->d_scalars = (double*)(P->ws + 8);
     place(P, P->m, rel);
     e = cudaMemset(P->ws, 0, P->off_xch);  // header and range codes
-    // test switch: the on-chip barrier's counters as two solves on one plan at
-    // once (a misuse) may leave them
+    // test switch: a count at the on-chip barrier, as if left by two solves on
+    // one plan at once (a misuse)
     if (const char* t = std::getenv("TPS_TEST_ONCHIP_RESIDUE")) {
-      const unsigned one[2] = {1u, 1u};
+      const unsigned one = 1u;
       if (t[0] == '1' && e == cudaSuccess)
-        e = cudaMemcpy(P->ws + 32, one, sizeof(one), cudaMemcpyHostToDevice);
+        e = cudaMemcpy(P->ws + 32, &one, sizeof(one), cudaMemcpyHostToDevice);
     }
     if (e != cudaSuccess) {
       tps_plan_destroy(P);

@@ -186,7 +186,7 @@ cudaError_t refine_step(tps_plan_s* P, const std::vector<LevelPlan>& levels, con
 size_t onchip_exchange_bytes();
 // The single-launch on-chip solve of one system if it fits on this device
 // (used = true), else nothing.  xch: onchip_exchange_bytes() of device
-// memory; bar: three device counters, status: a status word, all zero
+// memory; bar: a device counter, status: a status word, both zero
 // between solves; report: the solve's tps_status, or null.
 cudaError_t onchip_solve(int dtype, int64_t n, const void* a, const void* b, const void* c,
                          const void* d, void* x, void* xch, unsigned* bar, int* status,

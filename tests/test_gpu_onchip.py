@@ -184,14 +184,19 @@ def test_ctas_that_gave_up_are_done_again(dtype, n, monkeypatch):
 def test_barrier_that_opened_early(dtype, n, monkeypatch):
     """A count left at the barrier (by two solves on one plan at once, a misuse)
     lets CTAs read interface rows that others are still writing.  That solve
-    is spoiled, but its warps stay together and the context survives."""
+    is spoiled, but its warps stay together, the context survives, and the plan's
+    next solve finds nothing of it."""
     monkeypatch.setenv("TPS_TEST_ONCHIP_RESIDUE", "1")
     plan = binding.Plan(n, dtype=dtype)
     monkeypatch.delenv("TPS_TEST_ONCHIP_RESIDUE")
-    s = synth.system(53, n)
-    tdt = torch.float64
-    if dtype == "f32":
-        s, tdt = synth.to_f32(s), torch.float32
-    for _ in range(3):
-        solve(plan, s, tdt)
-    check(dtype, n, 53, 1)
+    tdt = torch.float32 if dtype == "f32" else torch.float64
+    one = np.ones(n)
+    s = {"a": -one, "b": 2.01 * one, "c": -one.copy()}  # every CTA needs the others' rows
+    rng = np.random.default_rng(n)
+    for k in range(12):
+        s["d"] = rng.uniform(-1, 1, n)
+        x, info = solve(plan, s, tdt)
+        if k > 0:
+            x0, _ = solve(binding.Plan(n, dtype=dtype), s, tdt)
+            assert info["status"] == 0 and info["onchip"] == 1, info
+            assert np.array_equal(x, x0)
