@@ -27,7 +27,7 @@ constexpr int kM0 = 64;           // rows per block at the top level
 constexpr int kMr = 32;           // rows per block at the reduced levels
 constexpr int kMaxLevels = 8;
 constexpr size_t kScratchBytes = size_t(2) << 20;  // 2 MiB per GPU
-constexpr size_t kHeadOnchip = 128;  // the on-chip solve's status word and counter
+constexpr size_t kHeadOnchip = 128;  // the on-chip solve's status word and counters
 
 // The scratch array.  In host code `g_scratch` names a host-side shadow,
 // not device memory: its device address comes from cudaGetSymbolAddress.
@@ -182,14 +182,17 @@ extern "C" tps_status tps_solve_noalloc(int32_t dtype, int64_t n, const void* a,
   // the whole system on chip where it fits, which reports and
   // clears its own status word (its words of the header, kHeadOnchip, are
   // zero between solves; its exchange rows sit where the levels would go);
-  // a test switch (TPS_TEST_NOALLOC_LEVELS=1) keeps the level-by-level route
+  // test switches: TPS_TEST_NOALLOC_LEVELS=1 keeps the level-by-level route,
+  // TPS_TEST_ONCHIP_GIVE_UP as for plans
   bool onchip = false;
   const char* lvl = std::getenv("TPS_TEST_NOALLOC_LEVELS");
   cudaError_t e = cudaSuccess;
   if (!(lvl && lvl[0] == '1')) {
+    const char* gu = std::getenv("TPS_TEST_ONCHIP_GIVE_UP");
+    const int test = gu && (gu[0] == '1' || gu[0] == '2') ? gu[0] - '0' + 1 : 0;
     unsigned* head = reinterpret_cast<unsigned*>(ws + kHeadOnchip);
     e = onchip_solve(dtype, n, a, b, c, d, x, ws + align_up(64), head + 1,
-                     reinterpret_cast<int*>(head), status_out, s, onchip);
+                     reinterpret_cast<int*>(head), status_out, test, s, onchip);
     if (e == cudaSuccess && onchip) return TPS_OK;
     if (e != cudaSuccess && launch_refused(e)) {
       cudaGetLastError();

@@ -93,15 +93,15 @@ static int oc_ctas_max() {
 }
 
 // Solve the system on chip if it fits (used = true), else leave it.  xch:
-// onchip_exchange_bytes() of device memory; bar: the barrier's counter, zero
-// between solves; extra_arrival:
-// 0, or to exercise the barrier one CTA more awaited than launched, in a
-// cooperative launch (1: it times out) or a chained one (2: every CTA gives
-// up and is done again); report: see OcShared (own_status where given).
+// onchip_exchange_bytes() of device memory; bar: the barrier's two counters,
+// the first zero between solves; test: 0, or to exercise the barrier one CTA
+// more awaited than launched, in a cooperative launch (1: it times out) or a
+// chained one (2: every CTA gives up and is done again), or every second CTA
+// giving up (3); report: see OcShared (own_status where given).
 template <class Ar, class Tin>
 static cudaError_t launch_onchip_raw(int64_t n, const Tin* a, const Tin* b, const Tin* c,
                                      const Tin* d, Tin* x, void* xch, unsigned* bar,
-                                     int* status, int extra_arrival, cudaStream_t s,
+                                     int* status, int test, cudaStream_t s,
                                      bool& used, bool codes, bool own_status = false,
                                      int32_t* report = nullptr) {
   used = false;
@@ -115,10 +115,9 @@ static cudaError_t launch_onchip_raw(int64_t n, const Tin* a, const Tin* b, cons
   // against cooperative: fp64 10007 rows 12.1 / 14.3 and 65536 14.7 / 16.4,
   // double-float 800000 19.9 / 20.5, but fp32 1000003 12.7 / 12.3 and as
   // Stage 2 of 256 fp32 systems 115.5 / 113.8 a batch: fp32 stays cooperative.
-  const bool coop = extra_arrival == 1 ||
-                    (std::is_same<Ar, ArF32>::value && g.G > 1 && extra_arrival == 0);
-  OcShared sh{bar, (unsigned)g.G + (extra_arrival ? 1u : 0u), status, report,
-              own_status ? 1 : 0, kFirst};
+  const bool coop = test == 1 || (std::is_same<Ar, ArF32>::value && g.G > 1 && test == 0);
+  OcShared sh{bar, (unsigned)g.G + (test == 1 || test == 2 ? 1u : 0u), status, report,
+              own_status ? 1 : 0, kFirst, test == 3};
   constexpr size_t smem = OcLayout<Ar, Tin>::kBytes;
   cudaError_t e;
   if (coop) {
@@ -149,7 +148,7 @@ static cudaError_t launch_onchip_raw(int64_t n, const Tin* a, const Tin* b, cons
     e = go(g.G);
     if (e == cudaSuccess && g.G > 1) {
       sh.mode = kFinish;
-      e = go(1);
+      e = go(std::min(g.G, kOcFinishCtas));
       if (e != cudaSuccess) cudaMemsetAsync(bar, 0, sizeof(unsigned), s);
     }
   }
@@ -165,12 +164,12 @@ static cudaError_t launch_onchip(tps_plan_s* P, int64_t n, const Tin* a, const T
   used = false;
   if (P->desc.flags & TPS_NO_ONCHIP) return cudaSuccess;
   if (P->desc.flags & TPS_EXTERNAL_WORKSPACE) {  // the caller may have used it in between
-    const cudaError_t e = cudaMemsetAsync(P->ws + 32, 0, sizeof(unsigned), s);
+    const cudaError_t e = cudaMemsetAsync(P->ws + 32, 0, 2 * sizeof(unsigned), s);
     if (e != cudaSuccess) return e;
   }
   return launch_onchip_raw<Ar, Tin>(n, a, b, c, d, x, P->ws + P->off_xch,
                                     reinterpret_cast<unsigned*>(P->ws + 32), P->d_status,
-                                    P->test_barrier_extra, s, used, codes);
+                                    P->test_onchip, s, used, codes);
 }
 
 unsigned* level0_dmax(tps_plan_s* P) {
@@ -756,13 +755,13 @@ tps_status run_truncated(tps_plan_s* P, int64_t n, const void* a, const void* b,
 
 cudaError_t onchip_solve(int dtype, int64_t n, const void* a, const void* b, const void* c,
                          const void* d, void* x, void* xch, unsigned* bar, int* status,
-                         int32_t* report, cudaStream_t s, bool& used) {
+                         int32_t* report, int test, cudaStream_t s, bool& used) {
   return dispatch(dtype, [&](auto ar, auto* tin, auto* tred) -> cudaError_t {
     using Ar = decltype(ar);
     using Tin = std::remove_pointer_t<decltype(tin)>;
     (void)tred;
     return launch_onchip_raw<Ar, Tin>(n, (const Tin*)a, (const Tin*)b, (const Tin*)c,
-                                      (const Tin*)d, (Tin*)x, xch, bar, status, 0, s, used,
+                                      (const Tin*)d, (Tin*)x, xch, bar, status, test, s, used,
                                       dtype == TPS_F64_DF, true, report);
   });
 }

@@ -110,7 +110,7 @@ struct WsLayout {
 static WsLayout workspace_layout(const tps_plan_s* P, int32_t m, bool rel) {
   WsLayout W = {};
   size_t off = 0;
-  off = align_up(off + 64);  // status word, refinement maxima, grid-barrier counter
+  off = align_up(off + 64);  // status word, refinement maxima, grid-barrier counters
   W.dmax = off;              // per-system range codes (zero between solves)
   off = align_up(off + 4 * kCodes * (size_t)std::max<int64_t>(1, P->desc.batch_max));
   W.xch = off;               // interface rows of the on-chip solve
@@ -270,9 +270,9 @@ tps_status tps_plan(const tps_plan_desc* desc, tps_plan_t* out) {
   P->ws_needed = workspace_size(P, P->m, rel);
 
   if (const char* t = std::getenv("TPS_TEST_ONCHIP_TIMEOUT"))
-    P->test_barrier_extra = t[0] == '1' ? 1 : 0;
+    P->test_onchip = t[0] == '1' ? 1 : 0;
   if (const char* t = std::getenv("TPS_TEST_ONCHIP_GIVE_UP"))
-    if (t[0] == '1') P->test_barrier_extra = 2;
+    if (t[0] == '1' || t[0] == '2') P->test_onchip = t[0] - '0' + 1;
   // test switch: the mixed solve's corrections as three separate passes
   // on every route (to compare them with the fused step)
   if (const char* t = std::getenv("TPS_TEST_UNFUSED_REFINE"))

@@ -135,8 +135,9 @@ struct tps_plan_s {
   // test hooks at plan creation: the on-chip solve's grid barrier waits for
   // one CTA more than it launches, so the bounded wait runs out and the solve
   // reports TPS_ERR_TIMEOUT (1, TPS_TEST_ONCHIP_TIMEOUT=1) or does every CTA
-  // again (2, TPS_TEST_ONCHIP_GIVE_UP=1)
-  int test_barrier_extra = 0;
+  // again (2, TPS_TEST_ONCHIP_GIVE_UP=1); or every second CTA's wait runs out
+  // and those are done again (3, TPS_TEST_ONCHIP_GIVE_UP=2)
+  int test_onchip = 0;
   bool test_unfused_refine = false;  // TPS_TEST_UNFUSED_REFINE=1 at plan time
   int32_t last_refine_fused = 0;     // the last mixed solve used refine_step
   // batched work list (device) and its capacity in entries
@@ -186,11 +187,12 @@ cudaError_t refine_step(tps_plan_s* P, const std::vector<LevelPlan>& levels, con
 size_t onchip_exchange_bytes();
 // The single-launch on-chip solve of one system if it fits on this device
 // (used = true), else nothing.  xch: onchip_exchange_bytes() of device
-// memory; bar: a device counter, status: a status word, both zero
-// between solves; report: the solve's tps_status, or null.
+// memory; bar: two device counters, status: a status word, zero between
+// solves; report: the solve's tps_status, or null; test:
+// tps_plan_s::test_onchip.
 cudaError_t onchip_solve(int dtype, int64_t n, const void* a, const void* b, const void* c,
                          const void* d, void* x, void* xch, unsigned* bar, int* status,
-                         int32_t* report, cudaStream_t s, bool& used);
+                         int32_t* report, int test, cudaStream_t s, bool& used);
 // TPS_TRUNCATE: the windowed solve of one device-resident system.
 tps_status run_truncated(tps_plan_s* P, int64_t n, const void* a, const void* b, const void* c,
                          const void* d, void* x, cudaStream_t s);

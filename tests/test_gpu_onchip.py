@@ -200,3 +200,22 @@ def test_barrier_that_opened_early(dtype, n, monkeypatch):
             x0, _ = solve(binding.Plan(n, dtype=dtype), s, tdt)
             assert info["status"] == 0 and info["onchip"] == 1, info
             assert np.array_equal(x, x0)
+
+
+@pytest.mark.parametrize("dtype", ["f64", "f64_df", "f32"])
+@pytest.mark.parametrize("n", [500, 6000, 10007, 100003, 800001])
+def test_some_ctas_gave_up(dtype, n, monkeypatch):
+    """Every second CTA gives up: some rows come from the first launch, some from
+    the second, whose CTAs share them."""
+    monkeypatch.setenv("TPS_TEST_ONCHIP_GIVE_UP", "2")
+    plan = binding.Plan(n, dtype=dtype)
+    monkeypatch.delenv("TPS_TEST_ONCHIP_GIVE_UP")
+    s = synth.system(34 + n, n, kind=synth.KIND_RATIO, ratio=1.1)
+    tdt = torch.float64
+    if dtype == "f32":
+        s, tdt = synth.to_f32(s), torch.float32
+    x0, info0 = solve(binding.Plan(n, dtype=dtype), s, tdt)
+    for _ in range(2):
+        x, info = solve(plan, s, tdt)
+        assert info["status"] == 0 and info["onchip"] == 1, info
+        assert np.array_equal(x, x0)

@@ -88,3 +88,14 @@ def test_noalloc_rejects_sizes_beyond_its_maximum():
     too_big = 262144 + 1
     assert f(0, too_big, p, p, p, p, p, None, None) == 1  # TPS_ERR_INVALID_ARG
     assert f(2, 10, p, p, p, p, p, None, None) == 1       # mixed precision is not served
+
+
+@pytest.mark.parametrize("give_up", ["1", "2"])
+@pytest.mark.parametrize("dtype", ["f64_df", "f64", "f32"])
+def test_noalloc_when_ctas_gave_up(dtype, give_up, monkeypatch):
+    """All or every second CTA's rows come from the second launch, whose CTAs
+    share them; the last of these to finish reports the status."""
+    monkeypatch.setenv("TPS_TEST_ONCHIP_GIVE_UP", give_up)
+    check_two_calls(dtype)
+    monkeypatch.delenv("TPS_TEST_ONCHIP_GIVE_UP")
+    check_two_calls(dtype)
