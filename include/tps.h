@@ -83,6 +83,9 @@ typedef enum {
                          /* row whose |b[i]| is so large against the system    */
                          /* that the residual could suffer, and for an x at or  */
                          /* above 2^101.  TPS_F64 has none of these limits.     */
+                         /* (A pivot whose reciprocal is subnormal, 2^1022 or   */
+                         /* more in TPS_F64, above 2^126 in TPS_F32, is         */
+                         /* reported as TPS_ERR_ZERO_PIVOT.)                    */
 } tps_dtype;
 
 typedef enum {

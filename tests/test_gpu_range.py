@@ -212,6 +212,50 @@ def test_non_finite_x_is_reported_in_every_dtype(dtype):
     assert plan.query()["status_name"] == "TPS_ERR_RANGE"
 
 
+ROUTE_SIZES = {"levels": (binding.NO_ONCHIP, 100003), "onchip": (0, 20011), "one_warp": (0, 60)}
+
+
+@pytest.mark.parametrize("route", ROUTE_SIZES)
+def test_fp64_quotients_over_the_whole_range(route):
+    """Decoupled rows b x = d with b over every exponent, random fractions, powers
+    of two and their neighbours: x is a reciprocal to 2^-52 and one or two
+    roundings away from d / b."""
+    flags, n = ROUTE_SIZES[route]
+    rng = np.random.default_rng(3)
+    frac = rng.uniform(1, 2, n)
+    frac[::3] = 1.0
+    frac[1::9] = 2.0 - 2.0 ** -52
+    frac[2::9] = 1.0 + 2.0 ** -52
+    e = np.linspace(-1022, 1021, n).astype(int)
+    rng.shuffle(e)
+    b = np.ldexp(frac * rng.choice([-1.0, 1.0], n), e)
+    xt = rng.uniform(1, 1.9, n)
+    d = b * xt
+    zero = np.zeros(n)
+    x, info = solve({"a": zero, "b": b, "c": zero, "d": d}, dtype="f64", flags=flags, m=0)
+    assert info["status"] == 0, info
+    assert (np.abs(x - d / b) <= 2.0 ** -51 * np.abs(d / b)).all()
+
+
+@pytest.mark.parametrize("route", ROUTE_SIZES)
+@pytest.mark.parametrize("dtype,big", [("f64", 2.0 ** 1022), ("f64", -1.9 * 2.0 ** 1022),
+                                       ("f64", 1.7e308), ("f32", 1.5 * 2.0 ** 126),
+                                       ("f32", -2.0 ** 127)])
+def test_pivot_with_a_subnormal_reciprocal_is_reported(route, dtype, big):
+    flags, n = ROUTE_SIZES[route]
+    s = synth.system(83, n)
+    tdt = torch.float64
+    if dtype == "f32":
+        s, tdt = synth.to_f32(s), torch.float32
+    s = {k: np.array(s[k], dtype=np.float64) for k in "abcd"}
+    for i in (n // 3, n // 2 + 7):
+        s["b"][i] = s["d"][i] = big  # x = 1 there
+    a, b, c, d = (torch.as_tensor(s[k]).to("cuda", tdt) for k in "abcd")
+    plan = binding.Plan(n, dtype=dtype, flags=flags)
+    plan.solve(a, b, c, d, torch.empty_like(b))
+    assert plan.query()["status_name"] == "TPS_ERR_ZERO_PIVOT"
+
+
 def test_one_warp_solve_range():
     for n in (1, 2, 40, 64):
         s = synth.system(80 + n, n)
