@@ -320,16 +320,19 @@ __device__ __forceinline__ void oc_pcr_small(double& p, double& u, double& v, do
   v = ArF64::neg(ArF64::mul(v, vq));
 }
 
-// a value of 4 or 8 bytes read from L2, past the (non-coherent) L1
+// a value of 4 or 8 bytes that another CTA or kernel wrote, read from L2, past
+// the (non-coherent) L1, where the program says (volatile: not ahead of a wait)
 template <class T>
 __device__ __forceinline__ T ld_l2(const T* p) {
   static_assert(sizeof(T) == 4 || sizeof(T) == 8, "element size");
   T r;
   if constexpr (sizeof(T) == 8) {
-    const unsigned long long v = __ldcg(reinterpret_cast<const unsigned long long*>(p));
+    unsigned long long v;
+    asm volatile("ld.global.cg.u64 %0, [%1];\n" : "=l"(v) : "l"(p) : "memory");
     memcpy(&r, &v, 8);
   } else {
-    const unsigned v = __ldcg(reinterpret_cast<const unsigned*>(p));
+    unsigned v;
+    asm volatile("ld.global.cg.u32 %0, [%1];\n" : "=r"(v) : "l"(p) : "memory");
     memcpy(&r, &v, 4);
   }
   return r;
@@ -395,9 +398,8 @@ static __global__ void k_onchip_end(OcShared sh) {
 // arithmetic).
 template <class Ar, class Tin>
 __global__ void __launch_bounds__(kOcThreads, 1)
-    k_onchip(int64_t n, int mt, int64_t p, int G, const Tin* __restrict__ a,
-             const Tin* __restrict__ b, const Tin* __restrict__ c, const Tin* __restrict__ d,
-             Tin* __restrict__ x, typename Ar::T* __restrict__ xch, OcShared sh, int vec16,
+    k_onchip(int64_t n, int mt, int64_t p, int G, const Tin* a, const Tin* b, const Tin* c,
+             const Tin* d, Tin* __restrict__ x, typename Ar::T* xch, OcShared sh, int vec16,
              int codes) {
   using T = typename Ar::T;
   using Lay = OcLayout<Ar, Tin>;

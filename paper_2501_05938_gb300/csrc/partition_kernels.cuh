@@ -125,6 +125,9 @@ struct Bounds {
 // between two kernels costs about 0.5 us where an ordinary one costs 1.5 us
 // and is then rounded up to the next 2.048 us (measured back to back: 1 us of
 // work a kernel takes 1.5 against 4.1 us, 5 us of work 5.4 against 8.2).
+// The memory such a kernel reads may still change while it runs, which
+// const __restrict__ on a parameter would deny: the compiler could then read it
+// before the wait.  So its inputs are plain pointers.
 __device__ __forceinline__ void chain_wait() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
@@ -477,11 +480,10 @@ constexpr size_t stage1_smem_per_warp() {
 template <class Ar, class Tin, class Tred, int R, int K, int W, bool kVec16, bool kRef = false,
           bool kRel = false>
 __global__ void __launch_bounds__(W * 32)
-    k_stage1(Level lv, const Tin* __restrict__ a, const Tin* __restrict__ b,
-             const Tin* __restrict__ c, const Tin* __restrict__ d, Tred* __restrict__ ra,
-             Tred* __restrict__ rb, Tred* __restrict__ rc, Tred* __restrict__ rd,
-             Tred* __restrict__ ck_gam, Tred* __restrict__ ck_y, Tred* __restrict__ ck_v,
-             int* __restrict__ status, RefineIO rf = {}, RelIO rl = {}) {
+    k_stage1(Level lv, const Tin* a, const Tin* b, const Tin* c, const Tin* d,
+             Tred* __restrict__ ra, Tred* __restrict__ rb, Tred* __restrict__ rc,
+             Tred* __restrict__ rd, Tred* __restrict__ ck_gam, Tred* __restrict__ ck_y,
+             Tred* __restrict__ ck_v, int* __restrict__ status, RefineIO rf = {}, RelIO rl = {}) {
   using T = typename Ar::T;
   using TL = Tile<Tin, R, kRef ? 5 : 4>;
   constexpr bool kSkip = Ar::kSkipChain || kRel;  // decayed chains are skipped
@@ -833,11 +835,9 @@ __global__ void __launch_bounds__(W * 32)
 // result is added to x in place and the maxima go to rf.max2.
 template <class Ar, class Tin, class Tred, int R, int W, bool kVec16, bool kRef = false>
 __global__ void __launch_bounds__(W * 32)
-    k_stage3(Level lv, const Tin* __restrict__ a, const Tin* __restrict__ b,
-             const Tin* __restrict__ c, const Tin* __restrict__ d, const Tred* __restrict__ xred,
-             const Tred* __restrict__ ck_gam, const Tred* __restrict__ ck_y,
-             const Tred* __restrict__ ck_v, Tin* __restrict__ x, int* __restrict__ status,
-             RefineIO rf = {}) {
+    k_stage3(Level lv, const Tin* a, const Tin* b, const Tin* c, const Tin* d, const Tred* xred,
+             const Tred* ck_gam, const Tred* ck_y, const Tred* ck_v, Tin* __restrict__ x,
+             int* __restrict__ status, RefineIO rf = {}) {
   using T = typename Ar::T;
   using TL = Tile<Tin, R, kRef ? 5 : 4>;
   using TL3 = Tile3<Tin, Tred, R, kRef ? 5 : 4>;
@@ -1071,7 +1071,7 @@ struct BackTile {
 };
 template <class Ar, class Tin, class Tred, int R, bool kVec16, bool kRef = false>
 __global__ void __launch_bounds__(32)
-    k_back(Level lv, const Tred* __restrict__ xred, Tin* __restrict__ x, int* __restrict__ status,
+    k_back(Level lv, const Tred* xred, Tin* __restrict__ x, int* __restrict__ status,
            RelIO rl, RefineIO rf) {
   using T = typename Ar::T;
   using TL = Tile<Tin, R, 1>;
@@ -1239,9 +1239,8 @@ constexpr int kBaseMax = 64;
 // per-system range codes, raised here; x is checked for range.
 template <class Ar, class Tin, class Tout>
 __global__ void __launch_bounds__(32)
-    k_base(int64_t n, const Tin* __restrict__ a, const Tin* __restrict__ b,
-           const Tin* __restrict__ c, const Tin* __restrict__ d, Tout* __restrict__ x,
-           const int64_t* __restrict__ bnd, int64_t nbnd, int* __restrict__ status,
+    k_base(int64_t n, const Tin* a, const Tin* b, const Tin* c, const Tin* d,
+           Tout* __restrict__ x, const int64_t* bnd, int64_t nbnd, int* __restrict__ status,
            unsigned* __restrict__ dmax) {
   using T = typename Ar::T;
   __shared__ T sa[kBaseMax], sb[kBaseMax], sc[kBaseMax], sd[kBaseMax];

@@ -1,6 +1,9 @@
 """Host-side logic of libtps, no GPU: the paper's stream rule (Eq. 4, 6, 7)
 against Table 4, and the host MLP forward pass against the fp64 oracle."""
 import ctypes
+import glob
+import os
+import re
 
 import numpy as np
 import pytest
@@ -56,3 +59,19 @@ def test_host_forward_matches_fp64_oracle(lib):
         pf = {k: v.astype(np.float32).astype(np.float64) for k, v in p.items()}
         ref, _ = mlp.forward(pf, x.astype(np.float64)[None, :])
         np.testing.assert_allclose(y, ref[0], rtol=1e-4, atol=1e-5)
+
+
+def test_chained_kernels_do_not_promise_read_only_inputs():
+    """A kernel that starts before the one that writes its inputs has ended
+    (chain_wait) must not declare them const __restrict__, which lets the
+    compiler read them ahead of the wait."""
+    src = os.path.join(os.path.dirname(tps_build.__file__), "csrc")
+    seen = set()
+    for path in glob.glob(os.path.join(src, "*.cu*")):
+        text = open(path).read()
+        for m in re.finditer(r"__global__[^;{]*?\b(k_\w+)\(", text):
+            body = text[m.end():text.find("\n}", m.end())]
+            if "chain_wait()" in body:
+                seen.add(m.group(1))
+                assert not re.search(r"const\s+\w+\s*\*\s*__restrict__", body), m.group(1)
+    assert {"k_stage1", "k_stage3", "k_back", "k_base", "k_onchip", "k_dcode_check"} <= seen
