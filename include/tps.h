@@ -206,8 +206,10 @@ tps_status tps_set_workspace(tps_plan_t plan, void* dev_ptr, size_t bytes);
  *
  * Larger systems run level by level.  Up to 2^30 rows the workspace holds a
  * relation per row (24 bytes, fp32 12), from which Stage 3 recovers x without
- * reading a, b, c, d again; for more rows, or where tps_plan cannot allocate
- * that much, it repeats the elimination from checkpoints (1.2 bytes a row).
+ * reading a, b, c, d again; for more rows, or where that would take more than
+ * half of the memory that is free when tps_plan is called, it repeats the
+ * elimination from checkpoints (1.2 bytes a row).  A device plan all of whose
+ * systems fit on chip holds no relations either.
  * Terms that decay along a block are left out once they are 0 in the
  * arithmetic, with one exception: TPS_F64 leaves out of a block's first
  * unknown what would reach it from below in the same block through a product

@@ -753,6 +753,20 @@ tps_status run_truncated(tps_plan_s* P, int64_t n, const void* a, const void* b,
 }
 
 
+bool onchip_fits(int dtype, int64_t n) {
+  OcGeom g;
+  bool fits = n <= kBaseMax;
+  if (!fits)
+    dispatch(dtype, [&](auto ar, auto* tin, auto* tred) -> cudaError_t {
+      using Ar = decltype(ar);
+      using Tin = std::remove_pointer_t<decltype(tin)>;
+      (void)tred;
+      fits = oc_geometry<Ar, Tin>(n, oc_ctas_max<Ar, Tin>(), g);
+      return cudaSuccess;
+    });
+  return fits;
+}
+
 cudaError_t onchip_solve(int dtype, int64_t n, const void* a, const void* b, const void* c,
                          const void* d, void* x, void* xch, unsigned* bar, int* status,
                          int32_t* report, int test, cudaStream_t s, bool& used) {

@@ -150,6 +150,32 @@ static size_t workspace_size(const tps_plan_s* P, int32_t m, bool rel) {
   return v;
 }
 
+// Does the plan's own workspace hold relations?  Not where no solve of the plan
+// goes level by level (windows; every size on chip), nor above kRelRowsMax rows
+// (25 GB), nor where they would take more than half of the memory that is free:
+// that may be meant for the caller's arrays, and checkpoints need 1.2 bytes a row.
+static bool wants_relations(const tps_plan_s* P) {
+  const tps_plan_desc& d = P->desc;
+  if (const char* t = std::getenv("TPS_TEST_CHECKPOINTS"))  // test switch
+    if (t[0] == '1') return false;
+  if (d.n_max > kRelRowsMax || (d.flags & (TPS_EXTERNAL_WORKSPACE | TPS_TRUNCATE))) return false;
+  if (d.residency == TPS_DEVICE && !(d.flags & TPS_NO_ONCHIP) && d.batch_max <= 1 &&
+      onchip_fits(d.dtype, d.n_max))
+    return false;
+  size_t more = workspace_size(P, P->m, true);
+  more -= std::min(more, workspace_size(P, P->m, false));
+  if (d.flags & TPS_HOST_OVERLAP) more *= 2;  // the twin's
+  if (more < ((size_t)64 << 20)) return true;
+  size_t free_bytes = 0, total = 0;
+  if (cudaMemGetInfo(&free_bytes, &total) != cudaSuccess) {
+    cudaGetLastError();
+    return true;  // the allocation decides
+  }
+  if (const char* t = std::getenv("TPS_TEST_FREE_BYTES"))  // test switch
+    free_bytes = std::min(free_bytes, (size_t)std::strtoull(t, nullptr, 10));
+  return more <= free_bytes / 2;
+}
+
 // The plan takes block size m, with or without relations.
 static void place(tps_plan_s* P, int32_t m, bool rel) {
   const WsLayout W = workspace_layout(P, m, rel);
@@ -259,13 +285,8 @@ tps_status tps_plan(const tps_plan_desc* desc, tps_plan_t* out) {
   }
   default_params(d, P->m, P->m_reduced, P->streams);
 
-  // relations: up to kRelRowsMax rows (25 GB of workspace); above, and where
-  // that much memory is not free, Stage 3 works from checkpoints
-  // (a caller's workspace: if it is large enough, see tps_set_workspace)
-  bool rel = d.n_max <= kRelRowsMax && !(d.flags & TPS_EXTERNAL_WORKSPACE);
-  // test switch: checkpoints at any size
-  if (const char* t = std::getenv("TPS_TEST_CHECKPOINTS"))
-    if (t[0] == '1') rel = false;
+  // a caller's workspace decides in tps_set_workspace
+  bool rel = wants_relations(P);
   P->m_plan = P->m;
   P->ws_needed = workspace_size(P, P->m, rel);
 

@@ -185,7 +185,9 @@ cudaError_t refine_step(tps_plan_s* P, const std::vector<LevelPlan>& levels, con
                         unsigned long long* max2, cudaStream_t s);
 // Bytes of the on-chip solve's exchange rows (part of every plan workspace).
 size_t onchip_exchange_bytes();
-// The single-launch on-chip solve of one system if it fits on this device
+// Does one system of n rows (and so any smaller one) fit on chip, or one warp?
+bool onchip_fits(int dtype, int64_t n);
+// The on-chip solve of one system if it fits on this device
 // (used = true), else nothing.  xch: onchip_exchange_bytes() of device
 // memory; bar: two device counters, status: a status word, zero between
 // solves; report: the solve's tps_status, or null; test:

@@ -766,3 +766,24 @@ def test_workspace_of_the_size_asked_for_after_autotune(dtype):
     assert bool((buf[least:] == 0xA5).all())
     ref = oracle.thomas(s["a"], s["b"], s["c"], s["d"])
     assert oracle.rel_forward_error(x.cpu().numpy(), ref) <= F64_FWD
+
+
+def test_relations_are_held_only_where_they_are_used(monkeypatch):
+    """24 bytes a row: not in a plan whose systems all run on chip, nor where they
+    would take more than half of the free memory."""
+    row = lambda n, **kw: binding.Plan(n, **kw).workspace_size() / n
+    n = 500000
+    for dtype, bytes_a_row in (("f64", 24), ("f64_df", 24), ("f32", 12)):
+        assert row(n, dtype=dtype) < 8
+        assert row(n, dtype=dtype, batch_max=4) > bytes_a_row
+        assert row(n, dtype=dtype, flags=binding.NO_ONCHIP) > bytes_a_row
+    n = 6000011
+    assert row(n) > 24
+    monkeypatch.setenv("TPS_TEST_FREE_BYTES", str(n * 40))
+    assert row(n) < 8
+    plan = binding.Plan(n)
+    monkeypatch.delenv("TPS_TEST_FREE_BYTES")
+    s = synth.system(45, n)
+    x, info = run(plan, s)
+    assert info["status"] == 0
+    assert oracle.rel_forward_error(x, oracle.thomas(*(s[k] for k in "abcd"))) <= F64_FWD
