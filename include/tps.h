@@ -168,12 +168,16 @@ tps_status tps_plan_destroy(tps_plan_t plan);
 /* Device workspace the plan needs for n_max / batch_max, in bytes. */
 tps_status tps_workspace_size(tps_plan_t plan, size_t* bytes);
 
+/* The same with the relations (see tps_solve), which make larger solves
+ * faster: what a TPS_EXTERNAL_WORKSPACE buffer needs for them (not less than
+ * tps_workspace_size). */
+tps_status tps_workspace_size_relations(tps_plan_t plan, size_t* bytes);
+
 /* Hand the plan a caller-owned device buffer of at least
  * tps_workspace_size bytes (256-byte aligned).  Only for plans created with
- * TPS_EXTERNAL_WORKSPACE; the buffer must outlive every solve.  One that
- * also holds the relations (see tps_solve; 27 bytes a row of n_max and 1 MiB
- * more than tps_workspace_size, fp32 and mixed 14) makes larger solves
- * faster; with less the plan works from checkpoints. */
+ * TPS_EXTERNAL_WORKSPACE; the buffer must outlive every solve.  With
+ * tps_workspace_size_relations bytes the plan uses relations, with less it
+ * works from checkpoints. */
 tps_status tps_set_workspace(tps_plan_t plan, void* dev_ptr, size_t bytes);
 
 /* Solve one system of n <= n_max rows held in device memory (Sec. 2.2,

@@ -24,8 +24,8 @@ TRUNCATE = 128
 HOST_OVERLAP = 256
 
 # every symbol include/tps.h declares
-EXPORTS = ("tps_plan", "tps_plan_destroy", "tps_workspace_size", "tps_set_workspace", "tps_solve",
-           "tps_solve_batched", "tps_solve_host_async", "tps_solve_host_many_async",
+EXPORTS = ("tps_plan", "tps_plan_destroy", "tps_workspace_size", "tps_workspace_size_relations",
+           "tps_set_workspace", "tps_solve", "tps_solve_batched", "tps_solve_host_async", "tps_solve_host_many_async",
            "tps_plan_query", "tps_status_string", "tps_version", "tps_measure_fp64_rates")
 
 
@@ -69,6 +69,7 @@ def lib():
         L.tps_plan.argtypes = [ctypes.POINTER(PlanDesc), ctypes.POINTER(P)]
         L.tps_plan_destroy.argtypes = [P]
         L.tps_workspace_size.argtypes = [P, ctypes.POINTER(ctypes.c_size_t)]
+        L.tps_workspace_size_relations.argtypes = [P, ctypes.POINTER(ctypes.c_size_t)]
         L.tps_set_workspace.argtypes = [P, P, ctypes.c_size_t]
         L.tps_solve.argtypes = [P, I64, P, P, P, P, P, P]
         L.tps_solve_batched.argtypes = [P, I64, P, P, P, P, P, P, P, P]
@@ -143,6 +144,12 @@ class Plan:
     def workspace_size(self):
         v = ctypes.c_size_t()
         check(lib().tps_workspace_size(self._h, ctypes.byref(v)), "tps_workspace_size")
+        return v.value
+
+    def workspace_size_relations(self):
+        v = ctypes.c_size_t()
+        check(lib().tps_workspace_size_relations(self._h, ctypes.byref(v)),
+              "tps_workspace_size_relations")
         return v.value
 
     def set_workspace(self, buf):

@@ -150,18 +150,25 @@ static size_t workspace_size(const tps_plan_s* P, int32_t m, bool rel) {
   return v;
 }
 
-// Does the plan's own workspace hold relations?  Not where no solve of the plan
-// goes level by level (windows; every size on chip), nor above kRelRowsMax rows
-// (25 GB), nor where they would take more than half of the memory that is free:
-// that may be meant for the caller's arrays, and checkpoints need 1.2 bytes a row.
-static bool wants_relations(const tps_plan_s* P) {
+// Does the plan use relations where there is room for them?  Not where none of
+// its solves goes level by level (windows; every size on chip), nor above
+// kRelRowsMax rows (25 GB).
+static bool uses_relations(const tps_plan_s* P) {
+  const tps_plan_desc& d = P->desc;
+  if (d.n_max > kRelRowsMax || (d.flags & TPS_TRUNCATE)) return false;
+  return d.residency != TPS_DEVICE || (d.flags & TPS_NO_ONCHIP) || d.batch_max > 1 ||
+         !onchip_fits(d.dtype, d.n_max);
+}
+
+// Does the plan's own workspace hold them?  Not where they would take more than
+// half of the memory that is free: that may be meant for the caller's arrays,
+// and checkpoints need 1.2 bytes a row.  (A caller's workspace decides in
+// tps_set_workspace.)
+static bool holds_relations(const tps_plan_s* P) {
   const tps_plan_desc& d = P->desc;
   if (const char* t = std::getenv("TPS_TEST_CHECKPOINTS"))  // test switch
     if (t[0] == '1') return false;
-  if (d.n_max > kRelRowsMax || (d.flags & (TPS_EXTERNAL_WORKSPACE | TPS_TRUNCATE))) return false;
-  if (d.residency == TPS_DEVICE && !(d.flags & TPS_NO_ONCHIP) && d.batch_max <= 1 &&
-      onchip_fits(d.dtype, d.n_max))
-    return false;
+  if ((d.flags & TPS_EXTERNAL_WORKSPACE) || !uses_relations(P)) return false;
   size_t more = workspace_size(P, P->m, true);
   more -= std::min(more, workspace_size(P, P->m, false));
   if (d.flags & TPS_HOST_OVERLAP) more *= 2;  // the twin's
@@ -285,8 +292,7 @@ tps_status tps_plan(const tps_plan_desc* desc, tps_plan_t* out) {
   }
   default_params(d, P->m, P->m_reduced, P->streams);
 
-  // a caller's workspace decides in tps_set_workspace
-  bool rel = wants_relations(P);
+  bool rel = holds_relations(P);
   P->m_plan = P->m;
   P->ws_needed = workspace_size(P, P->m, rel);
 
@@ -428,6 +434,13 @@ tps_status tps_workspace_size(tps_plan_t P, size_t* bytes) {
   return TPS_OK;
 }
 
+tps_status tps_workspace_size_relations(tps_plan_t P, size_t* bytes) {
+  if (!P || !bytes) return TPS_ERR_INVALID_ARG;
+  *bytes = P->ws_needed;
+  if (uses_relations(P)) *bytes = std::max(*bytes, workspace_size(P, P->m, true));
+  return TPS_OK;
+}
+
 tps_status tps_set_workspace(tps_plan_t P, void* dev_ptr, size_t bytes) {
   if (!P || !dev_ptr) return TPS_ERR_INVALID_ARG;
   if (!(P->desc.flags & TPS_EXTERNAL_WORKSPACE)) return TPS_ERR_INVALID_ARG;
@@ -437,7 +450,7 @@ tps_status tps_set_workspace(tps_plan_t P, void* dev_ptr, size_t bytes) {
   // with relations if the buffer holds them; a block size that tps_autotune
   // chose on a larger buffer and that needs more than this one goes back to the
   // plan's, for which ws_needed suffices
-  const bool rel = P->desc.n_max <= kRelRowsMax && workspace_size(P, P->m, true) <= bytes;
+  const bool rel = uses_relations(P) && workspace_size(P, P->m, true) <= bytes;
   place(P, rel || workspace_size(P, P->m, false) <= bytes ? P->m : P->m_plan, rel);
   P->ws = (unsigned char*)dev_ptr;
   P->ws_bytes = bytes;

@@ -787,3 +787,38 @@ def test_relations_are_held_only_where_they_are_used(monkeypatch):
     x, info = run(plan, s)
     assert info["status"] == 0
     assert oracle.rel_forward_error(x, oracle.thomas(*(s[k] for k in "abcd"))) <= F64_FWD
+
+
+@pytest.mark.parametrize("dtype", ["f64", "f64_df", "f32", "mixed"])
+@pytest.mark.parametrize("m,mr", [(0, 0), (4, 0), (5, 4), (10, 0), (250, 0)])
+def test_external_workspace_gets_relations_by_asking(dtype, m, mr):
+    """tps_workspace_size_relations is exactly what they take: with it the answer
+    is, to the bit, that of a plan that allocated its own, with less (checkpoints)
+    it is right as well."""
+    n = 300007
+    s = synth.system(49, n)
+    tdt = torch.float64
+    if dtype == "f32":
+        s, tdt = synth.to_f32(s), torch.float32
+    a, b, c, d = (dev(s[k], tdt) for k in "abcd")
+    xs = []
+    own = binding.Plan(n, dtype=dtype, m=m, m_reduced=mr, flags=binding.NO_ONCHIP)
+    plan = binding.Plan(n, dtype=dtype, m=m, m_reduced=mr,
+                        flags=binding.NO_ONCHIP | binding.EXTERNAL_WORKSPACE)
+    least, most = plan.workspace_size(), plan.workspace_size_relations()
+    assert least < most == own.workspace_size() == own.workspace_size_relations()
+    buf = torch.empty(most, dtype=torch.uint8, device="cuda")
+    for p, size in ((own, 0), (plan, most), (plan, most - 1)):
+        if size:
+            p.set_workspace(buf[:size])
+        x = torch.full_like(b, float("nan"))
+        p.solve(a, b, c, d, x)
+        torch.cuda.synchronize()
+        assert p.query()["status"] == 0
+        xs.append(x)
+    assert torch.equal(xs[0], xs[1])
+    assert dtype == "mixed" or not torch.equal(xs[0], xs[2])
+    ref = oracle.thomas(*(np.asarray(s[k], dtype=np.float64) for k in "abcd"))
+    for x in xs:
+        err = oracle.rel_forward_error(x.double().cpu().numpy(), ref)
+        assert err <= (F32_FWD if dtype == "f32" else F64_FWD)
