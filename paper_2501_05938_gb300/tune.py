@@ -212,7 +212,8 @@ def target(best):
 def pick(recs):
     """The configuration to learn at a point: the fastest one, or of the block
     sizes within 1% of it the nearest to the one that gives 6.4 warps of 32
-    blocks an SM (16 to 128 rows).  (Systems solved on chip run the same with
+    blocks an SM (16 to 128 rows; tps_plan's own rule, which the grid does not
+    hold, aims at eight).  (Systems solved on chip run the same with
     every block size, and neighbouring ones often differ by less than the
     timing noise, which the network would otherwise learn.)"""
     best = min(recs, key=lambda r: r["ms"])
@@ -222,11 +223,16 @@ def pick(recs):
     return min(ties, key=lambda r: (abs(math.log2(r["m"]) - centre), r["ms"]))
 
 
-def dataset(rows, train=True):
+def training_points(rows):
+    """Points to train on, and every fourth of them, on which choose_seed compares
+    the seeds: the held-out points take no part in any choice."""
+    pts = [(k, r) for k, r in sorted(points(rows).items()) if not held_out(r[0])]
+    return pts, pts[1::4]
+
+
+def dataset(pts):
     X, T, keys = [], [], []
-    for key, recs in sorted(points(rows).items()):
-        if held_out(recs[0]) == train:
-            continue
+    for key, recs in pts:
         best = pick(recs)
         X.append(features(key[1], key[2], key[3], key[4]))
         T.append(target(best))
@@ -262,11 +268,25 @@ def init_params(seed=0):
     return np.concatenate(parts).astype(np.float32)
 
 
-def train(rows, out_path, steps=4000, lr=3e-3, seed=2, log=print):
+def choose_seed(rows, out_dir, seeds=range(6), log=print, **kw):
+    """The seed whose network, trained without the validation points, has the
+    smallest mean regret on them."""
+    pts, val = training_points(rows)
+    rest = [p for p in pts if p not in val]
+    w = os.path.join(out_dir, "weights_validation.bin")
+    mean = {}
+    for seed in seeds:
+        train(rows, w, seed=seed, log=lambda *_: None, pts=rest, **kw)
+        mean[seed] = evaluate(rows, w, val)[0]["mlp"]["mean"]
+        log(f"seed {seed} validation regret {mean[seed]:.5f}")
+    os.remove(w)
+    return min(mean, key=mean.get)
+
+
+def train(rows, out_path, steps=4000, lr=3e-3, seed=0, log=print, pts=None):
     import torch
 
-    # seed 2: of six equally good on the training points, the best held out
-    X, T, _ = dataset(rows, train=True)
+    X, T, _ = dataset(training_points(rows)[0] if pts is None else pts)
     fmean = X.mean(axis=0)
     fstd = X.std(axis=0)
     fscale = np.where(fstd > 0, 1.0 / np.where(fstd > 0, fstd, 1.0), 1.0)
@@ -412,7 +432,8 @@ def default_params(n, residency):
     return m, (4 if residency else 1), 0
 
 
-def evaluate(rows, weights_path):
+def evaluate(rows, weights_path, pts=None):
+    """Regret on the held-out points, or on `pts`."""
     L = binding.lib()
     L.tps_predict_load.argtypes = [ctypes.c_char_p]
     if L.tps_predict_load(weights_path.encode()) != 0:
@@ -420,9 +441,9 @@ def evaluate(rows, weights_path):
     coeffs = paper_rule_coeffs(rows)
     res = {"mlp": [], "paper_rule": [], "defaults": []}
     detail = []
-    for key, recs in sorted(points(rows).items()):
-        if not held_out(recs[0]):
-            continue
+    if pts is None:
+        pts = [(k, r) for k, r in sorted(points(rows).items()) if held_out(r[0])]
+    for key, recs in pts:
         kind, n, batch, dt, resid = key
         tbest = min(r["ms"] for r in recs)
         pm, pS, pc = _predict(dict(n_max=n, batch_max=batch if batch > 1 else 0,
@@ -596,7 +617,7 @@ def main(argv):
         collect(csv_path)
     rows = load(csv_path)
     if cmd in ("train", "all"):
-        hist = train(rows, w_path)
+        hist = train(rows, w_path, seed=choose_seed(rows, out))
         with open(os.path.join(out, "train_log.json"), "w") as f:
             json.dump(hist, f)
     if cmd in ("evaluate", "all"):

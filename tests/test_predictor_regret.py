@@ -36,3 +36,12 @@ def test_held_out_points_cover_every_kind(result):
     _, detail, _ = result
     kinds = {(d["kind"], d["dtype"]) for d in detail}
     assert {("device", 0), ("device", 1), ("host", 0), ("host", 1), ("batched", 0)} <= kinds
+
+
+def test_no_choice_is_made_on_the_held_out_points():
+    """Neither the network nor its seed: both come from the other points, and the
+    seed's own (validation) are kept from the networks that are compared."""
+    rows = tune.load(os.path.join(PRED, "timings_gb300.csv"))
+    pts, val = tune.training_points(rows)
+    assert len(val) >= 15 and all(p in pts for p in val)
+    assert not any(tune.held_out(r) for _, recs in pts for r in recs)
