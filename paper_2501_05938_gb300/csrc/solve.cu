@@ -185,6 +185,9 @@ cudaError_t dcode_check(tps_plan_s* P, int64_t count, cudaStream_t s) {
 }
 
 Level make_level(int64_t n, int m, int R) {
+  // a block longer than the system ends with its last chunk (m identity rows
+  // would be swept, one after the other)
+  m = (int)std::min<int64_t>(m, (n + R - 1) / R * R);
   Level lv{};
   lv.n = n;
   lv.m = m;
@@ -218,7 +221,7 @@ size_t build_levels(int64_t n, int m0, int mr, size_t top_elem, size_t red_elem,
     }
     L.rel = rel;
     if (rel) {
-      const size_t rows = (size_t)L.lv.p * (size_t)rel_cap(m);
+      const size_t rows = (size_t)L.lv.p * (size_t)rel_cap(L.lv.m);
       L.off_rel[0] = off;
       off = align_up(off + 2 * rows * red_elem);
       L.off_rel[1] = off;

@@ -59,9 +59,9 @@ struct LevelPlan {
   size_t off_rel[3];  // relation rows, al, na
 };
 
-// Block geometry for n rows and nominal block length m (m >= 2, n > m is
-// not required): p = ceil(n/m) blocks, the last one filled up to m rows with
-// identity rows (see partition_kernels.cuh).
+// Block geometry for n rows and nominal block length m >= 2: p = ceil(n/m)
+// blocks, the last one filled up to m rows with identity rows (see
+// partition_kernels.cuh).  R: chunk rows.
 // Argument checks shared by the entry points: managed memory or device
 // memory of `device`, aligned to `align`; the plan's device is current.
 bool device_ptr_ok(const void* p, size_t align, int device);

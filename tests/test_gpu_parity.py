@@ -822,3 +822,20 @@ def test_external_workspace_gets_relations_by_asking(dtype, m, mr):
     for x in xs:
         err = oracle.rel_forward_error(x.double().cpu().numpy(), ref)
         assert err <= (F32_FWD if dtype == "f32" else F64_FWD)
+
+
+@pytest.mark.parametrize("dtype", ["f64", "f64_df", "f32"])
+@pytest.mark.parametrize("n", [65, 1000, 20011])
+def test_block_longer_than_the_system(dtype, n):
+    """One block of n rows, not of m: neither swept nor held in the workspace."""
+    s = synth.system(46, n)
+    tdt = torch.float64
+    if dtype == "f32":
+        s, tdt = synth.to_f32(s), torch.float32
+    plan = binding.Plan(n, dtype=dtype, m=1 << 20, flags=binding.NO_ONCHIP)
+    assert plan.workspace_size() < (64 << 10) + 64 * n
+    x, info = run(plan, s, tdt)
+    assert info["status"] == 0 and info["m"] == 1 << 20
+    a, b, c, d = (np.asarray(s[k], dtype=np.float64) for k in "abcd")
+    assert oracle.rel_forward_error(x, oracle.thomas(a, b, c, d)) <= (
+        F32_FWD if dtype == "f32" else F64_FWD)
