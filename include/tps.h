@@ -10,10 +10,9 @@
  *   Stage 3  per block: recover the interior unknowns from the interface
  *            values.
  * Here all three stages run on the GPU; Stage 2 applies the same method
- * recursively until the reduced system fits in shared memory (one
- * cooperative launch finishes it) or in one warp (parallel cyclic
- * reduction).  The
- * host-resident pipeline (Sec. 2.2, Eq. 2) overlaps chunked host-to-device
+ * recursively until the reduced system fits in shared memory (one pass of
+ * the on-chip solve finishes it) or in one warp (parallel cyclic reduction).
+ * The host-resident pipeline (Sec. 2.2, Eq. 2) overlaps chunked host-to-device
  * copies, kernels and device-to-host copies on S CUDA streams, S a power of
  * two up to 32 (Sec. 2.1).
  *
@@ -199,12 +198,12 @@ tps_status tps_set_workspace(tps_plan_t plan, void* dev_ptr, size_t bytes);
  * fp64 and double-float, ~1.8 M in fp32 on 152 SMs; not for packed batches)
  * is solved in one pass that reads a, b, c, d once and writes x once: each
  * CTA eliminates its rows on chip, one grid barrier, every CTA solves for
- * its own interface rows, and recovers its rows on chip.  The reduced system of a larger solve takes the same path
- * once it fits.  TPS_NO_ONCHIP keeps every level on separate launches.
+ * its own interface rows, and recovers its rows on chip.  The reduced system
+ * of a larger solve takes the same path once it fits.  TPS_NO_ONCHIP keeps every level on separate launches.
  * The grid barrier waits a bounded time for CTAs that are not resident
  * (another such solve on another stream, or other long-running work holding
- * the SMs).  In fp64 and double-float a second launch then does the rows of
- * the CTAs that gave up.  In fp32 the launch is cooperative, so the CTAs are
+ * the SMs); a second launch then does the rows of the CTAs that gave up.  As
+ * Stage 2 of an fp32 solve the launch is cooperative instead, so the CTAs are
  * resident together; should the wait end all the same, the solve reports
  * TPS_ERR_TIMEOUT through tps_plan_query and the context stays usable.
  *
@@ -212,7 +211,7 @@ tps_status tps_set_workspace(tps_plan_t plan, void* dev_ptr, size_t bytes);
  * relation per row (24 bytes, fp32 12), from which Stage 3 recovers x without
  * reading a, b, c, d again; for more rows, or where that would take more than
  * half of the memory that is free when tps_plan is called, it repeats the
- * elimination from checkpoints (1.2 bytes a row).  A device plan all of whose
+ * elimination from checkpoints (about 3.5 bytes a row, fp32 1).  A device plan all of whose
  * systems fit on chip holds no relations either.
  * Terms that decay along a block are left out once they are 0 in the
  * arithmetic, with one exception: TPS_F64 leaves out of a block's first
@@ -224,9 +223,8 @@ tps_status tps_set_workspace(tps_plan_t plan, void* dev_ptr, size_t bytes);
  * corrections until ||delta||/||x|| <= tol or max_iters.  Where the system
  * is solved level by level, each correction is one fused pass of the
  * partition method: Stage 1 forms r = d - A x in fp64 from the rows and the
- * current x, Stage 3 adds the fp32 solution of
- * A delta = r to x in place (tps_info.refine_fused = 1); the
- * on-chip route keeps a separate residual pass, solve and update pass.
+ * current x, Stage 3 adds the fp32 solution of A delta = r to x in place
+ * (tps_info.refine_fused = 1); the on-chip route keeps a separate residual pass, solve and update pass.
  *
  * TPS_TRUNCATE (device plans, fp64 / double-float / fp32; not the paper's
  * method, an approximation for strongly dominant systems): windows of m kept
@@ -244,10 +242,7 @@ tps_status tps_set_workspace(tps_plan_t plan, void* dev_ptr, size_t bytes);
  * its dominance factor q and smallest |b|: (|a_cut| q^h + |c_cut| q^h) /
  * ((1 - q) min|b|) relative to max|x|; tps_plan_query reports the largest
  * bound of the last solve in last_correction and TPS_ERR_NO_CONVERGENCE if
- * it exceeds tol (default 1e-12).
- * The barrier waits a bounded time; if it runs out (which needs CTAs that
- * are not co-resident) the solve stops and tps_plan_query reports
- * TPS_ERR_TIMEOUT. */
+ * it exceeds tol (default 1e-12). */
 tps_status tps_solve(tps_plan_t plan, int64_t n, const void* a, const void* b, const void* c,
                      const void* d, void* x, void* stream);
 
@@ -294,8 +289,8 @@ tps_status tps_solve_host_async(tps_plan_t plan, int64_t n, const void* a, const
  * its x can leave before all of its rows have arrived (Stage 2 couples
  * them).
  *   plan        made with residency TPS_HOST_PINNED and TPS_HOST_OVERLAP
- *               (which implies TPS_NO_ONCHIP: two on-chip cooperative launches
- *               of different systems may not run at once; not with
+ *               (which implies TPS_NO_ONCHIP: the on-chip solves of two systems
+ *               would wait for each other's SMs; not with
  *               TPS_EXTERNAL_WORKSPACE); the twin follows the plan's m,
  *               m_reduced, S and chunk, including tps_autotune's choice
  *   n           rows of every system, 0 .. n_max

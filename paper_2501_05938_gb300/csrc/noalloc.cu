@@ -146,9 +146,8 @@ cudaError_t run(unsigned char* ws, const Layout& L, int idx, int64_t n, const Ti
 // Translate the status bits into a tps_status for the caller's output.
 __global__ void k_report(const int* st, int32_t* out) { *out = status_code(*st); }
 
-// A cooperative launch (fp32) the device refuses for its size or resources
-// (fewer SMs than the cached occupancy assumed, e.g. under an SM partition):
-// the level-by-level route serves instead.
+// A launch the device refuses for its resources: the level-by-level route serves
+// instead.
 bool launch_refused(cudaError_t e) {
   return e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorLaunchOutOfResources ||
          e == cudaErrorInvalidConfiguration;

@@ -97,12 +97,13 @@ static int oc_ctas_max() {
 // the first zero between solves; test: 0, or to exercise the barrier one CTA
 // more awaited than launched, in a cooperative launch (1: it times out) or a
 // chained one (2: every CTA gives up and is done again), or every second CTA
-// giving up (3); report: see OcShared (own_status where given).
+// giving up (3); nested: this is another solve's Stage 2; report: see OcShared
+// (own_status where given).
 template <class Ar, class Tin>
 static cudaError_t launch_onchip_raw(int64_t n, const Tin* a, const Tin* b, const Tin* c,
                                      const Tin* d, Tin* x, void* xch, unsigned* bar,
-                                     int* status, int test, cudaStream_t s,
-                                     bool& used, bool codes, bool own_status = false,
+                                     int* status, int test, cudaStream_t s, bool& used,
+                                     bool codes, bool nested, bool own_status = false,
                                      int32_t* report = nullptr) {
   used = false;
   OcGeom g;
@@ -110,12 +111,14 @@ static cudaError_t launch_onchip_raw(int64_t n, const Tin* a, const Tin* b, cons
   using T = typename Ar::T;
   const uintptr_t al = (uintptr_t)a | (uintptr_t)b | (uintptr_t)c | (uintptr_t)d | (uintptr_t)x;
   const int vec16 = (al % 16) == 0;
-  // Two chained launches or one cooperative one: the chained pair starts sooner
-  // but has a boundary more.  Measured back to back, us a solve, chained
-  // against cooperative: fp64 10007 rows 12.1 / 14.3 and 65536 14.7 / 16.4,
-  // double-float 800000 19.9 / 20.5, but fp32 1000003 12.7 / 12.3 and as
-  // Stage 2 of 256 fp32 systems 115.5 / 113.8 a batch: fp32 stays cooperative.
-  const bool coop = test == 1 || (std::is_same<Ar, ArF32>::value && g.G > 1 && test == 0);
+  // Two chained launches, or a cooperative one and k_onchip_end: the pair starts
+  // sooner, the cooperative launch is short of the look at who gave up.  Measured
+  // back to back, us a solve, pair against cooperative: fp64 10007 rows 12.3 /
+  // 14.3 and 65536 14.4 / 15.4, double-float 800000 19.2 / 20.5 and as Stage 2 of
+  // 3000017 rows 59.9 / 61.5, fp32 1000003 11.2 / 12.3, but as Stage 2 of 256
+  // fp32 systems 56.4 / 55.7: fp32 is cooperative there.
+  const bool coop =
+      test == 1 || (std::is_same<Ar, ArF32>::value && nested && g.G > 1 && test == 0);
   OcShared sh{bar, (unsigned)g.G + (test == 1 || test == 2 ? 1u : 0u), status, report,
               own_status ? 1 : 0, kFirst, test == 3};
   constexpr size_t smem = OcLayout<Ar, Tin>::kBytes;
@@ -160,7 +163,7 @@ static cudaError_t launch_onchip_raw(int64_t n, const Tin* a, const Tin* b, cons
 template <class Ar, class Tin>
 static cudaError_t launch_onchip(tps_plan_s* P, int64_t n, const Tin* a, const Tin* b,
                                  const Tin* c, const Tin* d, Tin* x, cudaStream_t s,
-                                 bool& used, bool codes) {
+                                 bool& used, bool codes, bool nested) {
   used = false;
   if (P->desc.flags & TPS_NO_ONCHIP) return cudaSuccess;
   if (P->desc.flags & TPS_EXTERNAL_WORKSPACE) {  // the caller may have used it in between
@@ -169,7 +172,7 @@ static cudaError_t launch_onchip(tps_plan_s* P, int64_t n, const Tin* a, const T
   }
   return launch_onchip_raw<Ar, Tin>(n, a, b, c, d, x, P->ws + P->off_xch,
                                     reinterpret_cast<unsigned*>(P->ws + 32), P->d_status,
-                                    P->test_onchip, s, used, codes);
+                                    P->test_onchip, s, used, codes, nested);
 }
 
 unsigned* level0_dmax(tps_plan_s* P) {
@@ -371,7 +374,7 @@ static cudaError_t run_levels(tps_plan_s* P, const std::vector<LevelPlan>& level
                           P->d_status, nullptr);
   }
   bool used = false;
-  cudaError_t eo = launch_onchip<Ar, Tin>(P, n, a, b, c, d, x, s, used, false);
+  cudaError_t eo = launch_onchip<Ar, Tin>(P, n, a, b, c, d, x, s, used, false, true);
   if (eo != cudaSuccess || used) {
     if (used) {
       P->last_onchip = 2;
@@ -650,7 +653,7 @@ static tps_status run_solve_direct(tps_plan_s* P, int64_t n, const void* a, cons
       (void)tred;
       return launch_onchip<Ar, Tin>(P, n, (const Tin*)a, (const Tin*)b, (const Tin*)c,
                                     (const Tin*)d, (Tin*)x, s, onchip,
-                                    level0_dmax(P) != nullptr);
+                                    level0_dmax(P) != nullptr, false);
     });
     if (onchip) {
       P->last_onchip = 1;
@@ -779,7 +782,7 @@ cudaError_t onchip_solve(int dtype, int64_t n, const void* a, const void* b, con
     (void)tred;
     return launch_onchip_raw<Ar, Tin>(n, (const Tin*)a, (const Tin*)b, (const Tin*)c,
                                       (const Tin*)d, (Tin*)x, xch, bar, status, test, s, used,
-                                      dtype == TPS_F64_DF, true, report);
+                                      dtype == TPS_F64_DF, false, true, report);
   });
 }
 

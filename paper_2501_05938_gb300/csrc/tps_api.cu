@@ -162,7 +162,7 @@ static bool uses_relations(const tps_plan_s* P) {
 
 // Does the plan's own workspace hold them?  Not where they would take more than
 // half of the memory that is free: that may be meant for the caller's arrays,
-// and checkpoints need 1.2 bytes a row.  (A caller's workspace decides in
+// and checkpoints need about 3.5 bytes a row.  (A caller's workspace decides in
 // tps_set_workspace.)
 static bool holds_relations(const tps_plan_s* P) {
   const tps_plan_desc& d = P->desc;
