@@ -43,9 +43,9 @@
 // fp64 leaves out the chain below 2^-60 and always writes alpha, which Stage 3
 // reads only where it may be seen.
 // Both sweeps are bound by memory: 49 and 25 bytes a row, at n = 2^25 in
-// double-float 260 and 131 us, 94% of the copy rate (k_stage1 with
+// double-float 268 and 132 us, 91% and 95% of the copy rate (k_stage1 with
 // checkpoints 215 us, k_stage3 218 us).  Native fp64 Stage 1 is bound by the
-// fp64 pipe: 480 us (k_stage3's half of that work is gone: 490 -> 129 us).
+// fp64 pipe: 532 us (k_stage3's half of that work is gone: 490 -> 131 us).
 //
 // Without the workspace that takes (24 bytes a row), Stage 1 writes the
 // relation only at every chunk boundary, as a checkpoint, and k_stage3 walks
@@ -458,9 +458,8 @@ __device__ __forceinline__ unsigned long long abs_bits(double v) {
 #define TPS_STAGE1_STAGES 2
 #endif
 // kRel compiles its row body twice (with and without the chain), so it is
-// unrolled by pairs of 16-byte row groups only: at n = 2^25 in double-float the
-// whole chunk unrolled takes 384 us (instruction fetch), four groups 308, two
-// 260, one 268.
+// unrolled by pairs of 16-byte row groups only: back to back at n = 2^25 in
+// double-float four groups take 318 us (instruction fetch), two 289, one 292.
 #ifndef TPS_REL_UNROLL
 #define TPS_REL_UNROLL 2
 #endif
@@ -548,11 +547,11 @@ __global__ void __launch_bounds__(W * 32)
 
   // The first interior unknown's chain (P, Q, S) only adds terms scaled by
   // S, whose magnitude falls by |c / beta| < 1 every row of a strictly
-  // diagonally dominant block.  Where the policy allows (Ar::kSkipChain),
-  // once every lane's |S| is below 2^-60 the rest of the chain is below
-  // rounding and the rows skip it (kChain false); they check |c| <= |beta|
-  // instead, so S cannot grow back, and a block where that fails reports a
-  // pivot failure (not dominant).
+  // diagonally dominant block.  In native fp64 (Ar::kSkipChain), once every
+  // lane's |S| is below 2^-60 the rest of the chain is below rounding (of an f
+  // no more than 2^60 times smaller than the x it hangs on) and the rows skip it
+  // (kChain false); they check |c| <= |beta| instead, so S cannot grow back, and
+  // a block where that fails reports a pivot failure (not dominant).
   // The last unknown's coupling to f, al, is never left out.  With kRel the
   // other policies skip too, S and al together, but only once both are 0 in
   // every lane (underflown, or cut off at a system boundary), from where on
@@ -624,7 +623,7 @@ __global__ void __launch_bounds__(W * 32)
       if constexpr (decltype(kChain)::value) {
         const T aw = Ar::mul(Ar::norm(al), rbeta);
         if (active) rel_al[row * nb + lane] = aw;
-        // not from w and aw, which would live longer: 260 against 296 us at n = 2^25
+        // not from w and aw, which would live longer and cost a tenth of Stage 1
         const T tt = Ar::mul_nn(S, rbeta);
         P = Ar::sub_mul_nn(P, tt, g);
         Q = Ar::sub_mul_nn(Q, tt, al);
