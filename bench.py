@@ -551,7 +551,7 @@ def extra_workloads(binding, synth, world, rank, stream, a):
     out["batched"] = res
     del gb, offs
     out["mixed"] = mixed_workloads(binding, synth, world, rank, stream, a)
-    # mid-size single systems: the single-launch on-chip solve against the
+    # mid-size single systems: the on-chip solve against the
     # level-by-level route (inputs fit in L2, so these are L2-warm times)
     mid = {}
     for n in (65536, 800000):

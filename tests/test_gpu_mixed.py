@@ -130,7 +130,7 @@ def solve_mixed_plan(s, n, monkeypatch, unfused, offsets=None, **kw):
 
 NO_OC = binding.NO_ONCHIP
 FUSED_CASES = [
-    # (n, m, flags, ratio): several tiles and a ragged tail (the single-launch
+    # (n, m, flags, ratio): several tiles and a ragged tail (the
     # on-chip solve off, so that level 0 runs as separate sweeps); m = 51
     # takes the element-by-element loads (m not a multiple of the 16-byte
     # vector); the tail block of m + 1 rows; a size the on-chip solve does

@@ -1,8 +1,9 @@
-"""The single-launch on-chip solve (one cooperative launch: each CTA
-eliminates its rows in shared memory, one grid barrier, the CTA interface
-system by parallel cyclic reduction, recovery on chip) against the CPU
-oracle, at its capacity edges, as the Stage 2 of larger solves, inside a
-captured CUDA graph, and with its barrier wait made to run out."""
+"""The on-chip solve (each CTA eliminates its rows in shared memory, one grid
+barrier, the CTA interface system by parallel cyclic reduction, recovery on
+chip; two chained launches, or a cooperative one as Stage 2 of fp32 solves)
+against the CPU oracle, at its capacity edges, as the Stage 2 of larger
+solves, inside a captured CUDA graph, and with its barrier wait made to run
+out for all CTAs or for some."""
 import numpy as np
 import pytest
 

@@ -56,8 +56,8 @@ CASES = [(1, 32), (2, 32), (3, 2), (63, 8), (64, 32), (65, 32), (65, 2), (100, 3
 @pytest.mark.parametrize("dtype", ["f64", "f64_df"])
 @pytest.mark.parametrize("n,m", CASES)
 def test_fp64_paths_match_oracle(dtype, n, m, onchip):
-    """Both routes: the single-launch on-chip solve where the system fits,
-    and the multi-launch levels (TPS_NO_ONCHIP)."""
+    """Both routes: the on-chip solve where the system fits, and the
+    multi-launch levels (TPS_NO_ONCHIP)."""
     s = synth.system(1000 + n, n)
     plan = binding.Plan(n, dtype=dtype, m=m, flags=0 if onchip else binding.NO_ONCHIP)
     x, info = run(plan, s)
@@ -563,7 +563,7 @@ def test_graph_mode_batched():
 
 def test_distinct_plans_from_two_host_threads():
     # two host threads, each with its own plan and stream, solving at the
-    # same time (levels route: no cooperative launch), both against the oracle
+    # same time (levels route), both against the oracle
     import threading
 
     n = 300001
@@ -599,8 +599,9 @@ def test_distinct_plans_from_two_host_threads():
         assert oracle.rel_residual(s["a"], s["b"], s["c"], s["d"], x) <= F64_RES
 
 
-# Stage 3 from relations: Stage 1 drops the terms of the block's first unknown
-# once they have decayed, which rests on dominant rows.
+# Stage 3 from relations: Stage 1 leaves out the terms of the block's first unknown
+# once they are 0 (native fp64: the chain for that unknown below 2^-60; Stage 3
+# reads al only where it is 2^-130 or more).
 def _weak_rows(n, seed, m):
     """Rows that decouple from the block's first unknown at once (|a|, |c| of
     1e-3), then, 64 rows into every block, a stretch of barely dominant rows
@@ -624,9 +625,8 @@ def _weak_rows(n, seed, m):
 @pytest.mark.parametrize("kind", ["weak", "not_dominant"])
 def test_relations_with_rows_that_stop_decaying(dtype, kind):
     """Also with rows that are not dominant (a = 1.5 b in one row of some
-    blocks, after everything has decayed): the warp starts over and keeps
-    every term.  The condition number stays below 1e4 in both, times the unit
-    roundoff (2^-53, 2^-46, 2^-24)."""
+    blocks, after everything has decayed).  The condition number stays below
+    1e4 in both, times the unit roundoff (2^-53, 2^-46, 2^-24)."""
     n, m = 128 * 700 + 57, 128
     s = _weak_rows(n, 7, m)
     if kind == "not_dominant":

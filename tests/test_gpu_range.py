@@ -11,7 +11,7 @@ by powers of two -- whole rows (x unchanged, at any magnitude fp64 holds),
 the right-hand side alone (x scaled), single rows -- and require either a
 result that matches the fp64 Thomas oracle (relative forward error <= 1e-10,
 relative residual <= 1e-12) or the range status, never TPS_OK with a wrong
-x.  Every route is covered: the level-by-level solve, the single-launch
+x.  Every route is covered: the level-by-level solve, the
 on-chip solve, the one-warp solve, packed batches, the host pipeline, the
 windowed approximation and the allocation-free entry point.
 """

@@ -3,7 +3,7 @@ cudaMalloc (a framework allocator that owns all device memory, a fixed
 device-memory budget, latency-critical loops).  Its result must agree with the
 ordinary plan-based tps_solve and with the CPU oracle, and two calls in a row
 must both be right even though they share the library's fixed scratch array.
-Both of its routes are run: the single-launch on-chip solve it takes for
+Both of its routes are run: the on-chip solve it takes for
 every accepted size on a GB300, and the level-by-level route it keeps for
 devices where that launch does not fit (forced here by a test switch).  This
 file is named so that pytest collects it last."""
