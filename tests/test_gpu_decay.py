@@ -91,14 +91,15 @@ def impulse_error(x, ref, peak, dtype):
 
 @pytest.mark.parametrize("checkpoints", [False, True])
 @pytest.mark.parametrize("dtype", ["f64", "f64_df", "f32"])
-@pytest.mark.parametrize("at", [0, 1, 17, 100, 255])
-def test_impulse_is_resolved_far_below_its_peak(dtype, checkpoints, at, monkeypatch):
+@pytest.mark.parametrize("m,tail,at", [(256, 0, 0), (256, 0, 1), (256, 0, 17), (256, 0, 100),
+                                       (256, 0, 255), (250, 57, 3), (1000, 1, 0), (123, 40, 122)])
+def test_impulse_is_resolved_far_below_its_peak(dtype, checkpoints, m, tail, at, monkeypatch):
     """One nonzero entry in d, `at` rows into a block: x falls by 2 + sqrt(3) a
     row on either side, with no cancellation anywhere, so every component has
     a small relative error (a few roundings a row: 4 n ulp with n the rows it
     has come).  Native fp64 is held to it downwards of the impulse; upwards it
     leaves out what reaches a block's first unknown over more than 2^-60."""
-    m, n = 256, 256 * 40
+    n = m * 40 + tail
     s = toeplitz(n, 4.0)
     row, peak = 11 * m + at, 2.0 ** 60
     s["d"] = np.zeros(n)
